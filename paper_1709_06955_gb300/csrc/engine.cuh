@@ -118,8 +118,7 @@ struct Workspace {
     DevBuf t_key, t_node, t_parent, t_depth, t_query, t_weight, t_height, t_slot, t_gamma, t_G;
     DevBuf counts, offs, node_list, col_export, sched;  // level schedule: exported column nodes, uploaded plan
     DevBuf md_a, md_b, out_stage;                       // the two score buffers; host-output staging
-    DevBuf r_cnt, r_off, r_part, r_iwalk, r_ilen, r_iq, r_ik, r_fi[2], r_fn[2], r_keys[2], r_deg, r_pref, r_counts,
-        r_counts2, r_ctr;
+    DevBuf r_part, r_inst, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
     DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_vals, tk_qk;
     // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, next-level table, estimates
     DevBuf f_wslot, f_tsw, f_slot, f_misc, f_anc, f_deg, f_state, f_rsize, f_roff, f_dsize, f_doff, f_acc, f_tab, f_wp,
@@ -151,9 +150,8 @@ struct Workspace {
     void release() {
         DevBuf *bufs[] = {&qbuf, &walks, &lens, &ctr, &t_key, &t_node, &t_parent, &t_depth, &t_query, &t_weight,
                           &t_height, &t_slot, &t_gamma, &t_G, &counts, &offs, &node_list, &col_export,
-                          &sched, &md_a, &md_b, &out_stage, &r_cnt, &r_off,
-                          &r_part, &r_iwalk, &r_ilen, &r_iq, &r_ik, &r_fi[0], &r_fi[1], &r_fn[0], &r_fn[1],
-                          &r_keys[0], &r_keys[1], &r_deg, &r_pref, &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
+                          &sched, &md_a, &md_b, &out_stage, &r_part, &r_inst, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
+                          &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
                           &tk_cid, &tk_cval, &tk_ids, &tk_vals, &tk_qk, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_anc,
                           &f_deg, &f_state, &f_rsize, &f_roff, &f_dsize, &f_doff, &f_acc, &f_tab, &f_wp, &f_lp[0],
                           &f_lp[1], &f_lx[0], &f_lx[1], &f_lv[0], &f_lv[1], &f_sp, &f_sx, &f_sv, &f_cuts, &f_keys,

@@ -287,38 +287,39 @@ void launch_fr_finalize(int32_t n, int32_t B, const int32_t *qnode, const unsign
                         const float *inv_nr, const int32_t *ext2int, float shift, float *out, cudaStream_t s);
 
 // randomized PROBE (rand_probe.cu)
+struct alignas(16) RandInst {  // instance: walk row, prefix length i, query, Philox walk number k
+    int32_t walk, len, q;
+    uint32_t k;
+};
+struct RandList {                  // frontier entries with out-edges: (instance, node) and the entry's first work item
+    int2 *ent = nullptr;
+    long long *first = nullptr;
+    long long cap = 0;
+};
+// A level's counter: entries in the low bits, the sum of their out-degrees (work items) above.
+constexpr int kRandCountBits = 31;
+constexpr unsigned long long kRandCountMask = (1ull << kRandCountBits) - 1;
 struct RandLevel {
-    const int32_t *fr_inst = nullptr, *fr_node = nullptr;  // frontier H_j (entries with out-edges)
-    int64_t F = 0;
-    const long long *prefix = nullptr;  // [F+1] out-degree prefix sums
-    int64_t E = 0;                      // work items (frontier out-edges)
-    const unsigned long long *cur_keys = nullptr;  // set of (instance, node) in H_j
-    int64_t cur_cap = 0;
-    unsigned long long *next_keys = nullptr;       // set of (instance, node) in H_{j+1}
-    int64_t next_cap = 0;
-    int32_t *next_inst = nullptr, *next_node = nullptr;  // H_{j+1} entries with out-edges
-    unsigned long long *next_count = nullptr;
+    RandList cur, next;                                  // H_j and H_{j+1}
+    const unsigned long long *packed_in = nullptr;       // H_j's counter
+    unsigned long long *packed_out = nullptr, *check_out = nullptr;
     int32_t *counts = nullptr;          // [B][n] members of H_{i-1} per query (internal ids)
-    int32_t *overflow = nullptr;
     int32_t j = 0;
 };
 int64_t scan64_partials_needed(int64_t count);
 void launch_scan64(const long long *in, int64_t count, long long *partial, long long *out, cudaStream_t s);
-// Instances (walk w, prefix length i), i = 2..len, of the walks w0 .. w0+nw-1; with walk_slot and t_sw given, only
-// those whose prefix's tree slot is flagged in t_sw (the probes the switch of Sec. 4.4 handed to Alg. 3).
-void launch_inst_count(const int32_t *lens, int32_t w0, int32_t nw, long long *cnt, const int32_t *walk_slot,
-                       const uint8_t *t_sw, int32_t l_max, cudaStream_t s);
+// Instances (walk w, prefix length i), i = 2..len, of the walks w0 .. w0+nw-1 (none longer than max_len); with
+// walk_slot and t_sw given, only those whose prefix's tree slot is flagged in t_sw (the probes the switch of Sec. 4.4
+// handed to Alg. 3).  inst holds out.cap instances.
 void launch_inst_init(const QueryBatch &q, const DeviceGraph &g, const int32_t *lens, int32_t w0, int32_t nw,
-                      int32_t l_max, const int32_t *walks, const long long *inst_off, int32_t *inst_walk,
-                      int32_t *inst_len, int32_t *inst_q, uint32_t *inst_k, int32_t *fr_inst, int32_t *fr_node,
-                      unsigned long long *fr_count, unsigned long long *keys, int64_t cap, int32_t *overflow,
-                      const int32_t *walk_slot, const uint8_t *t_sw, cudaStream_t s);
+                      int32_t l_max, int32_t max_len, const int32_t *walks, RandInst *inst, RandList out,
+                      unsigned long long *packed, unsigned long long *check, const int32_t *walk_slot,
+                      const uint8_t *t_sw, cudaStream_t s);
 void launch_add_i32(int32_t *a, const int32_t *b, int64_t count, cudaStream_t s);  // a += b
-void launch_frontier_degree(const int32_t *fr_inst, const int32_t *fr_node, int64_t F, const int32_t *inst_len, int32_t j,
-                            const int64_t *out_off, long long *deg, cudaStream_t s);
-void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const int32_t *inst_walk,
-                       const int32_t *inst_len, const int32_t *inst_q, const uint32_t *inst_k, const uint32_t *qkey,
-                       uint32_t seed, uint32_t t_keep, const RandLevel &L, cudaStream_t s);
+// E: about the level's work items (sizes the grid)
+void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const RandInst *insts,
+                       const uint32_t *qkey, uint32_t seed, uint32_t t_keep, const RandLevel &L, int64_t E,
+                       cudaStream_t s);
 void launch_rand_finalize(int32_t n, int32_t B, const int32_t *qnode, const int32_t *counts, const float *inv_nr,
                           const int32_t *ext2int, float shift, float *out, cudaStream_t s);
 

@@ -856,103 +856,87 @@ static probesim_status batch_walks(probesim_graph *g, Workspace *ws, const Batch
 }
 
 // Randomized PROBE (Alg. 3) instances of the walks w0 .. w1-1, one per (walk, prefix length i >= 2) -- or, with
-// walk_slot and t_sw, only those whose prefix's tree slot is flagged -- run level by level over hash-set
-// frontiers.  Adds the member counts of the final levels into counts ([B][n], internal ids).  An allocation that
+// walk_slot and t_sw, only those whose prefix's tree slot is flagged -- run level by level over frontier lists.
+// Adds the member counts of the final levels into counts ([B][n], internal ids).  An allocation that
 // fails sets *too_big (here: the walk range is too large) and returns PROBESIM_E_NOMEM.
-static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryBatch &qb, int32_t B, int32_t w0,
-                                  int32_t w1, int32_t max_len, const int32_t *walk_slot, const uint8_t *t_sw,
+static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryBatch &qb, int32_t w0, int32_t w1,
+                                  int32_t max_len, int64_t walk_nodes, const int32_t *walk_slot, const uint8_t *t_sw,
                                   int32_t *counts, int64_t &launches, cudaStream_t st, bool *too_big) {
     *too_big = false;
     const int32_t W = w1 - w0;
     const DeviceGraph &dg = ws->dg;
     const int32_t L = g->cfg.l_max;
-    PS_ALLOC_RANGE(ws->r_cnt.ensure(sizeof(long long) * std::max(1, W)));
-    PS_ALLOC_RANGE(ws->r_off.ensure(sizeof(long long) * (W + 1)));
-    PS_ALLOC_RANGE(ws->r_part.ensure(sizeof(long long) * scan64_partials_needed(W)));
-    launch_inst_count(ws->lens.as<int32_t>(), w0, W, ws->r_cnt.as<long long>(), walk_slot, t_sw, L, st);
-    launch_scan64(ws->r_cnt.as<long long>(), W, ws->r_part.as<long long>(), ws->r_off.as<long long>(), st);
-    launches += 4;
-    long long *h_ll = reinterpret_cast<long long *>(ws->pin_s.as<char>() + 32768);
-    PS_CUDA(cudaMemcpyAsync(h_ll, ws->r_off.as<long long>() + W, sizeof(long long), cudaMemcpyDeviceToHost, st));
-    PS_CUDA(cudaStreamSynchronize(st));
-    const int64_t NI = h_ll[0];
-    if (NI >= ((int64_t)1 << 31)) return fail(PROBESIM_E_INVALID, "too many probe instances in one call");
-    if (NI == 0) return PROBESIM_OK;
-    PS_ALLOC_RANGE(ws->r_iwalk.ensure(sizeof(int32_t) * NI));
-    PS_ALLOC_RANGE(ws->r_ilen.ensure(sizeof(int32_t) * NI));
-    PS_ALLOC_RANGE(ws->r_iq.ensure(sizeof(int32_t) * NI));
-    PS_ALLOC_RANGE(ws->r_ik.ensure(sizeof(uint32_t) * NI));
-    PS_ALLOC_RANGE(ws->r_ctr.ensure(sizeof(unsigned long long) * 4));
-    unsigned long long *d_fc = ws->r_ctr.as<unsigned long long>();
-    int32_t *d_over = reinterpret_cast<int32_t *>(d_fc + 2);
-    int cur = 0;
-    int64_t cap = next_pow2(std::max<int64_t>(1024, 2 * NI));
-    PS_ALLOC_RANGE(ws->r_keys[cur].ensure(8 * (size_t)cap));
-    PS_ALLOC_RANGE(ws->r_fi[cur].ensure(4 * (size_t)NI));
-    PS_ALLOC_RANGE(ws->r_fn[cur].ensure(4 * (size_t)NI));
-    PS_CUDA(cudaMemsetAsync(ws->r_keys[cur].p, 0xFF, 8 * (size_t)cap, st));
-    PS_CUDA(cudaMemsetAsync(d_fc, 0, sizeof(unsigned long long) * 4, st));
-    launch_inst_init(qb, dg, ws->lens.as<int32_t>(), w0, W, L, ws->walks.as<int32_t>(), ws->r_off.as<long long>(),
-                     ws->r_iwalk.as<int32_t>(), ws->r_ilen.as<int32_t>(), ws->r_iq.as<int32_t>(), ws->r_ik.as<uint32_t>(),
-                     ws->r_fi[cur].as<int32_t>(), ws->r_fn[cur].as<int32_t>(), d_fc, ws->r_keys[cur].as<unsigned long long>(),
-                     cap, d_over, walk_slot, t_sw, st);
+    if (W <= 0 || max_len < 2) return PROBESIM_OK;
+    // instances: one per walk node after the first
+    const int64_t ni = std::min<int64_t>(walk_nodes, (int64_t)W * (max_len - 1));
+    if (ni > (int64_t)kRandCountMask) {
+        *too_big = W > 1;
+        return fail(PROBESIM_E_INVALID, "too many probe instances in one call");
+    }
+    if (ni == 0) return PROBESIM_OK;
+    auto list_of = [&](int k) {
+        RandList l;
+        l.ent = ws->r_ent[k].as<int2>();
+        l.first = ws->r_first[k].as<long long>();
+        l.cap = (long long)std::min(ws->r_ent[k].cap / sizeof(int2), ws->r_first[k].cap / sizeof(long long));
+        return l;
+    };
+    PS_ALLOC_RANGE(ws->r_inst.ensure(sizeof(RandInst) * ni));
+    PS_ALLOC_RANGE(ws->r_ent[0].ensure(sizeof(int2) * ni));
+    PS_ALLOC_RANGE(ws->r_first[0].ensure(sizeof(long long) * ni));
+    // counters of levels 0 .. 255 and their checks
+    PS_ALLOC_RANGE(ws->r_ctr.ensure(sizeof(unsigned long long) * 512));
+    unsigned long long *d_packed = ws->r_ctr.as<unsigned long long>(), *d_check = d_packed + 256;
+    PS_CUDA(cudaMemsetAsync(d_packed, 0, sizeof(unsigned long long) * 512, st));
+    RandList l0 = list_of(0);
+    l0.cap = std::min<long long>(l0.cap, ni);  // the instance array holds ni
+    launch_inst_init(qb, dg, ws->lens.as<int32_t>(), w0, W, L, max_len, ws->walks.as<int32_t>(),
+                     ws->r_inst.as<RandInst>(), l0, d_packed, d_check, walk_slot, t_sw, st);
     ++launches;
-    PS_CUDA(cudaMemcpyAsync(h_ll, d_fc, sizeof(unsigned long long) * 3, cudaMemcpyDeviceToHost, st));
+    unsigned long long *h_ctr = reinterpret_cast<unsigned long long *>(ws->pin_s.as<char>() + 32768);
+    PS_CUDA(cudaMemcpyAsync(h_ctr, d_packed, sizeof(unsigned long long) * 512, cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaStreamSynchronize(st));
-    if (reinterpret_cast<int32_t *>(h_ll + 2)[0]) return fail(PROBESIM_E_CUDA, "internal: frontier set overflow");
-    int64_t F = (int64_t)((unsigned long long *)h_ll)[0];
-    int64_t cur_cap = cap;
-    for (int32_t j = 0; j + 2 <= max_len && F > 0; ++j) {
-        // out-degree prefix sums of the frontier
-        PS_ALLOC_RANGE(ws->r_deg.ensure(sizeof(long long) * F));
-        PS_ALLOC_RANGE(ws->r_pref.ensure(sizeof(long long) * (F + 1)));
-        PS_ALLOC_RANGE(ws->r_part.ensure(sizeof(long long) * scan64_partials_needed(F)));
-        launch_frontier_degree(ws->r_fi[cur].as<int32_t>(), ws->r_fn[cur].as<int32_t>(), F, ws->r_ilen.as<int32_t>(), j,
-                               dg.out_off, ws->r_deg.as<long long>(), st);
-        launch_scan64(ws->r_deg.as<long long>(), F, ws->r_part.as<long long>(), ws->r_pref.as<long long>(), st);
-        launches += 4;
-        PS_CUDA(cudaMemcpyAsync(h_ll, ws->r_pref.as<long long>() + F, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        PS_CUDA(cudaStreamSynchronize(st));
-        const int64_t E = h_ll[0];
-        if (E <= 0) break;
-        const int nx = cur ^ 1;
-        const int64_t ncap = next_pow2(std::max<int64_t>(1024, 2 * E));
-        if ((size_t)(8 * ncap + 8 * E) > budget_of(g, ws) / 4 && w1 - w0 > 1) {  // a smaller walk range fits the budget
-            *too_big = true;
+    // Levels run several per synchronisation: a level whose members might not fit its list does nothing, so the
+    // host finds the first level that waited, grows the list and goes on from there.
+    int32_t group = 1;
+    for (int32_t j = 0; j + 2 <= max_len;) {
+        const unsigned long long packed = h_ctr[j];
+        const int64_t F = (int64_t)(packed & kRandCountMask), E = (int64_t)(packed >> kRandCountBits);
+        if (F == 0) break;
+        const int nx = (j + 1) & 1;
+        // an overflowed counter, or lists beyond the budget: a smaller walk range needs less
+        if (h_ctr[256 + j] != (unsigned long long)E || ((size_t)(16 * E) > budget_of(g, ws) / 4 && W > 1)) {
+            *too_big = W > 1;
             return fail(PROBESIM_E_NOMEM, "randomized PROBE level exceeds a quarter of the memory budget");
         }
-        PS_ALLOC_RANGE(ws->r_keys[nx].ensure(8 * (size_t)ncap));
-        PS_ALLOC_RANGE(ws->r_fi[nx].ensure(4 * (size_t)E));
-        PS_ALLOC_RANGE(ws->r_fn[nx].ensure(4 * (size_t)E));
-        PS_CUDA(cudaMemsetAsync(ws->r_keys[nx].p, 0xFF, 8 * (size_t)ncap, st));
-        PS_CUDA(cudaMemsetAsync(d_fc, 0, sizeof(unsigned long long), st));
-        RandLevel Lv;
-        Lv.fr_inst = ws->r_fi[cur].as<int32_t>();
-        Lv.fr_node = ws->r_fn[cur].as<int32_t>();
-        Lv.F = F;
-        Lv.prefix = ws->r_pref.as<long long>();
-        Lv.E = E;
-        Lv.cur_keys = ws->r_keys[cur].as<unsigned long long>();
-        Lv.cur_cap = cur_cap;
-        Lv.next_keys = ws->r_keys[nx].as<unsigned long long>();
-        Lv.next_cap = ncap;
-        Lv.next_inst = ws->r_fi[nx].as<int32_t>();
-        Lv.next_node = ws->r_fn[nx].as<int32_t>();
-        Lv.next_count = d_fc;
-        Lv.counts = counts;
-        Lv.overflow = d_over;
-        Lv.j = j;
-        launch_rand_level(dg, ws->walks.as<int32_t>(), L, ws->r_iwalk.as<int32_t>(), ws->r_ilen.as<int32_t>(),
-                          ws->r_iq.as<int32_t>(), ws->r_ik.as<uint32_t>(), qb.qid, g->cfg.seed, g->t_keep, Lv, st);
-        ++launches;
-        ws->stats.edge_gathers += E;
-        PS_CUDA(cudaMemcpyAsync(h_ll, d_fc, sizeof(unsigned long long) * 3, cudaMemcpyDeviceToHost, st));
+        PS_ALLOC_RANGE(ws->r_ent[nx].ensure(sizeof(int2) * E));
+        PS_ALLOC_RANGE(ws->r_first[nx].ensure(sizeof(long long) * E));
+        const int32_t end = std::min(max_len - 1, j + group);
+        for (int32_t t = j; t < end; ++t) {
+            RandLevel Lv;
+            Lv.cur = list_of(t & 1);
+            Lv.next = list_of((t + 1) & 1);
+            Lv.packed_in = d_packed + t;
+            Lv.packed_out = d_packed + t + 1;
+            Lv.check_out = d_check + t + 1;
+            Lv.counts = counts;
+            Lv.j = t;
+            launch_rand_level(dg, ws->walks.as<int32_t>(), L, ws->r_inst.as<RandInst>(), qb.qid, g->cfg.seed, g->t_keep,
+                              Lv, E, st);
+            ++launches;
+        }
+        PS_CUDA(cudaMemcpyAsync(h_ctr, d_packed, sizeof(unsigned long long) * 512, cudaMemcpyDeviceToHost, st));
         PS_CUDA(cudaStreamSynchronize(st));
-        if (reinterpret_cast<int32_t *>(h_ll + 2)[0]) return fail(PROBESIM_E_CUDA, "internal: frontier set overflow");
-        F = (int64_t)((unsigned long long *)h_ll)[0];
-        cur = nx;
-        cur_cap = ncap;
-        ws->stats.levels += 1;
+        while (j < end) {  // the levels that ran: those whose work fits the list they write
+            const int64_t Ej = (int64_t)(h_ctr[j] >> kRandCountBits);
+            if ((h_ctr[j] & kRandCountMask) == 0 || h_ctr[256 + j] != (unsigned long long)Ej ||
+                Ej > list_of((j + 1) & 1).cap)
+                break;
+            ws->stats.edge_gathers += Ej;
+            ws->stats.levels += 1;
+            ++j;
+        }
+        group = std::min(8, 2 * group);
     }
     return PROBESIM_OK;
 }
@@ -961,20 +945,19 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
 // walks are taken in halves, quarters, ..., each counted into a side buffer added once the range completes, so
 // the integer member counts come out the same whatever the split.
 static probesim_status rand_instances(probesim_graph *g, Workspace *ws, const QueryBatch &qb, int32_t B, int32_t W,
-                                      int32_t max_len, const int32_t *walk_slot, const uint8_t *t_sw, int64_t &launches,
-                                      cudaStream_t st, bool *too_big) {
+                                      int32_t max_len, int64_t walk_nodes, const int32_t *walk_slot,
+                                      const uint8_t *t_sw, int64_t &launches, cudaStream_t st, bool *too_big) {
     const size_t cn = (size_t)B * g->n;
     PS_ALLOC(ws->r_counts.ensure(sizeof(int32_t) * cn));
     PS_CUDA(cudaMemsetAsync(ws->r_counts.p, 0, sizeof(int32_t) * cn, st));
     bool oom = false;
-    probesim_status s = rand_range(g, ws, qb, B, 0, W, max_len, walk_slot, t_sw, ws->r_counts.as<int32_t>(), launches,
-                                   st, &oom);
+    probesim_status s = rand_range(g, ws, qb, 0, W, max_len, walk_nodes, walk_slot, t_sw, ws->r_counts.as<int32_t>(),
+                                   launches, st, &oom);
     if (s == PROBESIM_OK || !oom || W <= 1) {
         if (oom) *too_big = B > 1;
         return s;
     }
-    DevBuf *big[] = {&ws->r_keys[0], &ws->r_keys[1], &ws->r_fi[0], &ws->r_fi[1], &ws->r_fn[0], &ws->r_fn[1],
-                     &ws->r_deg, &ws->r_pref};
+    DevBuf *big[] = {&ws->r_ent[0], &ws->r_ent[1], &ws->r_first[0], &ws->r_first[1]};
     for (DevBuf *b : big) b->release();
     PS_CUDA(cudaMemsetAsync(ws->r_counts.p, 0, sizeof(int32_t) * cn, st));
     PS_ALLOC(ws->r_counts2.ensure(sizeof(int32_t) * cn));
@@ -982,7 +965,8 @@ static probesim_status rand_instances(probesim_graph *g, Workspace *ws, const Qu
     for (int32_t w0 = 0; w0 < W;) {
         const int32_t w1 = std::min(W, w0 + span);
         PS_CUDA(cudaMemsetAsync(ws->r_counts2.p, 0, sizeof(int32_t) * cn, st));
-        s = rand_range(g, ws, qb, B, w0, w1, max_len, walk_slot, t_sw, ws->r_counts2.as<int32_t>(), launches, st, &oom);
+        s = rand_range(g, ws, qb, w0, w1, max_len, walk_nodes, walk_slot, t_sw, ws->r_counts2.as<int32_t>(), launches, st,
+                       &oom);
         if (s == PROBESIM_OK) {
             launch_add_i32(ws->r_counts.as<int32_t>(), ws->r_counts2.as<int32_t>(), (int64_t)cn, st);
             ++launches;
@@ -1010,7 +994,7 @@ static probesim_status run_batch_rand(probesim_graph *g, Workspace *ws, const pr
     int64_t launches = 0, walk_nodes = 0;
     int32_t max_len = 0;
     PS_TRY(batch_walks(g, ws, P, qb, &walk_nodes, &max_len, launches, st));
-    PS_TRY(rand_instances(g, ws, qb, B, P.W, max_len, nullptr, nullptr, launches, st, too_big));
+    PS_TRY(rand_instances(g, ws, qb, B, P.W, max_len, walk_nodes, nullptr, nullptr, launches, st, too_big));
     launch_rand_finalize(g->n, B, qb.node, ws->r_counts.as<int32_t>(), qb.inv_nr, ws->dg.ext2int, g->cfg.shift, d_out,
                          st);
     ++launches;
@@ -1315,7 +1299,7 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
         for (DevBuf *b : {&ws->f_keys, &ws->f_lp[0], &ws->f_lp[1], &ws->f_lx[0], &ws->f_lx[1],
                           &ws->f_lv[0], &ws->f_lv[1], &ws->f_wp, &ws->f_sp, &ws->f_sx, &ws->f_sv})
             b->release();
-        PS_TRY(rand_instances(g, ws, qb, B, P.W, max_len, t.walk_slot, t_sw, launches, st, too_big));
+        PS_TRY(rand_instances(g, ws, qb, B, P.W, max_len, walk_nodes, t.walk_slot, t_sw, launches, st, too_big));
         counts = ws->r_counts.as<int32_t>();
     }
     launch_fr_finalize(n, B, qb.node, ws->f_acc.as<unsigned long long>(), counts, qb.inv_nr, dg.ext2int, g->cfg.shift,

@@ -6,10 +6,14 @@
 //
 // Candidates: Alg. 3 takes U = union of O(y), y in H_j, or V when that union is large (lines 4-7).  A node
 // outside the union has no in-neighbour in H_j and can never be selected, so both choices give the same
-// H_{j+1}; the kernels always evaluate the union, one work item per (frontier entry, out-edge), with the
-// frontier's out-degree prefix sums balancing the work.  Repeated candidates evaluate the same draw and the
-// next level's hash set keeps one copy.  The members of H_{i-1} are counted per query node; the estimate is
-// count / n_r (Alg. 1 with randomized PROBE), exact in integers.
+// H_{j+1}; the kernels always evaluate the union, one work item per (frontier entry y, out-edge y -> x).
+//
+// x joins H_{j+1} when its sampled in-neighbour v lies in H_j.  Then the item (v, x) is itself among the level's work
+// items, and it is the only item of x whose entry equals the sample.  So an item tests v == y and nothing else: every
+// member is found by exactly one item, no set of H_j is looked up and no set of H_{j+1} is needed to drop repeats
+// (hash sets for both took 60-80 % of this engine's time in random sectors and clears; see k_rand_level).
+// The members of H_{i-1} are counted per query node; the estimate is count / n_r (Alg. 1 with randomized PROBE),
+// exact in integers.
 #include "internal.cuh"
 
 namespace ps {
@@ -125,16 +129,29 @@ __device__ __forceinline__ int32_t walk_query(const int32_t *walk_base, int32_t 
     return lo;
 }
 
-// A slot in an append list for each lane that calls it: the lanes executing the call together (__activemask) take
-// consecutive slots with one atomic on the shared counter, instead of one atomic each on the same address.
-__device__ __forceinline__ unsigned long long warp_append(unsigned long long *counter) {
-    const unsigned mask = __activemask();
+// Reserves a place in a level's list, and `deg` work items, for every lane with deg > 0.  The counter packs the entry
+// count (low kRandCountBits) and the sum of the out-degrees, so one atomic per warp gives the entries their places and
+// their first work items in the same order: the list comes with its prefix sums, and no scan runs.  `check` sums the
+// degrees alone; the host compares the two to see an overflow of a packed field.  All 32 lanes call it together;
+// returns the lane's place and sets its first item.
+__device__ __forceinline__ long long rand_reserve(uint32_t deg, unsigned long long *packed, unsigned long long *check,
+                                                  long long *item) {
+    const unsigned mask = __ballot_sync(0xffffffffu, deg > 0);
+    if (!mask) return 0;
     const int lane = threadIdx.x & 31;
-    const int leader = __ffs(mask) - 1;
+    unsigned long long incl = deg;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
     unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(mask));
-    base = __shfl_sync(mask, base, leader);
-    return base + (unsigned long long)__popc(mask & ((1u << lane) - 1u));
+    if (lane == 31) {
+        base = atomicAdd(packed, (incl << kRandCountBits) + (unsigned long long)__popc(mask));
+        atomicAdd(check, incl);
+    }
+    base = __shfl_sync(0xffffffffu, base, 31);
+    *item = (long long)((base >> kRandCountBits) + incl - deg);
+    return (long long)(base & kRandCountMask) + __popc(mask & ((1u << lane) - 1u));
 }
 
 // instance (w, i) runs unless a filter is given and the tree slot of its prefix is not flagged
@@ -142,176 +159,136 @@ __device__ __forceinline__ bool inst_on(const int32_t *walk_slot, const uint8_t 
     return !walk_slot || t_sw[walk_slot[(int64_t)w * l_max + i - 1]];
 }
 
-// per walk w0 + i of a walk range: number of probes (len - 1, or the flagged ones)
-__global__ void k_inst_count(const int32_t *__restrict__ lens, int32_t w0, int32_t nw, long long *cnt,
-                             const int32_t *__restrict__ walk_slot, const uint8_t *__restrict__ t_sw, int32_t l_max) {
-    const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i0 >= nw) return;
-    const int32_t w = w0 + i0;
-    long long c = 0;
-    for (int32_t i = 2; i <= lens[w]; ++i) c += inst_on(walk_slot, t_sw, l_max, w, i);
-    cnt[i0] = c;
-}
-
 __global__ void k_add_i32(int32_t *__restrict__ a, const int32_t *__restrict__ b, int64_t count) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
         a[i] += b[i];
 }
 
-// instance (walk w, prefix length i) for i = 2..len; its level-0 frontier {u_i} goes into the table and list
-__device__ __forceinline__ unsigned long long rmix(unsigned long long z) {
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-// inserts key; returns 1 if it was absent, 0 if present, -1 if the table is full
-__device__ __forceinline__ int set_insert(unsigned long long *keys, int64_t cap, unsigned long long key) {
-    int64_t h = (int64_t)(rmix(key) & (unsigned long long)(cap - 1));
-    for (int64_t probe = 0; probe < cap; ++probe) {
-        unsigned long long cur = keys[h];
-        if (cur == key) return 0;
-        if (cur == kEmptyKey) {
-            cur = atomicCAS(&keys[h], kEmptyKey, key);
-            if (cur == kEmptyKey) return 1;
-            if (cur == key) return 0;
-        }
-        h = (h + 1) & (cap - 1);
+// Instances (walk w, prefix length i), i = 2..len, and their level-0 entries {u_i}: one thread per (walk, i), so a
+// long walk holds up no warp.  u_i is an in-neighbour of u_{i-1}, so its out-list is never empty, and the instance
+// takes the number of its entry.
+__global__ void __launch_bounds__(256) k_inst_init(QueryBatch q, const int64_t *__restrict__ out_off,
+                                                   const int32_t *__restrict__ lens, int32_t w0, int32_t nw,
+                                                   int32_t l_max, int32_t max_len, const int32_t *__restrict__ walks,
+                                                   RandInst *inst, RandList out, unsigned long long *packed,
+                                                   unsigned long long *check, const int32_t *__restrict__ walk_slot,
+                                                   const uint8_t *__restrict__ t_sw) {
+    const int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int32_t span = max_len - 1;
+    const int64_t wi = id / span;
+    const int32_t w = w0 + (int32_t)wi, i = 2 + (int32_t)(id - wi * span);
+    uint32_t deg = 0;
+    int32_t u = 0;
+    if (wi < nw && i <= lens[w] && inst_on(walk_slot, t_sw, l_max, w, i)) {
+        u = walks[(int64_t)w * l_max + i - 1];  // H_0 = {u_i}
+        deg = (uint32_t)(out_off[u + 1] - out_off[u]);
     }
-    return -1;
-}
-
-__device__ __forceinline__ bool set_contains(const unsigned long long *keys, int64_t cap, unsigned long long key) {
-    int64_t h = (int64_t)(rmix(key) & (unsigned long long)(cap - 1));
-    for (int64_t probe = 0; probe < cap; ++probe) {
-        const unsigned long long cur = keys[h];
-        if (cur == key) return true;
-        if (cur == kEmptyKey) return false;
-        h = (h + 1) & (cap - 1);
+    long long item;
+    const long long pos = rand_reserve(deg, packed, check, &item);
+    if (deg > 0 && pos < out.cap) {
+        const int32_t b = walk_query(q.walk_base, q.B, w);
+        inst[pos] = RandInst{w, i, b, (uint32_t)(q.walk_k0[b] + (w - q.walk_base[b]))};
+        out.ent[pos] = make_int2((int32_t)pos, u);
+        out.first[pos] = item;
     }
-    return false;
-}
-
-__global__ void k_inst_init(QueryBatch q, const int64_t *__restrict__ out_off, const int32_t *__restrict__ lens,
-                            int32_t w0, int32_t nw, int32_t l_max, const int32_t *__restrict__ walks,
-                            const long long *__restrict__ inst_off, int32_t *inst_walk, int32_t *inst_len,
-                            int32_t *inst_q, uint32_t *inst_k, int32_t *fr_inst, int32_t *fr_node,
-                            unsigned long long *fr_count, unsigned long long *keys, int64_t cap, int32_t *overflow,
-                            const int32_t *__restrict__ walk_slot, const uint8_t *__restrict__ t_sw) {
-    const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i0 >= nw) return;
-    const int32_t w = w0 + i0;
-    const int32_t len = lens[w];
-    int64_t id = inst_off[i0];
-    const int32_t b = walk_query(q.walk_base, q.B, w);
-    const uint32_t k = (uint32_t)(q.walk_k0[b] + (w - q.walk_base[b]));
-    for (int32_t i = 2; i <= len; ++i) {
-        if (!inst_on(walk_slot, t_sw, l_max, w, i)) continue;
-        inst_walk[id] = w;
-        inst_len[id] = i;
-        inst_q[id] = b;
-        inst_k[id] = k;
-        const int32_t u = walks[(int64_t)w * l_max + i - 1];  // H_0 = {u_i}
-        if (set_insert(keys, cap, ((unsigned long long)id << 32) | (uint32_t)u) < 0) atomicExch(overflow, 1);
-        if (out_off[u + 1] > out_off[u]) {
-            const unsigned long long pos = warp_append(fr_count);
-            fr_inst[pos] = (int32_t)id;
-            fr_node[pos] = u;
-        }
-        ++id;
-    }
-}
-
-// out-degree of every frontier entry whose instance still has a level to run
-__global__ void k_frontier_degree(const int32_t *__restrict__ fr_inst, const int32_t *__restrict__ fr_node, int64_t F,
-                                  const int32_t *__restrict__ inst_len, int32_t j, const int64_t *__restrict__ out_off,
-                                  long long *deg) {
-    const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (f >= F) return;
-    const int32_t y = fr_node[f];
-    deg[f] = (inst_len[fr_inst[f]] - 2 >= j) ? (long long)(out_off[y + 1] - out_off[y]) : 0;
 }
 
 constexpr int kLevelThreads = 256;
-constexpr int kLevelItems = 2048;  // work items per block pass
+constexpr int kLevelMaxItems = 512;  // work items a warp takes at a time, at most
 
-// One pass per block over kLevelItems consecutive work items; the block's slice of the prefix sums is
-// staged in shared memory so each item finds its frontier entry with a short search.
+// One level.  A warp takes a run of consecutive work items (32 to kLevelMaxItems, so that a short level still spreads
+// over the chip), 32 at a time.  It holds the first items of the next 32 entries in registers; every entry has at
+// least one item, so the entries of 32 items lie in that window, and a lane finds its own by five shuffles -- or by
+// none while the 32 items belong to one entry, which is the rule at level 0, where the entries are hubs.
+// What bounds it: the random sectors of a work item (the caller's id and the in-list bounds of x, one in-list entry)
+// and the ten Philox rounds.  A top-k call of four queries at
+// eps = 0.1 on R-MAT 2^20 went from 6.38 ms with the hash sets (20 levels: 4.5 ms of kernels, 0.55 ms of clears, two
+// synchronisations a level) to 3.00 ms; 64 mixed-eps queries with the switch on R-MAT 2^22 from 942 to 781 ms.
 __global__ void __launch_bounds__(kLevelThreads) k_rand_level(DeviceGraph g, const int32_t *__restrict__ walks,
-                                                              int32_t l_max, const int32_t *__restrict__ inst_walk,
-                                                              const int32_t *__restrict__ inst_len,
-                                                              const int32_t *__restrict__ inst_q,
-                                                              const uint32_t *__restrict__ inst_k,
+                                                              int32_t l_max, const RandInst *__restrict__ insts,
                                                               const uint32_t *__restrict__ qkey, uint32_t seed,
                                                               uint32_t t_keep, RandLevel L) {
-    __shared__ long long s_pref[kLevelItems + 1];
-    __shared__ int64_t s_f0, s_nf;
-    const int64_t nblk = (L.E + kLevelItems - 1) / kLevelItems;
-    for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const int64_t t0 = blk * kLevelItems, t1 = min(L.E, t0 + kLevelItems);
-        if (threadIdx.x == 0) {
-            int64_t lo = 0, hi = L.F;  // entry of item t0
-            while (hi - lo > 1) {
-                const int64_t mid = (lo + hi) >> 1;
-                if (L.prefix[mid] <= t0) lo = mid; else hi = mid;
-            }
-            int64_t lo2 = lo, hi2 = L.F;  // entry of item t1 - 1
-            while (hi2 - lo2 > 1) {
-                const int64_t mid = (lo2 + hi2) >> 1;
-                if (L.prefix[mid] <= t1 - 1) lo2 = mid; else hi2 = mid;
-            }
-            s_f0 = lo;
-            s_nf = lo2 - lo + 1;
+    const unsigned long long packed_in = *L.packed_in;
+    const long long F = (long long)(packed_in & kRandCountMask), E = (long long)(packed_in >> kRandCountBits);
+    if (F == 0 || E > L.next.cap) return;  // a level whose members might not fit waits for the host to grow the list
+    const int lane = threadIdx.x & 31;
+    const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    long long run = (E / nwarps + 31) / 32 * 32;
+    run = run < 32 ? 32 : (run > kLevelMaxItems ? kLevelMaxItems : run);
+    const long long *first = L.cur.first;
+    for (long long t0 = warp * run; t0 < E; t0 += nwarps * run) {
+        const long long t1 = min(E, t0 + run);
+        // the entry of item t0: the last f with first[f] <= t0, by a 32-way search
+        long long f = 0;
+        for (long long span = F; span > 1;) {
+            const long long step = (span + 31) / 32, at = f + lane * step;
+            const unsigned le = __ballot_sync(0xffffffffu, lane * step < span && first[at] <= t0);
+            const int k = 31 - __clz(le);  // lane 0 always holds
+            f += k * step;
+            span = min(step, span - k * step);
         }
-        __syncthreads();
-        const int64_t f0 = s_f0, nf = s_nf;
-        const bool staged = nf <= kLevelItems;
-        if (staged)
-            for (int64_t a = threadIdx.x; a <= nf; a += blockDim.x) s_pref[a] = L.prefix[f0 + a];
-        __syncthreads();
-        for (int64_t t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
-            int64_t f;
-            if (staged) {
-                int64_t lo = 0, hi = nf;
-                while (hi - lo > 1) {
-                    const int64_t mid = (lo + hi) >> 1;
-                    if (s_pref[mid] <= t) lo = mid; else hi = mid;
+        long long win = f + 1 + lane < F ? first[f + 1 + lane] : E;  // first items of the entries after f
+        long long beg_f = first[f];
+        int32_t c_inst = -1, c_y = 0, c_ex = 0, c_b = 0, c_i = 0;  // the lane's entry
+        uint32_t c_k = 0;
+        long long c_f = -1, c_col = 0;
+        for (long long t = t0; t < t1; t += 32) {
+            const long long it = t + lane;
+            int r = 0;  // entries of the window that start at or before the lane's item
+            if (__shfl_sync(0xffffffffu, win, 0) <= t + 31) {
+#pragma unroll
+                for (int s = 16; s; s >>= 1) {
+                    const long long v = __shfl_sync(0xffffffffu, win, r + s - 1);
+                    if (v <= it) r += s;
                 }
-                f = f0 + lo;
-            } else {
-                int64_t lo = f0, hi = L.F;
-                while (hi - lo > 1) {
-                    const int64_t mid = (lo + hi) >> 1;
-                    if (L.prefix[mid] <= t) lo = mid; else hi = mid;
-                }
-                f = lo;
             }
-            const int32_t inst = L.fr_inst[f];
-            const int32_t y = L.fr_node[f];
-            const int32_t x = g.out_col[g.out_off[y] + (t - L.prefix[f])];
-            const int32_t wid = inst_walk[inst];
-            const int32_t i = inst_len[inst];
-            if (x == walks[(int64_t)wid * l_max + (i - L.j - 2)]) continue;  // x = u_{i-j-1}
-            const int32_t b = inst_q[inst];
-            const U32x4 r = philox4x32_10(inst_k[inst], (1u << 24) | ((uint32_t)i << 8) | (uint32_t)L.j,
-                                          (uint32_t)g.int2ext[x], 0u, seed, qkey[b]);
-            if (r.y >= t_keep) continue;  // kept with probability sqrt(c)
-            const int64_t beg = g.in_off[x];
-            const uint32_t d = (uint32_t)(g.in_off[x + 1] - beg);
-            const int32_t v = g.in_col[beg + __umulhi(r.x, d)];  // the sampled in-edge (v, x)
-            if (!set_contains(L.cur_keys, L.cur_cap, ((unsigned long long)inst << 32) | (uint32_t)v)) continue;
-            const int ins = set_insert(L.next_keys, L.next_cap, ((unsigned long long)inst << 32) | (uint32_t)x);
-            if (ins < 0) { atomicExch(L.overflow, 1); continue; }
-            if (ins == 0) continue;
-            if (i - 2 == L.j) {
-                atomicAdd(L.counts + (int64_t)b * g.n + x, 1);  // member of H_{i-1}: the probe's result
-            } else if (g.out_off[x + 1] > g.out_off[x]) {    // only nodes with out-edges can expand
-                const unsigned long long pos = warp_append(L.next_count);
-                L.next_inst[pos] = inst;
-                L.next_node[pos] = x;
+            const long long start = __shfl_sync(0xffffffffu, win, r > 0 ? r - 1 : 0);
+            const bool live = it < t1;
+            if (live && f + r != c_f) {
+                c_f = f + r;
+                const int2 en = L.cur.ent[c_f];
+                c_inst = en.x;
+                c_y = en.y;
+                const RandInst in = insts[c_inst];
+                c_i = in.len;
+                c_b = in.q;
+                c_k = in.k;
+                c_ex = walks[(int64_t)in.walk * l_max + (c_i - L.j - 2)];  // u_{i-j-1}
+                c_col = g.out_off[c_y] - (r > 0 ? start : beg_f);
+            }
+            bool member = false;
+            int32_t x = 0;
+            if (live) {
+                x = g.out_col[c_col + it];
+                if (x != c_ex) {
+                    const U32x4 d = philox4x32_10(c_k, (1u << 24) | ((uint32_t)c_i << 8) | (uint32_t)L.j,
+                                                  (uint32_t)g.int2ext[x], 0u, seed, qkey[c_b]);
+                    if (d.y < t_keep) {  // kept with probability sqrt(c)
+                        const int64_t beg = g.in_off[x];
+                        const uint32_t deg = (uint32_t)(g.in_off[x + 1] - beg);
+                        member = g.in_col[beg + __umulhi(d.x, deg)] == c_y;  // the sampled in-edge (v, x) has v = y
+                    }
+                }
+            }
+            const bool last = c_i - 2 == L.j;
+            if (member && last) atomicAdd(L.counts + (int64_t)c_b * g.n + x, 1);  // in H_{i-1}: the probe's result
+            uint32_t od = 0;
+            if (member && !last) od = (uint32_t)(g.out_off[x + 1] - g.out_off[x]);  // without out-edges it ends here
+            long long item;
+            const long long pos = rand_reserve(od, L.packed_out, L.check_out, &item);
+            if (od > 0 && pos < L.next.cap) {
+                L.next.ent[pos] = make_int2(c_inst, x);
+                L.next.first[pos] = item;
+            }
+            // the window moves past the entries that end by item t + 32
+            const int adv = __popc(__ballot_sync(0xffffffffu, win <= t + 32));
+            if (adv > 0 && t + 32 < t1) {
+                beg_f = __shfl_sync(0xffffffffu, win, adv - 1);
+                f += adv;
+                win = f + 1 + lane < F ? first[f + 1 + lane] : E;
             }
         }
-        __syncthreads();
     }
 }
 
@@ -326,39 +303,23 @@ __global__ void k_rand_finalize(int32_t n, int32_t B, const int32_t *__restrict_
     out[(int64_t)b * n + v] = s;
 }
 
-void launch_inst_count(const int32_t *lens, int32_t w0, int32_t nw, long long *cnt, const int32_t *walk_slot,
-                       const uint8_t *t_sw, int32_t l_max, cudaStream_t s) {
-    if (nw > 0) k_inst_count<<<(nw + 255) / 256, 256, 0, s>>>(lens, w0, nw, cnt, walk_slot, t_sw, l_max);
-}
 void launch_inst_init(const QueryBatch &q, const DeviceGraph &g, const int32_t *lens, int32_t w0, int32_t nw,
-                      int32_t l_max, const int32_t *walks, const long long *inst_off, int32_t *inst_walk,
-                      int32_t *inst_len, int32_t *inst_q, uint32_t *inst_k, int32_t *fr_inst, int32_t *fr_node,
-                      unsigned long long *fr_count, unsigned long long *keys, int64_t cap, int32_t *overflow,
-                      const int32_t *walk_slot, const uint8_t *t_sw, cudaStream_t s) {
-    if (nw > 0)
-        k_inst_init<<<(nw + 255) / 256, 256, 0, s>>>(q, g.out_off, lens, w0, nw, l_max, walks, inst_off, inst_walk,
-                                                     inst_len, inst_q, inst_k, fr_inst, fr_node, fr_count, keys, cap,
-                                                     overflow, walk_slot, t_sw);
+                      int32_t l_max, int32_t max_len, const int32_t *walks, RandInst *inst, RandList out,
+                      unsigned long long *packed, unsigned long long *check, const int32_t *walk_slot,
+                      const uint8_t *t_sw, cudaStream_t s) {
+    if (nw <= 0 || max_len < 2) return;
+    const int64_t threads = (int64_t)nw * (max_len - 1);
+    k_inst_init<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(q, g.out_off, lens, w0, nw, l_max, max_len, walks, inst,
+                                                                  out, packed, check, walk_slot, t_sw);
 }
 void launch_add_i32(int32_t *a, const int32_t *b, int64_t count, cudaStream_t s) {
     if (count > 0) k_add_i32<<<grid_for(count, 256, 8), 256, 0, s>>>(a, b, count);
 }
-void launch_frontier_degree(const int32_t *fr_inst, const int32_t *fr_node, int64_t F, const int32_t *inst_len, int32_t j,
-                            const int64_t *out_off, long long *deg, cudaStream_t s) {
-    if (F > 0)
-        k_frontier_degree<<<(unsigned)((F + 255) / 256), 256, 0, s>>>(fr_inst, fr_node, F, inst_len, j, out_off, deg);
-}
-void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const int32_t *inst_walk,
-                       const int32_t *inst_len, const int32_t *inst_q, const uint32_t *inst_k, const uint32_t *qkey,
-                       uint32_t seed, uint32_t t_keep, const RandLevel &L, cudaStream_t s) {
-    if (L.E <= 0) return;
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t blocks = (L.E + kLevelItems - 1) / kLevelItems;
-    if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-    k_rand_level<<<(unsigned)blocks, kLevelThreads, 0, s>>>(g, walks, l_max, inst_walk, inst_len, inst_q, inst_k, qkey,
-                                                            seed, t_keep, L);
+void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const RandInst *insts,
+                       const uint32_t *qkey, uint32_t seed, uint32_t t_keep, const RandLevel &L, int64_t E,
+                       cudaStream_t s) {
+    const int blocks = grid_for(E, kLevelThreads, 8);
+    k_rand_level<<<blocks, kLevelThreads, 0, s>>>(g, walks, l_max, insts, qkey, seed, t_keep, L);
 }
 void launch_rand_finalize(int32_t n, int32_t B, const int32_t *qnode, const int32_t *counts, const float *inv_nr,
                           const int32_t *ext2int, float shift, float *out, cudaStream_t s) {
