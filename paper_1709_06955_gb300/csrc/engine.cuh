@@ -102,12 +102,12 @@ struct PinnedBuf {
 // version beside it and publishes it, so queries never wait for updates nor updates for queries, and a version's
 // device memory is freed when its last reader lets go.
 struct StoreVersion {
-    DevBuf in_off, in_col, out_off, out_col, w, piece_v, piece_beg, piece_len, split_v;
+    DevBuf in_off, in_col, out_off, out_col, w, rec, piece_v, piece_beg, piece_len, split_v;
     std::shared_ptr<StoreVersion> base;  // set when this version reuses base's arrays (an update that changed nothing)
     ps::DeviceGraph dg;
     uint64_t epoch = 0;
     ~StoreVersion() {
-        for (DevBuf *b : {&in_off, &in_col, &out_off, &out_col, &w, &piece_v, &piece_beg, &piece_len, &split_v})
+        for (DevBuf *b : {&in_off, &in_col, &out_off, &out_col, &w, &rec, &piece_v, &piece_beg, &piece_len, &split_v})
             b->release();
     }
 };
@@ -118,7 +118,7 @@ struct Workspace {
     DevBuf t_key, t_node, t_parent, t_depth, t_query, t_weight, t_height, t_slot, t_gamma, t_G;
     DevBuf counts, offs, node_list, col_export, sched;  // level schedule: exported column nodes, uploaded plan
     DevBuf md_a, md_b, out_stage;                       // the two score buffers; host-output staging
-    DevBuf r_part, r_inst, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
+    DevBuf r_part, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
     DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_vals, tk_qk;
     // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, next-level table, estimates
     DevBuf f_wslot, f_tsw, f_slot, f_misc, f_anc, f_deg, f_state, f_rsize, f_roff, f_dsize, f_doff, f_acc, f_tab, f_wp,
@@ -150,7 +150,7 @@ struct Workspace {
     void release() {
         DevBuf *bufs[] = {&qbuf, &walks, &lens, &ctr, &t_key, &t_node, &t_parent, &t_depth, &t_query, &t_weight,
                           &t_height, &t_slot, &t_gamma, &t_G, &counts, &offs, &node_list, &col_export,
-                          &sched, &md_a, &md_b, &out_stage, &r_part, &r_inst, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
+                          &sched, &md_a, &md_b, &out_stage, &r_part, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
                           &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
                           &tk_cid, &tk_cval, &tk_ids, &tk_vals, &tk_qk, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_anc,
                           &f_deg, &f_state, &f_rsize, &f_roff, &f_dsize, &f_doff, &f_acc, &f_tab, &f_wp, &f_lp[0],

@@ -128,12 +128,21 @@ __global__ void __launch_bounds__(256) k_upd_rows(DeviceGraph g, UpdateBatch b, 
     }
 }
 
-// 4. w and the pull pieces
-__global__ void k_upd_w(int32_t n, const long long *__restrict__ new_off, float sqrt_c, float *w, long long *npieces) {
+// 4. w, the node records and the pull pieces (offsets fit 32 bits: m < 2^31)
+__global__ void k_upd_w(int32_t n, const long long *__restrict__ new_off, const int32_t *__restrict__ in_col,
+                        float sqrt_c, const int32_t *__restrict__ int2ext, int32_t rec_shift, float *w, int4 *rec,
+                        long long *npieces) {
     const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (v >= n) return;
-    const long long d = new_off[v + 1] - new_off[v];
+    const long long beg = new_off[v], d = new_off[v + 1] - beg;
     w[v] = d > 0 ? sqrt_c / (float)d : 0.f;
+    uint32_t splits = 0;
+    if (d > 0) {
+        int32_t x[kRecSplits];
+        for (int k = 0; k < kRecSplits; ++k) x[k] = in_col[beg + (k + 1) * d / (kRecSplits + 1)];
+        for (int k = 0; k < kRecSplits; ++k) splits |= (uint32_t)(int2ext[x[k]] >> rec_shift) << (8 * k);
+    }
+    rec[v] = make_int4((int32_t)beg, (int32_t)d, int2ext[v], (int32_t)splits);
     npieces[v] = d <= kPiece ? 1 : (d + kPiece - 1) / kPiece;
 }
 
@@ -221,8 +230,9 @@ void launch_upd_rows(const DeviceGraph &g, const UpdateBatchArgs &a, bool in_lis
     else k_upd_rows<false><<<blocks, 256, 0, s>>>(g, b, new_off, new_col);
 }
 
-void launch_upd_w(int32_t n, const long long *new_off, float sqrt_c, float *w, long long *npieces, cudaStream_t s) {
-    k_upd_w<<<blocks_for(n, 256), 256, 0, s>>>(n, new_off, sqrt_c, w, npieces);
+void launch_upd_w(int32_t n, const long long *new_off, const int32_t *in_col, float sqrt_c, const int32_t *int2ext,
+                  int32_t rec_shift, float *w, int4 *rec, long long *npieces, cudaStream_t s) {
+    k_upd_w<<<blocks_for(n, 256), 256, 0, s>>>(n, new_off, in_col, sqrt_c, int2ext, rec_shift, w, rec, npieces);
 }
 
 void launch_upd_pieces(int32_t n, const long long *new_off, unsigned long long *hist, unsigned long long *cursor,

@@ -65,9 +65,24 @@ struct DeviceGraph {
     int32_t *split_v = nullptr;
     int32_t n_active = 0;          // every node with out-edges has an internal id below n_active (all of them
                                    // come first at creation; update batches may leave gaps)
+    int4 *rec = nullptr;           // node records (see make_rec)
+    int32_t rec_shift = 0;         // splits of the records: caller's id >> rec_shift, in 8 bits
     int32_t *ext2int = nullptr;    // caller's node id -> internal id (descending out-degree order)
     int32_t *int2ext = nullptr;    // internal id -> caller's node id
 };
+
+// Node record, 16 bytes, so a sampled in-edge of x costs one gather for everything about x: in-list start, in-list
+// length d, the caller's id, and four splits of the in-list.  I(x) is sorted by the caller's id; split k = 1..4 holds
+// the id at position floor(k d / 5), shifted to 8 bits.  A draw r picks entry floor(r d / 2^32) of I(x); with b =
+// floor(5 r / 2^32) that entry lies between splits b and b + 1, so a node whose shifted id lies outside them is not the
+// one drawn, and four of five in-list reads are answered from the record (rand_probe.cu; 64 switch
+// queries on R-MAT 2^22: 742 -> 693 ms; no change at 2^20, whose lists stay in the L2).
+constexpr int kRecSplits = 4;
+__device__ __forceinline__ bool rec_may_be(int32_t splits, uint32_t r, uint32_t id8) {
+    const unsigned long long z = 0xFF0000000000ull | ((unsigned long long)(uint32_t)splits << 8);  // ends: 0 and 255
+    const uint32_t b = __umulhi(r, kRecSplits + 1) * 8;
+    return id8 >= ((uint32_t)(z >> b) & 0xFFu) && id8 <= ((uint32_t)(z >> (b + 8)) & 0xFFu);
+}
 
 // The queries of one launch.
 struct QueryBatch {
@@ -287,12 +302,19 @@ void launch_fr_finalize(int32_t n, int32_t B, const int32_t *qnode, const unsign
                         const float *inv_nr, const int32_t *ext2int, float shift, float *out, cudaStream_t s);
 
 // randomized PROBE (rand_probe.cu)
-struct alignas(16) RandInst {  // instance: walk row, prefix length i, query, Philox walk number k
-    int32_t walk, len, q;
-    uint32_t k;
+// A frontier entry of an instance (walk, prefix length), with everything its work items need, so a level reads its
+// entries in order and gathers nothing per entry.
+struct alignas(32) RandEntry {
+    int32_t y;             // the frontier node
+    int32_t ex;            // the node this level excludes, u_{i-j-1}
+    uint32_t k;            // Philox walk number
+    int32_t len;           // prefix length i
+    int32_t walk, q;       // walk row, query
+    uint32_t out_beg;      // start of O(y)
+    uint32_t id8;          // y's caller id, shifted to 8 bits (DeviceGraph::rec)
 };
-struct RandList {                  // frontier entries with out-edges: (instance, node) and the entry's first work item
-    int2 *ent = nullptr;
+struct RandList {          // frontier entries with out-edges, and each entry's first work item
+    RandEntry *ent = nullptr;
     long long *first = nullptr;
     long long cap = 0;
 };
@@ -301,6 +323,7 @@ constexpr int kRandCountBits = 31;
 constexpr unsigned long long kRandCountMask = (1ull << kRandCountBits) - 1;
 struct RandLevel {
     RandList cur, next;                                  // H_j and H_{j+1}
+    long long max_items = 0;                             // a level with more waits for the host to grow `next`
     const unsigned long long *packed_in = nullptr;       // H_j's counter
     unsigned long long *packed_out = nullptr, *check_out = nullptr;
     int32_t *counts = nullptr;          // [B][n] members of H_{i-1} per query (internal ids)
@@ -310,15 +333,13 @@ int64_t scan64_partials_needed(int64_t count);
 void launch_scan64(const long long *in, int64_t count, long long *partial, long long *out, cudaStream_t s);
 // Instances (walk w, prefix length i), i = 2..len, of the walks w0 .. w0+nw-1 (none longer than max_len); with
 // walk_slot and t_sw given, only those whose prefix's tree slot is flagged in t_sw (the probes the switch of Sec. 4.4
-// handed to Alg. 3).  inst holds out.cap instances.
+// handed to Alg. 3).
 void launch_inst_init(const QueryBatch &q, const DeviceGraph &g, const int32_t *lens, int32_t w0, int32_t nw,
-                      int32_t l_max, int32_t max_len, const int32_t *walks, RandInst *inst, RandList out,
-                      unsigned long long *packed, unsigned long long *check, const int32_t *walk_slot,
-                      const uint8_t *t_sw, cudaStream_t s);
+                      int32_t l_max, int32_t max_len, const int32_t *walks, RandList out, unsigned long long *packed,
+                      unsigned long long *check, const int32_t *walk_slot, const uint8_t *t_sw, cudaStream_t s);
 void launch_add_i32(int32_t *a, const int32_t *b, int64_t count, cudaStream_t s);  // a += b
 // E: about the level's work items (sizes the grid)
-void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const RandInst *insts,
-                       const uint32_t *qkey, uint32_t seed, uint32_t t_keep, const RandLevel &L, int64_t E,
+void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const uint32_t *qkey, uint32_t seed, uint32_t t_keep, const RandLevel &L, int64_t E,
                        cudaStream_t s);
 void launch_rand_finalize(int32_t n, int32_t B, const int32_t *qnode, const int32_t *counts, const float *inv_nr,
                           const int32_t *ext2int, float shift, float *out, cudaStream_t s);
@@ -342,7 +363,14 @@ void launch_upd_mark(const DeviceGraph &g, const UpdateBatchArgs &a, long long *
 void launch_upd_degrees(int32_t n, const int64_t *off, const long long *delta, long long *deg, cudaStream_t s);
 void launch_upd_rows(const DeviceGraph &g, const UpdateBatchArgs &a, bool in_lists, const long long *new_off,
                      int32_t *new_col, cudaStream_t s);
-void launch_upd_w(int32_t n, const long long *new_off, float sqrt_c, float *w, long long *npieces, cudaStream_t s);
+// w, the node records (DeviceGraph::rec) and the number of pull pieces of every row
+void launch_upd_w(int32_t n, const long long *new_off, const int32_t *in_col, float sqrt_c, const int32_t *int2ext,
+                  int32_t rec_shift, float *w, int4 *rec, long long *npieces, cudaStream_t s);
+inline int32_t rec_shift_for(int32_t n) {  // ids below n, shifted, fit 8 bits
+    int32_t b = 0;
+    while (((int64_t)(n - 1) >> b) > 255) ++b;
+    return b;
+}
 void launch_upd_pieces(int32_t n, const long long *new_off, unsigned long long *hist, unsigned long long *cursor,
                        int32_t *split_v, unsigned long long *n_split, int32_t *pv, int64_t *pb, int32_t *pl,
                        cudaStream_t s);

@@ -178,12 +178,14 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     // w and the pull pieces (in-lists cut into at most kPiece edges, longest first)
     const int64_t cap_pieces = (int64_t)n + mu / kPiece + 1;
     PS_CUDA(sv->w.ensure(sizeof(float) * n));
+    PS_CUDA(sv->rec.ensure(sizeof(int4) * n));
     PS_CUDA(sv->piece_v.ensure(sizeof(int32_t) * cap_pieces));
     PS_CUDA(sv->piece_beg.ensure(sizeof(int64_t) * cap_pieces));
     PS_CUDA(sv->piece_len.ensure(sizeof(int32_t) * cap_pieces));
     PS_CUDA(sv->split_v.ensure(sizeof(int32_t) * (size_t)n));
     PS_CUDA(t.hist.ensure(sizeof(unsigned long long) * (2 * (kPiece + 1) + 2)));
-    launch_upd_w(n, sv->in_off.as<long long>(), (float)std::sqrt(g->cfg.c), sv->w.as<float>(),
+    launch_upd_w(n, sv->in_off.as<long long>(), sv->in_col.as<int32_t>(), (float)std::sqrt(g->cfg.c),
+                 g->int2ext.as<int32_t>(), rec_shift_for(n), sv->w.as<float>(), sv->rec.as<int4>(),
                  t.indeg_i.as<long long>(), st);
     unsigned long long *hist = t.hist.as<unsigned long long>(), *cursor = hist + (kPiece + 1),
                        *nsplit = cursor + (kPiece + 1);
@@ -214,6 +216,8 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     d.out_off = sv->out_off.as<int64_t>();
     d.out_col = sv->out_col.as<int32_t>();
     d.w = sv->w.as<float>();
+    d.rec = sv->rec.as<int4>();
+    d.rec_shift = rec_shift_for(n);
     d.n_pieces = npieces;
     d.piece_v = sv->piece_v.as<int32_t>();
     d.piece_beg = sv->piece_beg.as<int64_t>();
@@ -858,11 +862,13 @@ static probesim_status batch_walks(probesim_graph *g, Workspace *ws, const Batch
 // Randomized PROBE (Alg. 3) instances of the walks w0 .. w1-1, one per (walk, prefix length i >= 2) -- or, with
 // walk_slot and t_sw, only those whose prefix's tree slot is flagged -- run level by level over frontier lists.
 // Adds the member counts of the final levels into counts ([B][n], internal ids).  An allocation that
-// fails sets *too_big (here: the walk range is too large) and returns PROBESIM_E_NOMEM.
+// fails sets *too_big (here: the walk range is too large) and returns PROBESIM_E_NOMEM.  A level's list holds
+// list_share entries per work item; *too_short is set, with PROBESIM_E_NOMEM, when a level had more members.
 static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryBatch &qb, int32_t w0, int32_t w1,
                                   int32_t max_len, int64_t walk_nodes, const int32_t *walk_slot, const uint8_t *t_sw,
-                                  int32_t *counts, int64_t &launches, cudaStream_t st, bool *too_big) {
-    *too_big = false;
+                                  int32_t *counts, double list_share, int64_t &launches, cudaStream_t st, bool *too_big,
+                                  bool *too_short) {
+    *too_big = *too_short = false;
     const int32_t W = w1 - w0;
     const DeviceGraph &dg = ws->dg;
     const int32_t L = g->cfg.l_max;
@@ -876,22 +882,23 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
     if (ni == 0) return PROBESIM_OK;
     auto list_of = [&](int k) {
         RandList l;
-        l.ent = ws->r_ent[k].as<int2>();
+        l.ent = ws->r_ent[k].as<RandEntry>();
         l.first = ws->r_first[k].as<long long>();
-        l.cap = (long long)std::min(ws->r_ent[k].cap / sizeof(int2), ws->r_first[k].cap / sizeof(long long));
+        l.cap = (long long)std::min(ws->r_ent[k].cap / sizeof(RandEntry), ws->r_first[k].cap / sizeof(long long));
         return l;
     };
-    PS_ALLOC_RANGE(ws->r_inst.ensure(sizeof(RandInst) * ni));
-    PS_ALLOC_RANGE(ws->r_ent[0].ensure(sizeof(int2) * ni));
+    // the work items whose members are taken to fit a list: `need` below gives at least that many entries
+    auto items_of = [&](const RandList &l) -> long long {
+        return l.cap <= 1024 ? l.cap : (long long)((double)(l.cap - 1) / list_share);
+    };
+    PS_ALLOC_RANGE(ws->r_ent[0].ensure(sizeof(RandEntry) * ni));
     PS_ALLOC_RANGE(ws->r_first[0].ensure(sizeof(long long) * ni));
     // counters of levels 0 .. 255 and their checks
     PS_ALLOC_RANGE(ws->r_ctr.ensure(sizeof(unsigned long long) * 512));
     unsigned long long *d_packed = ws->r_ctr.as<unsigned long long>(), *d_check = d_packed + 256;
     PS_CUDA(cudaMemsetAsync(d_packed, 0, sizeof(unsigned long long) * 512, st));
-    RandList l0 = list_of(0);
-    l0.cap = std::min<long long>(l0.cap, ni);  // the instance array holds ni
-    launch_inst_init(qb, dg, ws->lens.as<int32_t>(), w0, W, L, max_len, ws->walks.as<int32_t>(),
-                     ws->r_inst.as<RandInst>(), l0, d_packed, d_check, walk_slot, t_sw, st);
+    launch_inst_init(qb, dg, ws->lens.as<int32_t>(), w0, W, L, max_len, ws->walks.as<int32_t>(), list_of(0), d_packed,
+                     d_check, walk_slot, t_sw, st);
     ++launches;
     unsigned long long *h_ctr = reinterpret_cast<unsigned long long *>(ws->pin_s.as<char>() + 32768);
     PS_CUDA(cudaMemcpyAsync(h_ctr, d_packed, sizeof(unsigned long long) * 512, cudaMemcpyDeviceToHost, st));
@@ -904,25 +911,31 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
         const int64_t F = (int64_t)(packed & kRandCountMask), E = (int64_t)(packed >> kRandCountBits);
         if (F == 0) break;
         const int nx = (j + 1) & 1;
+        if (F > list_of(j & 1).cap) {
+            *too_short = true;
+            return fail(PROBESIM_E_NOMEM, "internal: a randomized PROBE level outgrew its list");
+        }
+        const int64_t need = std::max<int64_t>(1024, (int64_t)(list_share * (double)E) + 1);
         // an overflowed counter, or lists beyond the budget: a smaller walk range needs less
-        if (h_ctr[256 + j] != (unsigned long long)E || ((size_t)(16 * E) > budget_of(g, ws) / 4 && W > 1)) {
+        if (h_ctr[256 + j] != (unsigned long long)E ||
+            ((sizeof(RandEntry) + sizeof(long long)) * (size_t)need > budget_of(g, ws) / 4 && W > 1)) {
             *too_big = W > 1;
             return fail(PROBESIM_E_NOMEM, "randomized PROBE level exceeds a quarter of the memory budget");
         }
-        PS_ALLOC_RANGE(ws->r_ent[nx].ensure(sizeof(int2) * E));
-        PS_ALLOC_RANGE(ws->r_first[nx].ensure(sizeof(long long) * E));
+        PS_ALLOC_RANGE(ws->r_ent[nx].ensure(sizeof(RandEntry) * need));
+        PS_ALLOC_RANGE(ws->r_first[nx].ensure(sizeof(long long) * need));
         const int32_t end = std::min(max_len - 1, j + group);
         for (int32_t t = j; t < end; ++t) {
             RandLevel Lv;
             Lv.cur = list_of(t & 1);
             Lv.next = list_of((t + 1) & 1);
+            Lv.max_items = items_of(Lv.next);
             Lv.packed_in = d_packed + t;
             Lv.packed_out = d_packed + t + 1;
             Lv.check_out = d_check + t + 1;
             Lv.counts = counts;
             Lv.j = t;
-            launch_rand_level(dg, ws->walks.as<int32_t>(), L, ws->r_inst.as<RandInst>(), qb.qid, g->cfg.seed, g->t_keep,
-                              Lv, E, st);
+            launch_rand_level(dg, ws->walks.as<int32_t>(), L, qb.qid, g->cfg.seed, g->t_keep, Lv, E, st);
             ++launches;
         }
         PS_CUDA(cudaMemcpyAsync(h_ctr, d_packed, sizeof(unsigned long long) * 512, cudaMemcpyDeviceToHost, st));
@@ -930,7 +943,7 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
         while (j < end) {  // the levels that ran: those whose work fits the list they write
             const int64_t Ej = (int64_t)(h_ctr[j] >> kRandCountBits);
             if ((h_ctr[j] & kRandCountMask) == 0 || h_ctr[256 + j] != (unsigned long long)Ej ||
-                Ej > list_of((j + 1) & 1).cap)
+                (int64_t)(h_ctr[j] & kRandCountMask) > list_of(j & 1).cap || Ej > items_of(list_of((j + 1) & 1)))
                 break;
             ws->stats.edge_gathers += Ej;
             ws->stats.levels += 1;
@@ -949,11 +962,25 @@ static probesim_status rand_instances(probesim_graph *g, Workspace *ws, const Qu
                                       const uint8_t *t_sw, int64_t &launches, cudaStream_t st, bool *too_big) {
     const size_t cn = (size_t)B * g->n;
     PS_ALLOC(ws->r_counts.ensure(sizeof(int32_t) * cn));
-    PS_CUDA(cudaMemsetAsync(ws->r_counts.p, 0, sizeof(int32_t) * cn, st));
+    // Members per work item: the item (y, x) is a member's with probability sqrt(c) / |I(x)|, and the sum of 1 / |I(x)|
+    // over all edges is the number of nodes with in-edges, so sqrt(c) n / m is the graph's mean.  Lists hold four times
+    // that (at least one entry for eight items); a range with more members runs again with lists for every item.
+    const double share = std::min(1.0, std::max(0.125, 4.0 * std::sqrt(g->cfg.c) * (double)g->n /
+                                                           (double)std::max<int64_t>(1, ws->dg.m)));
     bool oom = false;
-    probesim_status s = rand_range(g, ws, qb, 0, W, max_len, walk_nodes, walk_slot, t_sw, ws->r_counts.as<int32_t>(),
-                                   launches, st, &oom);
+    auto range = [&](int32_t w0, int32_t w1, DevBuf &counts) -> probesim_status {
+        bool too_short = false;
+        PS_CUDA(cudaMemsetAsync(counts.p, 0, sizeof(int32_t) * cn, st));
+        probesim_status s = rand_range(g, ws, qb, w0, w1, max_len, walk_nodes, walk_slot, t_sw, counts.as<int32_t>(),
+                                       share, launches, st, &oom, &too_short);
+        if (!too_short) return s;
+        PS_CUDA(cudaMemsetAsync(counts.p, 0, sizeof(int32_t) * cn, st));
+        return rand_range(g, ws, qb, w0, w1, max_len, walk_nodes, walk_slot, t_sw, counts.as<int32_t>(), 1.0, launches,
+                          st, &oom, &too_short);
+    };
+    probesim_status s = range(0, W, ws->r_counts);
     if (s == PROBESIM_OK || !oom || W <= 1) {
+        if (s == PROBESIM_OK) g_last_error.clear();  // a range that ran again is not an error
         if (oom) *too_big = B > 1;
         return s;
     }
@@ -964,9 +991,7 @@ static probesim_status rand_instances(probesim_graph *g, Workspace *ws, const Qu
     int32_t span = (W + 1) / 2;
     for (int32_t w0 = 0; w0 < W;) {
         const int32_t w1 = std::min(W, w0 + span);
-        PS_CUDA(cudaMemsetAsync(ws->r_counts2.p, 0, sizeof(int32_t) * cn, st));
-        s = rand_range(g, ws, qb, w0, w1, max_len, walk_nodes, walk_slot, t_sw, ws->r_counts2.as<int32_t>(), launches, st,
-                       &oom);
+        s = range(w0, w1, ws->r_counts2);
         if (s == PROBESIM_OK) {
             launch_add_i32(ws->r_counts.as<int32_t>(), ws->r_counts2.as<int32_t>(), (int64_t)cn, st);
             ++launches;
@@ -1462,7 +1487,7 @@ probesim_status probesim_graph_create(int32_t n, const int32_t *src, const int32
         if (cudaDeviceGetDefaultMemPool(&pool, g->device) == cudaSuccess) {
             const std::shared_ptr<StoreVersion> v = g->current();
             uint64_t keep = 0;
-            for (DevBuf *b : {&v->in_off, &v->in_col, &v->out_off, &v->out_col, &v->w, &v->piece_v, &v->piece_beg,
+            for (DevBuf *b : {&v->in_off, &v->in_col, &v->out_off, &v->out_col, &v->w, &v->rec, &v->piece_v, &v->piece_beg,
                               &v->piece_len, &v->split_v})
                 keep += b->cap;
             keep *= 3;
@@ -1654,7 +1679,9 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     PS_CUDA(n_pl.alloc_pooled(sizeof(int32_t) * cap_pieces, st));
     PS_CUDA(n_split.alloc_pooled(sizeof(int32_t) * (size_t)n, st));
     PS_CUDA(nv->w.alloc_pooled(sizeof(float) * (size_t)n, st));
-    launch_upd_w(n, n_in_off.as<long long>(), (float)std::sqrt(g->cfg.c), nv->w.as<float>(), deg, st);
+    PS_CUDA(nv->rec.alloc_pooled(sizeof(int4) * (size_t)n, st));
+    launch_upd_w(n, n_in_off.as<long long>(), n_in_col.as<int32_t>(), (float)std::sqrt(g->cfg.c),
+                 g->int2ext.as<int32_t>(), dg.rec_shift, nv->w.as<float>(), nv->rec.as<int4>(), deg, st);
     unsigned long long *hist = g->u_hist.as<unsigned long long>(), *cursor = hist + (kPiece + 1),
                        *nsplit = cursor + (kPiece + 1);
     launch_upd_pieces(n, n_in_off.as<long long>(), hist, cursor, n_split.as<int32_t>(), nsplit, n_pv.as<int32_t>(),
@@ -1681,6 +1708,7 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     ng.in_col = nv->in_col.as<int32_t>();
     ng.out_col = nv->out_col.as<int32_t>();
     ng.w = nv->w.as<float>();
+    ng.rec = nv->rec.as<int4>();
     ng.n_pieces = npieces;
     ng.piece_v = nv->piece_v.as<int32_t>();
     ng.piece_beg = nv->piece_beg.as<int64_t>();
