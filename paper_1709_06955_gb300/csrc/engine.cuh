@@ -120,13 +120,12 @@ struct Workspace {
     DevBuf md_a, md_b, out_stage;                       // the two score buffers; host-output staging
     DevBuf r_part, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
     DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_vals, tk_qk;
-    // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, next-level table, estimates
-    DevBuf f_wslot, f_tsw, f_slot, f_misc, f_anc, f_deg, f_state, f_rsize, f_roff, f_dsize, f_doff, f_acc, f_tab, f_wp,
-        f_lp[2], f_lx[2], f_lv[2], f_sp, f_sx, f_sv, f_cuts, f_keys, f_bcnt, f_bpre;
+    // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, deferral stack, tasks, global tables,
+    // estimates
+    DevBuf f_wslot, f_tsw, f_slot, f_misc, f_pr32, f_pr64, f_acc, f_tab, f_list[2], f_stack, f_tasks, f_keys;
     DevBuf pm_in, pm_meets;  // pairwise Monte Carlo: pairs and keys, meet counts
     DevBuf pull_err;         // set by the TMA pull when a stage's wait gives up
-    bool f_table_clean = false;  // f_keys (the level table) holds only empty slots (every pass's compaction empties
-                                 // its slots)
+    bool f_table_clean = false;  // f_keys (the global tables) holds only empty slots (every sweep empties its slots)
     PinnedBuf pin_q;  // query arrays of one batch
     PinnedBuf pin_s;  // counters and schedule offsets (fixed size, allocated at creation)
     int profiling = 0;
@@ -152,10 +151,8 @@ struct Workspace {
                           &t_height, &t_slot, &t_gamma, &t_G, &counts, &offs, &node_list, &col_export,
                           &sched, &md_a, &md_b, &out_stage, &r_part, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
                           &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
-                          &tk_cid, &tk_cval, &tk_ids, &tk_vals, &tk_qk, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_anc,
-                          &f_deg, &f_state, &f_rsize, &f_roff, &f_dsize, &f_doff, &f_acc, &f_tab, &f_wp, &f_lp[0],
-                          &f_lp[1], &f_lx[0], &f_lx[1], &f_lv[0], &f_lv[1], &f_sp, &f_sx, &f_sv, &f_cuts, &f_keys,
-                          &f_bcnt, &f_bpre, &pm_in, &pm_meets, &pull_err};
+                          &tk_cid, &tk_cval, &tk_ids, &tk_vals, &tk_qk, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_pr32, &f_pr64, &f_acc,
+                          &f_tab, &f_list[0], &f_list[1], &f_stack, &f_tasks, &f_keys, &pm_in, &pm_meets, &pull_err};
         for (DevBuf *b : bufs) b->release();
         f_table_clean = false;
         pin_q.release();

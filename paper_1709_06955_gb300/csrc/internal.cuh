@@ -246,58 +246,75 @@ cudaError_t topk_preload();
 constexpr int kFixShift = 44;  // scores and estimates accumulate as int64 multiples of 2^-44
 constexpr int32_t kProbeSwitched = 1, kProbeDense = 2;
 constexpr int64_t kFrontierMaxWalks = (int64_t)1 << 18;  // per query: keeps every fixed-point sum below 2^62
+// A probe's frontier: entries and the sum of their out-degrees (its work items), packed for one atomic per append.
+constexpr int kFrCountBits = 31;
+constexpr unsigned long long kFrCountMask = (1ull << kFrCountBits) - 1;
+// classes of a probe at a level (see frontier.cu), then the sweep of the global tables, then the range's totals
+enum {
+    kFrNone = 0, kFrLast, kFrSingle, kFrWarp, kFrBlock, kFrMid, kFrWide, kFrSlab, kFrGlobal, kFrSweep, kFrClasses,
+    kFrTotD = kFrClasses, kFrTotSlots, kFrTotGlobal, kFrTotItems, kFrTotEntries, kFrTotals
+};
+// bounds on the next frontier for the tables in shared memory: three quarters of their slots (half of the warp table's)
+constexpr unsigned kWarpD = 128, kBlockD = 1536, kMidD = 6144, kPartD = 12288;
+constexpr unsigned kSlabN = 24576, kSlabParts = 6;  // nodes of a slab part
+constexpr unsigned kMaxParts = 6;
+constexpr unsigned kFrChunk = 2048;                              // work items per warp task
 struct FrontierProbes {
     int32_t P = 0;
     int32_t *slot = nullptr;              // tree slot of the probed prefix
-    int32_t *anc = nullptr;               // tree slot of the node the current level excludes
-    unsigned long long *deg = nullptr;    // out-degree sum of the current level's kept entries
+    int32_t *anc = nullptr, *lev = nullptr;  // tree slot of the node that level lev excludes
+    int32_t *ex = nullptr;                // the node the planned level excludes
     int32_t *state = nullptr;             // kProbeSwitched | kProbeDense
-    long long *rsize = nullptr;           // region slots in the next level's table
-    long long *roff = nullptr;            // [P+1] region offsets (exclusive prefix sums of rsize over a probe range)
-    long long *dsize = nullptr;           // bound on the next level's entries: min(out-degree sum, n)
-    long long *doff = nullptr;            // [P+1] its exclusive prefix sums over a probe range
+    int32_t *cls = nullptr;               // class of the planned level
+    uint32_t *nt = nullptr;               // its tasks
+    unsigned long long *packed = nullptr, *packed_nx = nullptr;  // count and items of this level's and the next frontier
+    long long *beg = nullptr, *beg_nx = nullptr;                 // their segments' starts
+    long long *rsize = nullptr, *roff = nullptr;         // global class: region of the table
 };
-struct FrontierList {  // entries of the frontiers, grouped by probe in probe order
-    int32_t *p = nullptr;
-    int32_t *x = nullptr;
-    float *val = nullptr;                 // score (the fixed-point sum of its level, rounded to FP32)
+struct alignas(16) FrontierEntry {        // out-list start, first work item in the probe's segment, out-degree, score
+    uint32_t out_beg, first, deg;         // (the fixed-point sum of its level, rounded to FP32)
+    float val;
 };
-// One slot of a level's table: node + 1 (0 = empty) and the node's score sum (2^-44 units), in 16 bytes of one
+struct FrontierTask {
+    int32_t p;
+    uint32_t part;
+};
+struct FrontierBases {
+    long long at[kFrClasses] = {0};       // first task of each class
+};
+// One slot of a global table: node + 1 (0 = empty) and the node's score sum (2^-44 units), in 16 bytes of one
 // sector, so the sum's atomic lands in the sector that the key's lookup has just brought into the L2.
 struct alignas(16) FrontierSlot {
     int32_t key;
     int32_t pad;
     unsigned long long val;
 };
-struct FrontierExpand {
-    const long long *wp = nullptr;        // [nF+1] prefix sums of the entries' work (out-degrees)
-    int64_t f_lo = 0, f_hi = 0;           // entries of this pass
-    long long e_lo = 0, e_hi = 0;         // work items of this pass
-    int32_t j = 0;                        // level
-    FrontierSlot *tab = nullptr;          // next level's table (all slots empty between passes)
-    long long rbase = 0;                  // table offset of this pass's first region
+struct FrontierLevel {
+    const FrontierTask *tasks = nullptr;
+    const FrontierEntry *src = nullptr;   // this level's segments
+    FrontierEntry *dst = nullptr;         // the next level's
+    FrontierSlot *tab = nullptr;          // the global tables (all slots empty between levels)
     unsigned long long *acc = nullptr;    // [B][n] estimates (2^-44 units, internal ids)
-    int32_t n = 0;
+    const float *pw = nullptr;            // sqrt(c)^k
+    float eps_p = 0.f;
+    int32_t j = 0;
 };
 void launch_fr_list(TrieTable t, int32_t *slot, int32_t *count, cudaStream_t s);
-void launch_fr_init(TrieTable t, FrontierProbes P, FrontierList F, cudaStream_t s);
-void launch_fr_prune(FrontierList F, int64_t nF, TrieTable t, FrontierProbes P, const int64_t *out_off, const float *pw,
-                     float eps_p, int32_t j, long long *work, cudaStream_t s);
-void launch_fr_regions(TrieTable t, FrontierProbes P, int32_t p0, int32_t p1, int32_t j, int32_t n, const long long *thr,
-                       uint8_t *t_sw, cudaStream_t s);
+void launch_fr_init(TrieTable t, FrontierProbes P, const int64_t *out_off, const float *pw, float eps_p,
+                    FrontierEntry *list, cudaStream_t s);
+// switches the probes of [p0, p1) whose next frontier is certain to exceed the limit (no Rule 2; segments in src)
+void launch_fr_check(const DeviceGraph &g, TrieTable t, FrontierProbes P, int32_t p0, int32_t p1, int32_t j,
+                     const FrontierEntry *src, const long long *thr, uint8_t *t_sw, cudaStream_t s);
+void launch_fr_plan(TrieTable t, FrontierProbes P, int32_t p0, int32_t p1, int32_t j, int32_t n,
+                    const long long *thr, uint8_t *t_sw, unsigned long long *totals, cudaStream_t s);
+void launch_fr_tasks(FrontierProbes P, int32_t p0, int32_t p1, int32_t n, const FrontierBases &base,
+                     unsigned long long *cursor, FrontierTask *tasks, cudaStream_t s);
+cudaError_t launch_fr_level(const DeviceGraph &g, TrieTable t, FrontierProbes P, const FrontierLevel &a,
+                            const FrontierBases &base, const unsigned long long *ntasks, cudaStream_t s,
+                            int64_t *launches);
+void launch_fr_defer(FrontierProbes P, int32_t p0, int32_t p1, const FrontierEntry *src, FrontierEntry *stack,
+                     unsigned long long *top, cudaStream_t s);
 void launch_fr_count_switched(FrontierProbes P, unsigned long long *count, cudaStream_t s);
-void launch_fr_work(FrontierList F, int64_t nF, FrontierProbes P, long long *work, cudaStream_t s);
-void launch_fr_expand(const DeviceGraph &g, TrieTable t, FrontierProbes P, FrontierList F, const FrontierExpand &a,
-                      cudaStream_t s);
-int64_t fr_compact_blocks(long long T);
-void launch_fr_count(const FrontierSlot *tab, long long T, long long *bcount, cudaStream_t s);
-void launch_fr_write(FrontierSlot *tab, long long T, const long long *roff, int32_t p0,
-                     int32_t p1, long long rbase, const long long *bpre, FrontierList out, long long out_base,
-                     long long out_cap, cudaStream_t s);
-void launch_fr_advance(TrieTable t, FrontierProbes P, int32_t p0, int32_t p1, cudaStream_t s);
-// per cut probe c: first entry, work prefix there, region offset and entry-bound offset
-void launch_fr_bounds(const int32_t *fp, int64_t nF, const long long *wp, const long long *roff, const long long *doff,
-                      const int32_t *probes, int32_t count, long long *out, cudaStream_t s);
 void launch_fr_finalize(int32_t n, int32_t B, const int32_t *qnode, const unsigned long long *acc, const int32_t *counts,
                         const float *inv_nr, const int32_t *ext2int, float shift, float *out, cudaStream_t s);
 

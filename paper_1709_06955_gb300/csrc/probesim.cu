@@ -986,6 +986,8 @@ static probesim_status rand_instances(probesim_graph *g, Workspace *ws, const Qu
     }
     DevBuf *big[] = {&ws->r_ent[0], &ws->r_ent[1], &ws->r_first[0], &ws->r_first[1]};
     for (DevBuf *b : big) b->release();
+    // the frontier engine's lists and tables (in switch mode) are done with by now: their memory goes too
+    for (DevBuf *b : {&ws->f_list[0], &ws->f_list[1], &ws->f_stack, &ws->f_tasks, &ws->f_keys}) b->release();
     PS_CUDA(cudaMemsetAsync(ws->r_counts.p, 0, sizeof(int32_t) * cn, st));
     PS_ALLOC(ws->r_counts2.ensure(sizeof(int32_t) * cn));
     int32_t span = (W + 1) / 2;
@@ -1083,10 +1085,10 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
     launch_trie_insert(dg, qb, P.W, L, ws->walks.as<int32_t>(), ws->lens.as<int32_t>(), t, d_ctr, st);
     // the probes: tree nodes of depth >= 2
     PS_ALLOC(ws->f_slot.ensure(sizeof(int32_t) * std::max<int64_t>(1, walk_nodes)));
-    PS_ALLOC(ws->f_misc.ensure(64));
+    PS_ALLOC(ws->f_misc.ensure(512));
     int32_t *d_np = ws->f_misc.as<int32_t>();
     unsigned long long *d_fctr = reinterpret_cast<unsigned long long *>(ws->f_misc.as<char>() + 8);
-    PS_CUDA(cudaMemsetAsync(d_np, 0, 64, st));
+    PS_CUDA(cudaMemsetAsync(d_np, 0, 512, st));
     launch_fr_list(t, ws->f_slot.as<int32_t>(), d_np, st);
     launches += 2;
     LaunchCounters *h_ctr = ws->pin_s.as<LaunchCounters>();
@@ -1098,24 +1100,26 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
     const int32_t NP = reinterpret_cast<int32_t *>(h_ll)[0];
     ws->stats.probes += NP;
     ws->stats.tree_nodes += NP;
-    // per-probe state, the two frontier lists, the estimate sums
+    // per-probe state, the estimate sums
     FrontierProbes PR;
     PR.P = NP;
-    PS_ALLOC(ws->f_anc.ensure(sizeof(int32_t) * std::max(1, NP)));
-    PS_ALLOC(ws->f_deg.ensure(sizeof(unsigned long long) * std::max(1, NP)));
-    PS_ALLOC(ws->f_state.ensure(sizeof(int32_t) * std::max(1, NP)));
-    PS_ALLOC(ws->f_rsize.ensure(sizeof(long long) * (NP + 1)));
-    PS_ALLOC(ws->f_roff.ensure(sizeof(long long) * (NP + 1)));
-    PS_ALLOC(ws->f_dsize.ensure(sizeof(long long) * (NP + 1)));
-    PS_ALLOC(ws->f_doff.ensure(sizeof(long long) * (NP + 1)));
+    const size_t np1 = (size_t)std::max(1, NP);
+    PS_ALLOC(ws->f_pr32.ensure(sizeof(int32_t) * 6 * np1));
+    PS_ALLOC(ws->f_pr64.ensure(sizeof(long long) * 6 * np1));
     PR.slot = ws->f_slot.as<int32_t>();
-    PR.anc = ws->f_anc.as<int32_t>();
-    PR.deg = ws->f_deg.as<unsigned long long>();
-    PR.state = ws->f_state.as<int32_t>();
-    PR.rsize = ws->f_rsize.as<long long>();
-    PR.roff = ws->f_roff.as<long long>();
-    PR.dsize = ws->f_dsize.as<long long>();
-    PR.doff = ws->f_doff.as<long long>();
+    int32_t *i32 = ws->f_pr32.as<int32_t>();
+    PR.anc = i32, PR.lev = i32 + np1, PR.ex = i32 + 2 * np1, PR.state = i32 + 3 * np1, PR.cls = i32 + 4 * np1;
+    PR.nt = reinterpret_cast<uint32_t *>(i32 + 5 * np1);
+    long long *i64 = ws->f_pr64.as<long long>();
+    PR.rsize = i64 + 4 * np1, PR.roff = i64 + 5 * np1;
+    auto of_parity = [&](int cur) {  // this level's segments and counters and the next level's change places
+        FrontierProbes p = PR;
+        p.packed = reinterpret_cast<unsigned long long *>(i64 + cur * np1);
+        p.packed_nx = reinterpret_cast<unsigned long long *>(i64 + (cur ^ 1) * np1);
+        p.beg = i64 + (2 + cur) * np1;
+        p.beg_nx = i64 + (2 + (cur ^ 1)) * np1;
+        return p;
+    };
     const size_t accn = (size_t)B * n;
     PS_ALLOC(ws->f_acc.ensure(sizeof(unsigned long long) * accn));
     PS_CUDA(cudaMemsetAsync(ws->f_acc.p, 0, sizeof(unsigned long long) * accn, st));
@@ -1139,178 +1143,113 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
     }
     const float *d_pw = ws->f_tab.as<float>();
     const long long *d_thr = sw_mode ? reinterpret_cast<const long long *>(ws->f_tab.as<char>() + 256 * sizeof(float)) : nullptr;
-    // The deterministic rounds work on tasks: a probe range [p0, p1) at level j with its frontier entries.  A
-    // level whose next frontier might not fit the list budget processes the passes that fit and defers the other
-    // probes, with their level-j entries, to a stack; they resume once the processed range has run out.  Every
-    // probe's last-level pushes land in the estimate exactly once, whatever the split.
-    const long long pass_slots =
+    // The deterministic rounds work on probe ranges [p0, p1) at a level j.  A range whose next frontiers or global tables
+    // might not fit their part of the budget keeps as many of its first probes as the bounds allow and defers the
+    // others, with their level-j segments, to a stack; they resume once the kept probes have run out.  Every probe's
+    // last-level pushes land in the estimate exactly once, whatever the split.
+    const long long slot_cap =
         std::max<long long>((long long)n, (long long)(budget_of(g, ws) / 4 / sizeof(FrontierSlot)));
-    const long long list_cap = std::max<long long>((long long)n, (long long)(budget_of(g, ws) / 8 / 12));
-    auto list_of = [&](int k) {
-        FrontierList F;
-        F.p = ws->f_lp[k].as<int32_t>();
-        F.x = ws->f_lx[k].as<int32_t>();
-        F.val = ws->f_lv[k].as<float>();
-        return F;
-    };
-    auto grow_list = [&](int k, long long need, long long keep, cudaStream_t s) -> cudaError_t {
-        cudaError_t e = ws->f_lp[k].grow(sizeof(int32_t) * need, sizeof(int32_t) * keep, s);
-        if (e == cudaSuccess) e = ws->f_lx[k].grow(sizeof(int32_t) * need, sizeof(int32_t) * keep, s);
-        if (e == cudaSuccess) e = ws->f_lv[k].grow(sizeof(float) * need, sizeof(float) * keep, s);
-        return e;
-    };
-    struct Task {
+    const long long list_cap =
+        std::max<long long>((long long)n, (long long)(budget_of(g, ws) / 8 / sizeof(FrontierEntry)));
+    struct Range {
         int32_t p0, p1, j;
-        long long at, count;  // entries on the deferral stack
+        int cur;
+        bool on_stack;  // segments in the stack buffer, else in list cur
+        long long at;   // on_stack: the stack's height below them
     };
-    std::vector<Task> stack;
+    std::vector<Range> stack;
+    Range R{0, NP, 0, 0, false, 0};
     long long stack_top = 0;
-    int cur = 0;
-    int64_t nF = NP;
-    int32_t p0 = 0, p1 = NP, j = 0;
-    PS_ALLOC(grow_list(cur, std::max<int64_t>(1, nF), 0, st));
-    launch_fr_init(t, PR, list_of(cur), st);
+    unsigned long long *d_tot = d_fctr + 1, *d_cursor = d_tot + kFrTotals, *d_top = d_cursor + kFrTotals;
+    unsigned long long *h_tot = reinterpret_cast<unsigned long long *>(h_ll);
+    PS_ALLOC(ws->f_list[0].ensure(sizeof(FrontierEntry) * np1));
+    launch_fr_init(t, of_parity(0), dg.out_off, d_pw, g->cfg.eps_p, ws->f_list[0].as<FrontierEntry>(), st);
     ++launches;
+    bool live = NP > 0;
     for (;;) {
-        if (nF == 0) {  // the range ran out: resume the last deferred one
+        if (!live) {  // the range ran out: resume the last deferred one
             if (stack.empty()) break;
-            const Task tk = stack.back();
+            R = stack.back();
             stack.pop_back();
-            PS_ALLOC(grow_list(cur, std::max<long long>(1, tk.count), 0, st));
-            const FrontierList F = list_of(cur);
-            PS_CUDA(cudaMemcpyAsync(F.p, ws->f_sp.as<int32_t>() + tk.at, sizeof(int32_t) * tk.count, cudaMemcpyDeviceToDevice, st));
-            PS_CUDA(cudaMemcpyAsync(F.x, ws->f_sx.as<int32_t>() + tk.at, sizeof(int32_t) * tk.count, cudaMemcpyDeviceToDevice, st));
-            PS_CUDA(cudaMemcpyAsync(F.val, ws->f_sv.as<float>() + tk.at, sizeof(float) * tk.count, cudaMemcpyDeviceToDevice, st));
-            stack_top = tk.at;
-            p0 = tk.p0, p1 = tk.p1, j = tk.j, nF = tk.count;
             ws->stats.deferred += 1;
+            live = true;
         }
-        const FrontierList F = list_of(cur);
-        const int32_t np_ = p1 - p0;
-        PS_ALLOC(ws->f_wp.ensure(sizeof(long long) * (nF + 1)));
-        PS_ALLOC(ws->r_part.ensure(sizeof(long long) * scan64_partials_needed(std::max<int64_t>(nF, np_))));
-        long long *wp = ws->f_wp.as<long long>();
-        launch_fr_prune(F, nF, t, PR, dg.out_off, d_pw, g->cfg.eps_p, j, wp, st);
-        launch_fr_regions(t, PR, p0, p1, j, n, d_thr, t_sw, st);
-        launch_fr_work(F, nF, PR, wp, st);
-        launch_scan64(wp, nF, ws->r_part.as<long long>(), wp, st);  // in place: wp[f] = first work item of entry f
-        launch_scan64(PR.rsize + p0, np_, ws->r_part.as<long long>(), PR.roff + p0, st);
-        launch_scan64(PR.dsize + p0, np_, ws->r_part.as<long long>(), PR.doff + p0, st);
-        launches += 12;
-        PS_CUDA(cudaMemcpyAsync(h_ll, wp + nF, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        PS_CUDA(cudaMemcpyAsync(h_ll + 1, PR.roff + p1, sizeof(long long), cudaMemcpyDeviceToHost, st));
-        PS_CUDA(cudaMemcpyAsync(h_ll + 2, PR.doff + p1, sizeof(long long), cudaMemcpyDeviceToHost, st));
+        const FrontierEntry *src = R.on_stack ? ws->f_stack.as<FrontierEntry>() : ws->f_list[R.cur].as<FrontierEntry>();
+        PS_CUDA(cudaMemsetAsync(d_tot, 0, sizeof(unsigned long long) * 2 * kFrTotals, st));  // and the cursors
+        if (d_thr && g->cfg.eps_p <= 0.f) {
+            launch_fr_check(dg, t, of_parity(R.cur), R.p0, R.p1, R.j, src, d_thr, t_sw, st);
+            ++launches;
+        }
+        launch_fr_plan(t, of_parity(R.cur), R.p0, R.p1, R.j, n, d_thr, t_sw, d_tot, st);
+        ++launches;
+        PS_CUDA(cudaMemcpyAsync(h_tot, d_tot, sizeof(unsigned long long) * kFrTotals, cudaMemcpyDeviceToHost, st));
         PS_CUDA(cudaStreamSynchronize(st));
-        const long long E = h_ll[0], T = h_ll[1], Dtot = h_ll[2];
-        ws->stats.edge_gathers += E;
-        ws->stats.levels += 1;
-        if (E == 0) {  // nothing left to push: every probe of the range ended, switched or was pruned
-            nF = 0;
+        const long long D = (long long)h_tot[kFrTotD], G = (long long)h_tot[kFrTotGlobal];
+        if (h_tot[kFrTotItems] == 0) {  // nothing left to push: every probe of the range ended, switched or was pruned
+            if (R.on_stack) stack_top = R.at;
+            live = false;
             continue;
         }
-        const int nx = cur ^ 1;
-        // passes: probe ranges whose regions fit pass_slots (roff and doff are relative to p0)
-        std::vector<int32_t> cuts{p0};
-        if (T > pass_slots) {
-            std::vector<long long> roff(np_ + 1);
-            PS_CUDA(cudaMemcpyAsync(roff.data(), PR.roff + p0, sizeof(long long) * (np_ + 1), cudaMemcpyDeviceToHost, st));
-            PS_CUDA(cudaStreamSynchronize(st));
-            int32_t a = 0;
-            while (a < np_) {
-                int32_t b = (int32_t)(std::upper_bound(roff.begin() + a + 1, roff.end(), roff[a] + pass_slots) -
-                                      roff.begin()) - 1;
-                if (b <= a) b = a + 1;
-                cuts.push_back(p0 + b);
-                a = b;
-            }
-        } else {
-            cuts.push_back(p1);
-        }
-        const int32_t npass = (int32_t)cuts.size() - 1;
-        // per cut: first entry, work prefix, region offset, next-entry bound offset
-        std::vector<long long> cb(4 * (size_t)(npass + 1));
-        if (npass == 1) {
-            cb = {0, 0, 0, 0, nF, E, T, Dtot};
-        } else {
-            PS_ALLOC(ws->f_cuts.ensure(sizeof(int32_t) * cuts.size() + 32 * cuts.size() + 16));
-            int32_t *d_cuts = ws->f_cuts.as<int32_t>();
-            long long *d_cb = reinterpret_cast<long long *>(ws->f_cuts.as<char>() + ((sizeof(int32_t) * cuts.size() + 15) / 16 * 16));
-            PS_CUDA(cudaMemcpyAsync(d_cuts, cuts.data(), sizeof(int32_t) * cuts.size(), cudaMemcpyHostToDevice, st));
-            launch_fr_bounds(F.p, nF, wp, PR.roff, PR.doff, d_cuts, (int32_t)cuts.size(), d_cb, st);
-            ++launches;
-            PS_CUDA(cudaMemcpyAsync(cb.data(), d_cb, sizeof(long long) * cb.size(), cudaMemcpyDeviceToHost, st));
-            PS_CUDA(cudaStreamSynchronize(st));
-        }
-        ws->stats.table_passes += npass;
-        ws->stats.max_table_slots = std::max<int64_t>(ws->stats.max_table_slots, T);
-        const long long tslots = std::max<long long>(1, std::min<long long>(T, pass_slots + n));
-        {
-            const void *k0 = ws->f_keys.p;
-            PS_ALLOC(ws->f_keys.ensure(sizeof(FrontierSlot) * tslots));
-            if (ws->f_keys.p != k0 || !ws->f_table_clean) {  // new memory, or a failed call left slots behind
-                PS_CUDA(cudaMemsetAsync(ws->f_keys.p, 0, ws->f_keys.cap, st));
-                ws->f_table_clean = true;
-            }
-        }
-        PS_ALLOC(ws->f_bcnt.ensure(sizeof(long long) * (fr_compact_blocks(tslots) + 1)));
-        PS_ALLOC(ws->f_bpre.ensure(sizeof(long long) * (fr_compact_blocks(tslots) + 1)));
-        PS_ALLOC(ws->r_part.ensure(sizeof(long long) * scan64_partials_needed(std::max<int64_t>(
-                                       std::max<int64_t>(nF, np_), fr_compact_blocks(tslots)))));
-        long long out_n = 0;
-        int32_t pk = p1;  // probes [p0, pk) advance to level j + 1
-        for (int32_t c = 0; c < npass; ++c) {
-            const long long f_lo = cb[4 * c], e_lo = cb[4 * c + 1], r0 = cb[4 * c + 2], d0 = cb[4 * c + 3];
-            const long long f_hi = cb[4 * (c + 1)], e_hi = cb[4 * (c + 1) + 1], r1 = cb[4 * (c + 1) + 2],
-                            d1 = cb[4 * (c + 1) + 3];
-            if (out_n > 0 && out_n + (d1 - d0) > list_cap) {  // defer probes [cuts[c], p1) at level j
-                const long long cnt = nF - f_lo;
-                PS_ALLOC(ws->f_sp.grow(sizeof(int32_t) * (stack_top + cnt), sizeof(int32_t) * stack_top, st));
-                PS_ALLOC(ws->f_sx.grow(sizeof(int32_t) * (stack_top + cnt), sizeof(int32_t) * stack_top, st));
-                PS_ALLOC(ws->f_sv.grow(sizeof(float) * (stack_top + cnt), sizeof(float) * stack_top, st));
-                PS_CUDA(cudaMemcpyAsync(ws->f_sp.as<int32_t>() + stack_top, F.p + f_lo, sizeof(int32_t) * cnt, cudaMemcpyDeviceToDevice, st));
-                PS_CUDA(cudaMemcpyAsync(ws->f_sx.as<int32_t>() + stack_top, F.x + f_lo, sizeof(int32_t) * cnt, cudaMemcpyDeviceToDevice, st));
-                PS_CUDA(cudaMemcpyAsync(ws->f_sv.as<float>() + stack_top, F.val + f_lo, sizeof(float) * cnt, cudaMemcpyDeviceToDevice, st));
-                stack.push_back({cuts[c], p1, j, stack_top, cnt});
-                stack_top += cnt;
-                pk = cuts[c];
-                break;
-            }
-            const long long Tc = r1 - r0;
-            FrontierExpand a;
-            a.wp = wp;
-            a.f_lo = f_lo;
-            a.f_hi = f_hi;
-            a.e_lo = e_lo;
-            a.e_hi = e_hi;
-            a.j = j;
-            a.tab = ws->f_keys.as<FrontierSlot>();
-            a.rbase = r0;
-            a.acc = ws->f_acc.as<unsigned long long>();
-            a.n = n;
-            if (Tc > 0) ws->f_table_clean = false;  // until this pass's compaction has emptied its slots
-            launch_fr_expand(dg, t, PR, F, a, st);
-            ++launches;
-            if (Tc > 0) {  // count the pass's occupied slots, grow the next list to hold them, write them
-                const int64_t nb = fr_compact_blocks(Tc);
-                launch_fr_count(a.tab, Tc, ws->f_bcnt.as<long long>(), st);
-                launch_scan64(ws->f_bcnt.as<long long>(), nb, ws->r_part.as<long long>(), ws->f_bpre.as<long long>(), st);
-                PS_CUDA(cudaMemcpyAsync(h_ll, ws->f_bpre.as<long long>() + nb, sizeof(long long), cudaMemcpyDeviceToHost, st));
+        if ((D > list_cap || G > slot_cap) && R.p1 - R.p0 > 1) {  // defer the range's last probes
+            const double keep = 0.9 * std::min(D > 0 ? (double)list_cap / (double)D : 1.0,
+                                               G > 0 ? (double)slot_cap / (double)G : 1.0);
+            const int32_t pm = R.p0 + std::max(1, (int32_t)std::min<double>(keep * (R.p1 - R.p0), R.p1 - R.p0 - 1));
+            Range tail{pm, R.p1, R.j, R.cur, true, R.on_stack ? R.at : stack_top};
+            if (!R.on_stack) {
+                const long long cnt = (long long)h_tot[kFrTotEntries];  // of the whole range: enough
+                PS_ALLOC(ws->f_stack.grow(sizeof(FrontierEntry) * (stack_top + cnt), sizeof(FrontierEntry) * stack_top,
+                                          st));
+                h_tot[0] = (unsigned long long)stack_top;
+                PS_CUDA(cudaMemcpyAsync(d_top, h_tot, sizeof(unsigned long long), cudaMemcpyHostToDevice, st));
+                launch_fr_defer(of_parity(R.cur), pm, R.p1, src, ws->f_stack.as<FrontierEntry>(), d_top, st);
+                ++launches;
+                PS_CUDA(cudaMemcpyAsync(h_tot, d_top, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
                 PS_CUDA(cudaStreamSynchronize(st));
-                const long long need = std::max<long long>(1, out_n + h_ll[0]);
-                PS_ALLOC(grow_list(nx, need, out_n, st));
-                launch_fr_write(a.tab, Tc, PR.roff, cuts[c], cuts[c + 1], r0, ws->f_bpre.as<long long>(),
-                                list_of(nx), out_n, need, st);
-                launches += 5;
-                out_n += h_ll[0];
-                ws->f_table_clean = true;
+                stack_top = (long long)h_tot[0];
             }
+            // a range read from the stack leaves its tail where it is: the tail then owns the space down to R.at
+            stack.push_back(tail);
+            if (R.on_stack) R.at = stack_top;
+            R.p1 = pm;
+            continue;
         }
-        launch_fr_advance(t, PR, p0, pk, st);
+        ws->stats.edge_gathers += (int64_t)h_tot[kFrTotItems];
+        ws->stats.levels += 1;
+        if (D > 0) ws->stats.table_passes += 1;
+        ws->stats.max_table_slots = std::max<int64_t>(ws->stats.max_table_slots, (int64_t)h_tot[kFrTotSlots]);
+        FrontierBases base;
+        long long nt = 0;
+        for (int c = kFrNone + 1; c < kFrClasses; ++c) {
+            base.at[c] = nt;
+            nt += (long long)h_tot[c];
+            if (h_tot[c] >= ((unsigned long long)1 << 31)) return fail(PROBESIM_E_INVALID, "too much work in one call");
+        }
+        const int nx = R.cur ^ 1;
+        PS_ALLOC(ws->f_list[nx].ensure(sizeof(FrontierEntry) * std::max<long long>(1, D)));
+        PS_ALLOC(ws->f_tasks.ensure(sizeof(FrontierTask) * std::max<long long>(1, nt)));
+        if (G > 0) {
+            const void *k0 = ws->f_keys.p;
+            PS_ALLOC(ws->f_keys.ensure(sizeof(FrontierSlot) * G));
+            if (ws->f_keys.p != k0 || !ws->f_table_clean)  // new memory, or a failed call left slots behind
+                PS_CUDA(cudaMemsetAsync(ws->f_keys.p, 0, ws->f_keys.cap, st));
+            ws->f_table_clean = false;  // until this level's sweep has emptied its slots
+        }
+        launch_fr_tasks(of_parity(R.cur), R.p0, R.p1, n, base, d_cursor, ws->f_tasks.as<FrontierTask>(), st);
         ++launches;
-        p1 = pk;
-        nF = out_n;
-        cur = nx;
-        ++j;
+        FrontierLevel a;
+        a.tasks = ws->f_tasks.as<FrontierTask>();
+        a.src = src;
+        a.dst = ws->f_list[nx].as<FrontierEntry>();
+        a.tab = ws->f_keys.as<FrontierSlot>();
+        a.acc = ws->f_acc.as<unsigned long long>();
+        a.pw = d_pw;
+        a.eps_p = g->cfg.eps_p;
+        a.j = R.j;
+        PS_CUDA(launch_fr_level(dg, t, of_parity(R.cur), a, base, h_tot, st, &launches));
+        PS_CUDA(cudaGetLastError());
+        if (G > 0) ws->f_table_clean = true;
+        if (R.on_stack) stack_top = R.at;
+        R = Range{R.p0, R.p1, R.j + 1, nx, false, 0};
     }
     launch_fr_count_switched(PR, d_fctr, st);
     PS_CUDA(cudaMemcpyAsync(h_ll, d_fctr, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
@@ -1320,10 +1259,6 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
     // Sec. 4.4: Alg. 3 for every walk through a switched tree node
     const int32_t *counts = nullptr;
     if (switched > 0) {
-        // the deterministic rounds' tables and lists are done with: their memory goes to Alg. 3's hash sets
-        for (DevBuf *b : {&ws->f_keys, &ws->f_lp[0], &ws->f_lp[1], &ws->f_lx[0], &ws->f_lx[1],
-                          &ws->f_lv[0], &ws->f_lv[1], &ws->f_wp, &ws->f_sp, &ws->f_sx, &ws->f_sv})
-            b->release();
         PS_TRY(rand_instances(g, ws, qb, B, P.W, max_len, walk_nodes, t.walk_slot, t_sw, launches, st, too_big));
         counts = ws->r_counts.as<int32_t>();
     }
