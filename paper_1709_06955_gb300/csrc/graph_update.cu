@@ -146,55 +146,99 @@ __global__ void k_upd_w(int32_t n, const long long *__restrict__ new_off, const 
     npieces[v] = d <= kPiece ? 1 : (d + kPiece - 1) / kPiece;
 }
 
-// counts pieces per length (0..kPiece) and lists the split rows
-__global__ void k_upd_piece_hist(int32_t n, const long long *__restrict__ new_off, unsigned long long *hist,
-                                 int32_t *split_v, unsigned long long *n_split) {
-    const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    const long long d = new_off[v + 1] - new_off[v];
-    if (d <= kPiece) {
-        atomicAdd(&hist[d], 1ull);
-    } else {
-        atomicAdd(&hist[kPiece], (unsigned long long)(d / kPiece));
-        if (d % kPiece) atomicAdd(&hist[d % kPiece], 1ull);
-        split_v[atomicAdd(n_split, 1ull)] = (int32_t)v;
-    }
+// Pull pieces, a counting sort by (row has out-edges first, then length, longest first): the pieces of the rows that
+// somebody reads (below *n_active) come first, so a pull whose result is only gathered runs over them alone.  Bucket of
+// a piece: length for an active row, kPiece + 1 + length for another.  A block takes a range of rows and counts in shared
+// memory; with one global counter per length a million rows queued on a few hot counters (R-MAT 2^21: 0.81 and 1.01 ms
+// for the two passes, now 0.01 and 0.12).
+constexpr int kPieceBuckets = 2 * (kPiece + 1);
+constexpr int kPieceThreads = 256;
+
+__device__ __forceinline__ void piece_counts(long long d, bool active, int *full, int *rest, int *fb, int *rb) {
+    const int base = active ? 0 : kPiece + 1;
+    *full = d <= kPiece ? 0 : (int)(d / kPiece);
+    *rest = d <= kPiece ? 1 : (d % kPiece != 0);
+    *fb = base + kPiece;
+    *rb = base + (d <= kPiece ? (int)d : (int)(d % kPiece));
 }
 
-// bucket starts, longest first: start[len] = sum of hist[l] for l > len
-__global__ void k_upd_piece_starts(unsigned long long *hist, unsigned long long *cursor) {
+__global__ void __launch_bounds__(kPieceThreads) k_upd_piece_hist(int32_t n, const long long *__restrict__ new_off,
+                                                                  const int32_t *__restrict__ n_active,
+                                                                  unsigned long long *hist, int32_t *split_v,
+                                                                  unsigned long long *n_split) {
+    __shared__ unsigned s_h[kPieceBuckets];
+    for (int i = threadIdx.x; i < kPieceBuckets; i += kPieceThreads) s_h[i] = 0;
+    __syncthreads();
+    const int64_t per = ((int64_t)n + gridDim.x - 1) / gridDim.x;
+    const int64_t beg = blockIdx.x * per, end = min((int64_t)n, beg + per);
+    const int32_t act = *n_active;
+    for (int64_t v = beg + threadIdx.x; v < end; v += kPieceThreads) {
+        const long long d = new_off[v + 1] - new_off[v];
+        int full, rest, fb, rb;
+        piece_counts(d, v < act, &full, &rest, &fb, &rb);
+        if (full) {
+            atomicAdd(&s_h[fb], (unsigned)full);
+            split_v[atomicAdd(n_split, 1ull)] = (int32_t)v;
+        }
+        if (rest) atomicAdd(&s_h[rb], 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kPieceBuckets; i += kPieceThreads)
+        if (s_h[i]) atomicAdd(&hist[i], (unsigned long long)s_h[i]);
+}
+
+// bucket starts: active rows' pieces longest first, then the others'
+__global__ void k_upd_piece_starts(const unsigned long long *hist, unsigned long long *cursor) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     unsigned long long acc = 0;
-    for (int len = kPiece; len >= 0; --len) {
-        cursor[len] = acc;
-        acc += hist[len];
-    }
+    for (int c = 0; c < 2; ++c)
+        for (int len = kPiece; len >= 0; --len) {
+            cursor[c * (kPiece + 1) + len] = acc;
+            acc += hist[c * (kPiece + 1) + len];
+        }
 }
 
-__global__ void k_upd_piece_fill(int32_t n, const long long *__restrict__ new_off, unsigned long long *cursor,
-                                 int32_t *pv, int64_t *pb, int32_t *pl) {
-    const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    const long long beg = new_off[v], d = new_off[v + 1] - beg;
-    if (d <= kPiece) {
-        const unsigned long long i = atomicAdd(&cursor[d], 1ull);
-        pv[i] = (int32_t)v;
-        pb[i] = beg;
-        pl[i] = (int32_t)d;
-        return;
+__global__ void __launch_bounds__(kPieceThreads) k_upd_piece_fill(int32_t n, const long long *__restrict__ new_off,
+                                                                  const int32_t *__restrict__ n_active,
+                                                                  unsigned long long *cursor, int32_t *pv, int64_t *pb,
+                                                                  int32_t *pl) {
+    __shared__ unsigned s_h[kPieceBuckets];
+    __shared__ unsigned long long s_at[kPieceBuckets];
+    for (int i = threadIdx.x; i < kPieceBuckets; i += kPieceThreads) s_h[i] = 0;
+    __syncthreads();
+    const int64_t per = ((int64_t)n + gridDim.x - 1) / gridDim.x;
+    const int64_t beg = blockIdx.x * per, end = min((int64_t)n, beg + per);
+    const int32_t act = *n_active;
+    for (int64_t v = beg + threadIdx.x; v < end; v += kPieceThreads) {
+        int full, rest, fb, rb;
+        piece_counts(new_off[v + 1] - new_off[v], v < act, &full, &rest, &fb, &rb);
+        if (full) atomicAdd(&s_h[fb], (unsigned)full);
+        if (rest) atomicAdd(&s_h[rb], 1u);
     }
-    const long long full = d / kPiece, rest = d % kPiece;
-    for (long long c = 0; c < full; ++c) {
-        const unsigned long long i = atomicAdd(&cursor[kPiece], 1ull);
-        pv[i] = (int32_t)v;
-        pb[i] = beg + c * kPiece;
-        pl[i] = kPiece | (int32_t)0x80000000;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kPieceBuckets; i += kPieceThreads) {
+        if (s_h[i]) s_at[i] = atomicAdd(&cursor[i], (unsigned long long)s_h[i]);
+        s_h[i] = 0;  // each row's places are counted off again
     }
-    if (rest) {
-        const unsigned long long i = atomicAdd(&cursor[rest], 1ull);
-        pv[i] = (int32_t)v;
-        pb[i] = beg + full * kPiece;
-        pl[i] = (int32_t)rest | (int32_t)0x80000000;
+    __syncthreads();
+    for (int64_t v = beg + threadIdx.x; v < end; v += kPieceThreads) {
+        const long long b0 = new_off[v], d = new_off[v + 1] - b0;
+        int full, rest, fb, rb;
+        piece_counts(d, v < act, &full, &rest, &fb, &rb);
+        if (full) {
+            const unsigned long long i0 = s_at[fb] + atomicAdd(&s_h[fb], (unsigned)full);
+            for (int c = 0; c < full; ++c) {
+                pv[i0 + c] = (int32_t)v;
+                pb[i0 + c] = b0 + (long long)c * kPiece;
+                pl[i0 + c] = kPiece | (int32_t)0x80000000;
+            }
+        }
+        if (rest) {
+            const unsigned long long i = s_at[rb] + atomicAdd(&s_h[rb], 1u);
+            pv[i] = (int32_t)v;
+            pb[i] = b0 + (long long)full * kPiece;
+            pl[i] = d <= kPiece ? (int32_t)d : ((int32_t)(d % kPiece) | (int32_t)0x80000000);
+        }
     }
 }
 
@@ -235,14 +279,15 @@ void launch_upd_w(int32_t n, const long long *new_off, const int32_t *in_col, fl
     k_upd_w<<<blocks_for(n, 256), 256, 0, s>>>(n, new_off, in_col, sqrt_c, int2ext, rec_shift, w, rec, npieces);
 }
 
-void launch_upd_pieces(int32_t n, const long long *new_off, unsigned long long *hist, unsigned long long *cursor,
-                       int32_t *split_v, unsigned long long *n_split, int32_t *pv, int64_t *pb, int32_t *pl,
-                       cudaStream_t s) {
-    cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * (kPiece + 1), s);
+void launch_upd_pieces(int32_t n, const long long *new_off, const int32_t *n_active, unsigned long long *hist,
+                       unsigned long long *cursor, int32_t *split_v, unsigned long long *n_split, int32_t *pv,
+                       int64_t *pb, int32_t *pl, cudaStream_t s) {
+    cudaMemsetAsync(hist, 0, sizeof(unsigned long long) * kPieceBuckets, s);
     cudaMemsetAsync(n_split, 0, sizeof(unsigned long long), s);
-    k_upd_piece_hist<<<blocks_for(n, 256), 256, 0, s>>>(n, new_off, hist, split_v, n_split);
+    const int blocks = grid_for(n, 4 * kPieceThreads, 4);
+    k_upd_piece_hist<<<blocks, kPieceThreads, 0, s>>>(n, new_off, n_active, hist, split_v, n_split);
     k_upd_piece_starts<<<1, 32, 0, s>>>(hist, cursor);
-    k_upd_piece_fill<<<blocks_for(n, 256), 256, 0, s>>>(n, new_off, cursor, pv, pb, pl);
+    k_upd_piece_fill<<<blocks, kPieceThreads, 0, s>>>(n, new_off, n_active, cursor, pv, pb, pl);
 }
 
 void launch_i64_copy(const long long *a, int64_t *b, int64_t count, cudaStream_t s) {

@@ -44,8 +44,8 @@ __device__ __forceinline__ U32x4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
 // ---------------------------------------------------------------------------------------------
 // Device graph store: in-adjacency I(v) sorted by source id (walks pick the k-th entry), out-
 // adjacency O(x) sorted by destination id, w[v] = sqrt(c)/|I(v)| (0 when |I(v)| = 0), and the work
-// decomposition of the pull kernel: every in-list cut into pieces of at most kPiece edges, ordered
-// by length (longest first).  A piece of a vertex cut into several pieces is added atomically.
+// decomposition of the pull kernel: every in-list cut into pieces of at most kPiece edges, those of rows with
+// out-edges first, ordered by length (longest first).  A piece of a vertex cut into several pieces is added atomically.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPiece = 128;
 
@@ -58,6 +58,7 @@ struct DeviceGraph {
     int32_t *out_col = nullptr;
     float *w = nullptr;
     int64_t n_pieces = 0;
+    int64_t n_pieces_active = 0;   // the first of them: those of the rows below n_active
     int32_t *piece_v = nullptr;
     int64_t *piece_beg = nullptr;
     int32_t *piece_len = nullptr;  // length | (split ? 1 << 31 : 0)
@@ -388,9 +389,10 @@ inline int32_t rec_shift_for(int32_t n) {  // ids below n, shifted, fit 8 bits
     while (((int64_t)(n - 1) >> b) > 255) ++b;
     return b;
 }
-void launch_upd_pieces(int32_t n, const long long *new_off, unsigned long long *hist, unsigned long long *cursor,
-                       int32_t *split_v, unsigned long long *n_split, int32_t *pv, int64_t *pb, int32_t *pl,
-                       cudaStream_t s);
+// hist and cursor hold 2 (kPiece + 1) counters (see k_upd_piece_hist); *n_active (device) is launch_active_rows' result
+void launch_upd_pieces(int32_t n, const long long *new_off, const int32_t *n_active, unsigned long long *hist,
+                       unsigned long long *cursor, int32_t *split_v, unsigned long long *n_split, int32_t *pv,
+                       int64_t *pb, int32_t *pl, cudaStream_t s);
 void launch_i64_copy(const long long *a, int64_t *b, int64_t count, cudaStream_t s);
 
 // device-side initial build of the graph store (graph_build.cu)
