@@ -132,7 +132,7 @@ struct LaunchCounters {
 // tile of 32 columns then gathers 128 B per row from inside one block of n KB whatever the total width,
 // while the kernels that touch many columns of one row (accumulate, gamma) still find them in one row.
 // Every layout has one spare row, row n: the pull pads the last chunk of an in-list with index n, and that
-// row is zeroed before each pull reads the matrix (launch_zero_spare_row).
+// row is zeroed before each pull reads the matrix (launch_prepare_pull).
 constexpr int32_t kGroup = 256;
 constexpr int64_t kGroupSkew = kGroup + 5 * 32;  // floats: the spare row, then five 128-byte lines
 
@@ -189,20 +189,22 @@ void launch_sched_count(TrieTable t, int32_t *ncount, int32_t *scount, int32_t *
 void launch_sched_export(TrieTable t, int32_t *out, int32_t *count, cudaStream_t s);
 void launch_node_lists(TrieTable t, const int32_t *node_off, int32_t *ncur, int32_t *node_list, cudaStream_t s);
 void launch_set_slots(TrieTable t, const int32_t *pairs, int32_t count, cudaStream_t s);
-void launch_scatter_gamma(const int32_t *nodes, int32_t cnt, TrieTable t, float *D, ColLayout L, cudaStream_t s);
+// scatters the gammas of the tree nodes two depths down into B, and zeroes B's spare row and A's split rows over the
+// pulled columns
+void launch_prepare_pull(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *B, ColLayout Lb,
+                         float *A, ColLayout La, int32_t width, cudaStream_t s);
 // inherited = false: push nodes whose column is in the push block (slot >= h0); true: those whose column
 // was inherited from the parent (slot < h0)
 void launch_push_h2(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *MD, ColLayout L,
                     int32_t h0, bool inherited, cudaStream_t s);
 // Parts of at most four sources: p1 (the first part of every group: bit 30 of the destination = set, else add)
 // then p2 (later parts: add).  Sources are -1 where absent.
-void launch_accumulate(int32_t n, float *B, ColLayout L, const int32_t *p1dst, const int4 *p1src, int32_t np1,
-                       const int32_t *p2dst, const int4 *p2src, int32_t np2, cudaStream_t s);
+// W = the columns of a row of B that hold data (a multiple of 4), nsrc = the sources of all parts.
+cudaError_t launch_accumulate(int32_t n, float *B, ColLayout L, int32_t W, int64_t nsrc, const int32_t *p1dst,
+                              const int4 *p1src, int32_t np1, const int32_t *p2dst, const int4 *p2src, int32_t np2,
+                              cudaStream_t s);
 // zeroes columns [c0, c0 + width) rounded up to a multiple of 4 (c0 a multiple of 4, inside the pitch)
 void launch_zero_cols(int32_t n, float *MD, ColLayout L, int32_t c0, int32_t width, cudaStream_t s);
-void launch_zero_split_rows(const DeviceGraph &g, float *MD, ColLayout L, int32_t width, cudaStream_t s);
-// zeroes columns [0, width) of the spare row n
-void launch_zero_spare_row(float *MD, ColLayout L, int32_t width, cudaStream_t s);
 // pull MD[v][c] = w[v] * sum_{x in I(v)} D[x][c] over ntiles tiles of `tile` columns.  D and MD point at the
 // first tile's column in row 0; their rows are dpitch / pitch floats apart; tile j of D starts (j / dsub) * dts +
 // (j % dsub) * tile floats after the first, and likewise for MD with mts / msub (ColLayout::tile_stride/sub).

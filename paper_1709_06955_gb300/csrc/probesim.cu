@@ -630,6 +630,7 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
     // accumulate's first phase, the others add in a second phase (so one node with many children does not
     // hold up a block).  Records of depth d: first parts [p1_at[d], p1_at[d+1]), later parts likewise.
     std::vector<int32_t> pairs, p1dst, p1src, p2dst, p2src, p1_at(D1 + 1, 0), p2_at(D1 + 1, 0);
+    std::vector<int64_t> acc_src(D1, 0);  // sources of a depth's parts
     pairs.reserve(2 * (size_t)ncol_nodes);
     for (int32_t i = 0; i < ncol_nodes; ++i) {
         pairs.push_back(h_exp[5 * i]);
@@ -650,6 +651,7 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
             std::sort(kids[i].begin(), kids[i].end());
             const bool own = heir[i] < 0 && pheir[i] < 0;  // no heir of any kind: the column is set
             if (kids[i].empty() && !own) continue;            // its column already is its heir's MD
+            acc_src[d] += (int64_t)kids[i].size();
             put_part(p1dst, p1src, col[i] | (own ? (1 << 30) : 0), kids[i], 0);
             for (size_t f = 4; f < kids[i].size(); f += 4) put_part(p2dst, p2src, col[i], kids[i], f);
         }
@@ -749,24 +751,15 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
             ph.begin(2);  // D of this depth's dense nodes, in place in B (the MD of depth d+1)
             const int32_t np1 = p1_at[d + 1] - p1_at[d], np2 = p2_at[d + 1] - p2_at[d];
             if (np1 > 0)
-                launch_accumulate(dg.n_active, Bm, Lb, d_sched + o_p1dst + p1_at[d],
-                                  reinterpret_cast<const int4 *>(d_sched + o_p1src) + p1_at[d], np1,
-                                  d_sched + o_p2dst + p2_at[d],
-                                  reinterpret_cast<const int4 *>(d_sched + o_p2src) + p2_at[d], np2, st);
+                PS_CUDA(launch_accumulate(dg.n_active, Bm, Lb, rpv[d + 1], acc_src[d], d_sched + o_p1dst + p1_at[d],
+                                          reinterpret_cast<const int4 *>(d_sched + o_p1src) + p1_at[d], np1,
+                                          d_sched + o_p2dst + p2_at[d],
+                                          reinterpret_cast<const int4 *>(d_sched + o_p2src) + p2_at[d], np2, st));
             ph.end();
             ++launches;
-            if (d + 2 <= Dmax) {
-                ph.begin(3);
-                launch_scatter_gamma(node_list + node_off[d + 2], ncount[d + 2], t, Bm, Lb, st);
-                ph.end();
-                ++launches;
-            }
-            ph.begin(4);
-            launch_zero_spare_row(Bm, Lb, dw[d], st);  // the pull's padding gathers read it
-            if (dg.n_split > 0) {
-                launch_zero_split_rows(dg, A, La, dw[d], st);
-                ++launches;
-            }
+            ph.begin(3);  // gamma scatter into D; the spare row and the split rows zeroed for the pull
+            launch_prepare_pull(dg, d + 2 <= Dmax ? node_list + node_off[d + 2] : nullptr,
+                                d + 2 <= Dmax ? ncount[d + 2] : 0, t, Bm, Lb, A, La, dw[d], st);
             ph.end();
             ++launches;
             cudaEvent_t e0 = nullptr, e1 = nullptr;
