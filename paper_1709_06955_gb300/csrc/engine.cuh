@@ -186,7 +186,7 @@ struct probesim_graph {
     }
     std::vector<int32_t> h_ext2int;  // host copy of the id map (update batches are sorted by internal ids)
     // update scratch
-    DevBuf u_batch, u_valid, u_vpre, u_delta, u_deg, u_part, u_hist;
+    DevBuf u_batch, u_valid, u_vpre, u_delta, u_deg, u_part, u_hist, u_bounds;
     uint64_t epoch = 0;
     Workspace ws0;
     std::atomic<size_t> budget{0};  // device memory one call's working buffers may take (set while calls run)

@@ -381,8 +381,10 @@ struct UpdateBatchArgs {
 void launch_upd_mark(const DeviceGraph &g, const UpdateBatchArgs &a, long long *in_delta, long long *out_delta,
                      cudaStream_t s);
 void launch_upd_degrees(int32_t n, const int64_t *off, const long long *delta, long long *deg, cudaStream_t s);
+// bounds: scratch of upd_bounds_bytes(a.k)
+size_t upd_bounds_bytes(int64_t k);
 void launch_upd_rows(const DeviceGraph &g, const UpdateBatchArgs &a, bool in_lists, const long long *new_off,
-                     int32_t *new_col, cudaStream_t s);
+                     int32_t *new_col, void *bounds, cudaStream_t s);
 // w, the node records (DeviceGraph::rec) and the number of pull pieces of every row
 void launch_upd_w(int32_t n, const long long *new_off, const int32_t *in_col, float sqrt_c, const int32_t *int2ext,
                   int32_t rec_shift, float *w, int4 *rec, long long *npieces, cudaStream_t s);

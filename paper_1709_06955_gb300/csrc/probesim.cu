@@ -1496,7 +1496,7 @@ probesim_status probesim_graph_destroy(probesim_graph *g) {
     if (!g) return PROBESIM_OK;
     g->store.reset();
     DevBuf *bufs[] = {&g->ext2int, &g->int2ext, &g->u_batch, &g->u_valid,
-                      &g->u_vpre, &g->u_delta, &g->u_deg, &g->u_part, &g->u_hist};
+                      &g->u_vpre, &g->u_delta, &g->u_deg, &g->u_part, &g->u_hist, &g->u_bounds};
     for (DevBuf *b : bufs) b->release();
     g->ws0.release();
     delete g;
@@ -1566,6 +1566,7 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     const DeviceGraph &dg = old->dg;
     auto nv = std::make_shared<StoreVersion>();  // the next version, built beside the current one
     PS_CUDA(g->u_batch.ensure(sizeof(int32_t) * 5 * K));
+    PS_CUDA(g->u_bounds.ensure(upd_bounds_bytes(K)));
     PS_CUDA(g->u_valid.ensure(sizeof(long long) * 2 * K));
     PS_CUDA(g->u_vpre.ensure(sizeof(long long) * 2 * (K + 1)));
     PS_CUDA(g->u_delta.ensure(sizeof(long long) * 2 * (size_t)n));
@@ -1607,8 +1608,8 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     if (m2 >= ((int64_t)1 << 31)) return fail(PROBESIM_E_INVALID, "edge count would reach 2^31");
     PS_CUDA(n_in_col.alloc_pooled(sizeof(int32_t) * std::max<int64_t>(1, m2), st));
     PS_CUDA(n_out_col.alloc_pooled(sizeof(int32_t) * std::max<int64_t>(1, m2), st));
-    launch_upd_rows(dg, a, true, n_in_off.as<long long>(), n_in_col.as<int32_t>(), st);
-    launch_upd_rows(dg, a, false, n_out_off.as<long long>(), n_out_col.as<int32_t>(), st);
+    launch_upd_rows(dg, a, true, n_in_off.as<long long>(), n_in_col.as<int32_t>(), g->u_bounds.p, st);
+    launch_upd_rows(dg, a, false, n_out_off.as<long long>(), n_out_col.as<int32_t>(), g->u_bounds.p, st);
     // w and pieces of the new in-lists
     const int64_t cap_pieces = (int64_t)n + m2 / kPiece + 1;
     DevBuf &n_pv = nv->piece_v, &n_pb = nv->piece_beg, &n_pl = nv->piece_len, &n_split = nv->split_v;
