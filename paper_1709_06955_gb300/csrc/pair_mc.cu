@@ -3,8 +3,7 @@
 // with r >= ln(1/delta) / (2 eps^2) it is within eps of s(u, v) with probability 1 - delta (Chernoff).  It serves
 // as the single-pair "expert" that gauges pooled top-k candidates on graphs too large for the Power Method.
 //
-// One thread per walk pair t: the two walks advance in lockstep, their i-th nodes compared at every position
-// both reach.  Walk t from u draws Philox counter (t, s, 0, 0) under key (seed, key_u) at step s -- the draws
+// The two walks of a walk pair t advance in lockstep, their i-th nodes compared at every position both reach.  Walk t from u draws Philox counter (t, s, 0, 0) under key (seed, key_u) at step s -- the draws
 // of query key_u's walk t in the single-source path -- and likewise from v under (seed, key_v).
 #include <algorithm>
 
@@ -16,21 +15,13 @@ namespace {
 
 constexpr int kThreads = 256;
 
-// one step of a sqrt(c)-walk at node x (internal id): false when it stops there
-__device__ __forceinline__ bool walk_step(const int64_t *__restrict__ in_off, const int32_t *__restrict__ in_col,
-                                          int32_t &x, uint32_t t, uint32_t s, uint32_t seed, uint32_t key,
-                                          uint32_t t_stop) {
-    const U32x4 r = philox4x32_10(t, s, 0u, 0u, seed, key);
-    if (r.x < t_stop) return false;
-    const int64_t beg = in_off[x];
-    const uint32_t d = (uint32_t)(in_off[x + 1] - beg);
-    if (d == 0) return false;
-    x = in_col[beg + __umulhi(r.y, d)];
-    return true;
-}
-
-// grid.y = pair; meets[pair] += walk pairs t in [0, r) that meet
-__global__ void __launch_bounds__(kThreads) k_pair_mc(const int64_t *__restrict__ in_off, const int32_t *__restrict__ in_col,
+// grid.y = pair; meets[pair] += walk pairs t in [0, r) that meet.  A thread takes its next walk pair as soon as one ends
+// (both walks go on with probability c, so a pair takes 2.5 steps on average, the longest of a warp's 32 about 8): the
+// loop's body is one step of whatever pair the thread holds.  A step's draws come before its gathers, which only pairs
+// that go on make: the node records of both nodes, then one in-list entry each.
+// What bounds it: issue slots (68 % of the SM busy, two thirds of it Philox).  50 pairs of 2^20 walk pairs on R-MAT
+// 2^20: 1.51 ms with a loop over pairs around a loop over steps, 0.59 now (0.79 with 8 blocks per SM, 0.65 with 128).
+__global__ void __launch_bounds__(kThreads) k_pair_mc(const int4 *__restrict__ rec, const int32_t *__restrict__ in_col,
                                                       const int32_t *__restrict__ ext2int, const int32_t *__restrict__ pu,
                                                       const int32_t *__restrict__ pv, const uint32_t *__restrict__ ku,
                                                       const uint32_t *__restrict__ kv, int64_t r, int32_t l_max,
@@ -42,18 +33,41 @@ __global__ void __launch_bounds__(kThreads) k_pair_mc(const int64_t *__restrict_
     const int32_t pair = blockIdx.y;
     const int32_t u0 = ext2int[pu[pair]], v0 = ext2int[pv[pair]];
     const uint32_t keyu = ku[pair], keyv = kv[pair];
+    const int4 ru = rec[u0], rv = rec[v0];
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
     unsigned local = 0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < r; t += (int64_t)gridDim.x * blockDim.x) {
+    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (u0 == v0) {  // equal nodes meet at once
+        for (; t < r; t += step) ++local;
+    } else {
         int32_t a = u0, b = v0;
-        bool meet = a == b;
-        // positions 1, 2, ... exist while both walks continue; a walk holds at most l_max nodes
-        for (uint32_t s = 0; !meet && (int32_t)s + 1 < l_max; ++s) {
-            const bool ga = walk_step(in_off, in_col, a, (uint32_t)t, s, seed, keyu, t_stop);
-            const bool gb = walk_step(in_off, in_col, b, (uint32_t)t, s, seed, keyv, t_stop);
-            if (!ga || !gb) break;
-            meet = a == b;
+        int4 ra = ru, rb = rv;
+        uint32_t s = 0;
+        while (t < r) {
+            // positions 1, 2, ... exist while both walks continue; a walk holds at most l_max nodes
+            const U32x4 da = philox4x32_10((uint32_t)t, s, 0u, 0u, seed, keyu);
+            const U32x4 db = philox4x32_10((uint32_t)t, s, 0u, 0u, seed, keyv);
+            bool on = da.x >= t_stop && db.x >= t_stop && (int32_t)s + 1 < l_max;
+            if (on && s > 0) {
+                ra = __ldg(rec + a);
+                rb = __ldg(rec + b);
+            }
+            on = on && ra.y > 0 && rb.y > 0;
+            bool meet = false;
+            if (on) {
+                a = __ldg(in_col + ra.x + (int32_t)__umulhi(da.y, (uint32_t)ra.y));
+                b = __ldg(in_col + rb.x + (int32_t)__umulhi(db.y, (uint32_t)rb.y));
+                meet = a == b;
+                ++s;
+            }
+            if (!on || meet) {  // the next pair, from the start
+                local += meet;
+                t += step;
+                s = 0;
+                ra = ru;
+                rb = rv;
+            }
         }
-        local += meet;
     }
     for (int o = 16; o; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
     if ((threadIdx.x & 31) == 0 && local) atomicAdd(&s_cnt, local);
@@ -70,10 +84,10 @@ void launch_pair_mc(const DeviceGraph &g, const int32_t *pu, const int32_t *pv, 
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int64_t bx = (r + kThreads - 1) / kThreads;  // blocks per pair: about 8 per SM over all pairs
-    bx = std::min<int64_t>(bx, std::max<int64_t>(1, (int64_t)sms * 8 / npairs));
+    int64_t bx = (r + kThreads - 1) / kThreads;  // blocks per pair: about 32 per SM over all pairs
+    bx = std::min<int64_t>(bx, std::max<int64_t>(1, (int64_t)sms * 32 / npairs));
     dim3 grid((unsigned)bx, (unsigned)npairs);
-    k_pair_mc<<<grid, kThreads, 0, s>>>(g.in_off, g.in_col, g.ext2int, pu, pv, ku, kv, r, l_max, seed, t_stop, meets);
+    k_pair_mc<<<grid, kThreads, 0, s>>>(g.rec, g.in_col, g.ext2int, pu, pv, ku, kv, r, l_max, seed, t_stop, meets);
 }
 
 }  // namespace ps
