@@ -198,20 +198,22 @@ __global__ void __launch_bounds__(256) k_inst_init(QueryBatch q, DeviceGraph g, 
 }
 
 constexpr int kLevelThreads = 256;
+constexpr int kLevelSteps = 4;        // steps of 32 items whose loads go out together
 constexpr int kLevelBuffer = 128;     // members a warp holds back before it appends them
 constexpr int kLevelMaxItems = 4096;  // work items a warp takes at a time, at most
 
 // One level.  A warp takes a run of consecutive work items (32 to kLevelMaxItems, so that a short level still spreads
-// over the chip).  It holds the first items of the next 32 entries in registers; every entry has at least one item, so
-// the entries of 32 items lie in that window and a lane finds its own by five shuffles.  Where one entry holds the next
-// 64 items or more (the rule at level 0, whose entries are hubs), its items run through a pipeline of four stages --
-// out-edge, record, draw, in-edge -- with a load of each in flight; else 32 items of several entries go at once.
+// over the chip) and holds a window of 32 entries, one per lane.  A step's entry starts form a 32-bit mask (one warp
+// reduction) whose set bits up to a lane count the entries to the lane's own; shuffles bring that entry's fields where
+// they are used.  kLevelSteps steps go together, stage by stage -- out-edges, records, draws, in-edges -- so a warp waits
+// for three gathers per 128 items, whether they belong to one hub or to a hundred short lists.
 // What bounds it: dependent random sectors (a record per item; an in-list entry for a fifth of them) at 32 warps per
-// SM, then the ten Philox rounds (a third of the time at level 0 goes when they are left out).
+// SM, then the ten Philox rounds (a third of the time at level 0 went when they were left out).
 // A top-k call of four queries at eps = 0.1 on R-MAT 2^20: 6.2 ms with hash sets (4.5 ms of level kernels, 0.55 ms of
-// clears, two synchronisations a level); 3.0 without them; 2.3 with the records, the pipeline, self-contained entries
-// (a level of 60 million items in 0.49 ms; 0.81 before) and appends gathered per warp.  64 mixed-eps queries with the
-// switch on R-MAT 2^22: 332 ms of level kernels with hash sets, 115 now.
+// clears, two synchronisations a level); 3.0 without them; 2.3 with the records, appends gathered per warp and an entry
+// load per 32 items; 1.8 with the window (its level 1, short lists: 0.55 -> 0.30 ms; level 0, 60 million items, 0.49 ->
+// 0.44).  64 mixed-eps queries with the switch on R-MAT 2^22: 332 ms of level kernels with hash sets, 72 now (the call
+// 97 ms; 109 at two steps, 101 at three, 114 at four with three blocks per SM).
 __global__ void __launch_bounds__(kLevelThreads, 4) k_rand_level(DeviceGraph g, const int32_t *__restrict__ walks,
                                                               int32_t l_max,
                                                               const uint32_t *__restrict__ qkey, uint32_t seed,
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(kLevelThreads, 4) k_rand_level(DeviceGraph g, 
     };
     const long long *first = L.cur.first;
     for (long long t0 = warp * run; t0 < E; t0 += nwarps * run) {
-        const long long t1 = min(E, t0 + run);
+        const int32_t n_items = (int32_t)(min(E, t0 + run) - t0);  // positions below count from t0
         // the entry of item t0: the last f with first[f] <= t0, by a 32-way search
         long long f = 0;
         for (long long span = F; span > 1;) {
@@ -267,86 +269,68 @@ __global__ void __launch_bounds__(kLevelThreads, 4) k_rand_level(DeviceGraph g, 
             f += k * step;
             span = min(step, span - k * step);
         }
-        long long win = f + 1 + lane < F ? first[f + 1 + lane] : E;  // first items of the entries after f
-        long long beg_f = first[f];
-        int32_t c_y = 0, c_ex = 0, c_b = 0, c_i = 0;  // the lane's entry
-        uint32_t c_k = 0, c_key = 0, c_id8 = 0;
-        long long c_f = -1, c_col = 0;
-        // stage 3 of an item: the draw; idx >= 0 asks for that in-list entry
-        auto draw = [&](int32_t x, int4 rec) -> int32_t {
-            const U32x4 d = philox4x32_10(c_k, (1u << 24) | ((uint32_t)c_i << 8) | (uint32_t)L.j, (uint32_t)rec.z, 0u,
-                                          seed, c_key);
-            // kept with probability sqrt(c); then the sampled in-edge (v, x) must have v = y
-            const bool may = x != c_ex && d.y < t_keep && rec_may_be(rec.w, d.x, c_id8);
-            return may ? rec.x + (int32_t)__umulhi(d.x, (uint32_t)rec.y) : -1;
-        };
-        // stage 4: members are counted at an instance's last level, else kept for the next level's list
-        auto settle = [&](int32_t x, int32_t idx, int32_t v) {
-            const bool member = idx >= 0 && v == c_y, last = c_i - 2 == L.j;
-            if (member && last) atomicAdd(L.counts + (int64_t)c_b * g.n + x, 1);  // in H_{i-1}: the result
-            const unsigned m = __ballot_sync(0xffffffffu, member && !last);
-            if (m) {
-                if (member && !last) buf[kept + __popc(m & ((1u << lane) - 1u))] = make_int2((int32_t)c_f, x);
-                kept += __popc(m);
-                if (kept > kLevelBuffer - 32) flush();
+        for (int32_t p = 0; p < n_items; f += 32) {
+            // the window: entry f + lane, its start (clamped to this run) and its out-list minus its start
+            RandEntry en = {};
+            int32_t start = 1 << 30;
+            uint32_t base = 0, key = 0;
+            if (f + lane < F) {
+                en = L.cur.ent[f + lane];
+                const long long rel = first[f + lane] - t0;
+                start = rel < 0 ? -1 : (int32_t)min(rel, (long long)(1 << 30));
+                base = en.out_beg - (uint32_t)rel;
+                key = qkey[en.q];
             }
-        };
-        for (long long t = t0; t < t1;) {
-            const long long next_first = __shfl_sync(0xffffffffu, win, 0);
-            int r = 0;  // entries of the window that start at or before the lane's item
-            if (next_first <= t + 31) {
-                const long long it = t + lane;
+            const uint32_t meta = ((uint32_t)en.len << 8) | en.id8;
+            const long long wend = (f + 32 < F ? first[f + 32] : E) - t0;
+            const int32_t lim = (int32_t)min((long long)n_items, wend);
+            int32_t before = __popc(__ballot_sync(0xffffffffu, start < p));  // window entries that start before p
+            while (p < lim) {
+                int32_t x[kLevelSteps], r[kLevelSteps], idx[kLevelSteps];
+                int4 rec[kLevelSteps];
 #pragma unroll
-                for (int s = 16; s; s >>= 1) {
-                    const long long v = __shfl_sync(0xffffffffu, win, r + s - 1);
-                    if (v <= it) r += s;
+                for (int u = 0; u < kLevelSteps; ++u) {
+                    const int32_t q = p + 32 * u;
+                    const uint32_t off = (uint32_t)(start - q);
+                    const unsigned starts = __reduce_or_sync(0xffffffffu, off < 32u && q < lim ? 1u << off : 0u);
+                    r[u] = (before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1) & 31;
+                    const uint32_t col = __shfl_sync(0xffffffffu, base, r[u]);
+                    x[u] = q + lane < lim ? __ldg(g.out_col + (uint32_t)(col + q + lane)) : -1;
+                    before += __popc(starts);
                 }
-            }
-            const long long start = __shfl_sync(0xffffffffu, win, r > 0 ? r - 1 : 0);
-            if (f + r != c_f) {
-                c_f = f + r;
-                if (c_f < F) {  // past the last entry only for lanes past the last item
-                    const RandEntry e = L.cur.ent[c_f];
-                    c_y = e.y;
-                    c_id8 = e.id8;
-                    c_i = e.len;
-                    c_b = e.q;
-                    c_k = e.k;
-                    c_key = qkey[e.q];
-                    c_ex = e.ex;
-                    c_col = (long long)e.out_beg - (r > 0 ? start : beg_f);
+#pragma unroll
+                for (int u = 0; u < kLevelSteps; ++u) rec[u] = __ldg(g.rec + max(x[u], 0));
+#pragma unroll
+                for (int u = 0; u < kLevelSteps; ++u) {  // the draws
+                    const uint32_t m = __shfl_sync(0xffffffffu, meta, r[u]);
+                    const uint32_t k = __shfl_sync(0xffffffffu, en.k, r[u]), ky = __shfl_sync(0xffffffffu, key, r[u]);
+                    const int32_t ex = __shfl_sync(0xffffffffu, en.ex, r[u]);
+                    const U32x4 d = philox4x32_10(k, (1u << 24) | (m & 0xFFFFFF00u) | (uint32_t)L.j, (uint32_t)rec[u].z,
+                                                  0u, seed, ky);
+                    // kept with probability sqrt(c); then the sampled in-edge (v, x) must have v = y
+                    const bool may = x[u] >= 0 && x[u] != ex && d.y < t_keep && rec_may_be(rec[u].w, d.x, m & 0xFFu);
+                    idx[u] = may ? rec[u].x + (int32_t)__umulhi(d.x, (uint32_t)rec[u].y) : -1;
                 }
-            }
-            const long long left = min(t1, next_first) - t;
-            if (left >= 64) {  // one entry: its items in a pipeline of four stages, a load of each in flight
-                const int32_t *col = g.out_col + c_col + t + lane;
-                const int32_t steps = (int32_t)(left >> 5);
-                int32_t x0 = __ldg(col), x1 = __ldg(col + 32), xp = 0, vp = 0, ip = -1;
-                int4 r0 = __ldg(g.rec + x0);
-                for (int32_t k = 0; k < steps; ++k) {
-                    const int32_t x2 = k + 2 < steps ? __ldg(col + 32 * (k + 2)) : x1;
-                    const int4 r1 = __ldg(g.rec + x1);
-                    const int32_t idx = draw(x0, r0);
-                    const int32_t v = __ldg(g.in_col + max(idx, 0));
-                    settle(xp, ip, vp);
-                    xp = x0, ip = idx, vp = v;
-                    x0 = x1, r0 = r1, x1 = x2;
+                int32_t v[kLevelSteps];
+#pragma unroll
+                for (int u = 0; u < kLevelSteps; ++u) v[u] = idx[u] >= 0 ? __ldg(g.in_col + idx[u]) : -1;
+#pragma unroll
+                for (int u = 0; u < kLevelSteps; ++u) {
+                    const int32_t y = __shfl_sync(0xffffffffu, en.y, r[u]);
+                    const bool member = v[u] == y && idx[u] >= 0;
+                    if (!__any_sync(0xffffffffu, member)) continue;
+                    // members are counted at an instance's last level, else kept for the next level's list
+                    const bool last = (int32_t)(__shfl_sync(0xffffffffu, meta, r[u]) >> 8) - 2 == L.j;
+                    if (member && last) atomicAdd(L.counts + (int64_t)L.cur.ent[f + r[u]].q * g.n + x[u], 1);
+                    const unsigned m = __ballot_sync(0xffffffffu, member && !last);
+                    if (m) {
+                        if (member && !last)
+                            buf[kept + __popc(m & ((1u << lane) - 1u))] = make_int2((int32_t)(f + r[u]), x[u]);
+                        kept += __popc(m);
+                        if (kept > kLevelBuffer - 32) flush();
+                    }
                 }
-                settle(xp, ip, vp);
-                t += 32ll * steps;
-            } else {
-                const bool live = t + lane < t1;
-                const int32_t x = live ? __ldg(g.out_col + c_col + t + lane) : c_ex;
-                const int32_t idx = live ? draw(x, __ldg(g.rec + x)) : -1;
-                settle(x, idx, __ldg(g.in_col + max(idx, 0)));
-                t += 32;
-            }
-            // the window moves past the entries that start by item t
-            const int adv = __popc(__ballot_sync(0xffffffffu, win <= t));
-            if (adv > 0 && t < t1) {
-                beg_f = __shfl_sync(0xffffffffu, win, adv - 1);
-                f += adv;
-                win = f + 1 + lane < F ? first[f + 1 + lane] : E;
+                p = min(lim, p + 32 * kLevelSteps);
             }
         }
     }
