@@ -677,8 +677,8 @@ def profile_case(args):
     frontier: R-MAT 2^20 drawn on the GPU, switch mode c0 = 0.01, two calls of four queries at eps = 0.1.
     billion:  R-MAT 2^25 with 10^9 edges drawn and built on the GPU, switch mode c0 = 0.01, one call of 64 top-50
               queries at eps = 0.1 (the billion-edge leg's call).
-    pull:     R-MAT 2^18 (the host generator, m = 2^22), deterministic PROBE with the full tiles pinned to single
-              32-column tiles at 8 blocks per SM (no tuner, so a capture does not depend on timings taken under a
+    pull:     R-MAT 2^18 (the host generator, m = 2^22), deterministic PROBE with the full tiles pinned to the
+              default shape at 8 blocks per SM (no tuner, so a capture does not depend on timings taken under a
               profiler), two queries at eps = 0.1 one per call."""
     import numpy as np
     import torch

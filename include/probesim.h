@@ -211,7 +211,8 @@ probesim_status probesim_autotune(probesim_graph *g, void *stream);
 /* The current choice: *wide_tile in {16, 32, 64, 96} (see probesim_set_tuning); blocks_per_sm[6] for tile widths
  * 1, 2, 4, 8, 16, 32. */
 probesim_status probesim_get_tuning(const probesim_graph *g, int32_t *wide_tile, int32_t *blocks_per_sm);
-/* Sets the launch shape by hand: wide_tile in {16, 32, 64, 96} (64: 32-column tiles two per pass; 96: 32-column
+/* Sets the launch shape by hand: wide_tile in {16, 32, 64, 96} (32: 32-column tiles, four or two of them taken as one
+ * 128- or 64-column tile where a depth has enough of them; 64: 32-column tiles two per pass; 96: 32-column
  * tiles whose rows the Tensor Memory Accelerator gathers into shared memory, E_UNSUPPORTED without a tensor-map
  * encoder in the driver); blocks_per_sm (may be null: keep the current ones) holds 8 entries in [1, 32], for tile
  * widths 1, 2, 4, 8, 16, 32, the pairs and the TMA launch (at most 3 fit).  Set it while no call runs on the graph

@@ -774,8 +774,13 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
                     PS_CUDA(cudaStreamWaitEvent(ss, ws->ev_ready, 0));
                 }
                 const int32_t c = 32 * nfull[d];
-                launch_pull(dgl, Bm + Lb.base(c), Lb.rpitch(c), 0, 1 << 30, A + La.base(c), La.rpitch(c), 0, 1 << 30, 1,
-                            tail[d], g->tune_bps[tail[d]], zmask_at(d) ? zmask_at(d) + nfull[d] : nullptr, ss);
+                const uint32_t *zm = zmask_at(d) ? zmask_at(d) + nfull[d] : nullptr;
+                if (dgl.n_pieces <= kNarrowPieces)
+                    launch_pull_narrow(dgl, Bm + Lb.base(c), Lb.rpitch(c), A + La.base(c), La.rpitch(c), tail[d],
+                                       g->tune_bps[tail[d]], zm, ss);
+                else
+                    launch_pull(dgl, Bm + Lb.base(c), Lb.rpitch(c), 0, 1 << 30, A + La.base(c), La.rpitch(c), 0, 1 << 30,
+                                1, tail[d], g->tune_bps[tail[d]], zm, ss);
                 ++launches;
             }
             if (nfull[d] > 0 && wide == kPullTma) {  // 32-column tiles, rows gathered by the TMA
@@ -784,10 +789,25 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
                                         g->tune_bps[kPullTma], zmask_at(d), d_pull_err, st));
                 ++launches;
             } else if (nfull[d] > 0) {  // 32-column tiles (or their 16-column halves, or pairs of them)
-                const int32_t nt = nfull[d] * (32 / tw);
-                launch_pull(dgl, Bm, Lb.rpitch(0), Lb.tile_stride(), Lb.tile_sub(tw), A, La.rpitch(0), La.tile_stride(),
-                            La.tile_sub(tw), nt, wide, g->tune_bps[wide], zmask_at(d), st);
-                ++launches;
+                // tiles of 128 or 64 columns first (see kPullWide), then what is left
+                const int32_t per = dg.n_active <= kPullWideRows ? 4 : 2;
+                int32_t nw = wide == 32 ? nfull[d] / per : 0;
+                if (dgl.n_pieces * nw * per / 4 < kPullWideWarps) nw = 0;
+                if (nw > 0) {
+                    launch_pull(dgl, Bm, Lb.rpitch(0), Lb.tile_stride(), Lb.tile_sub(32 * per), A, La.rpitch(0),
+                                La.tile_stride(), La.tile_sub(32 * per), nw, per == 4 ? kPullWide : kPullMid,
+                                g->tune_bps[32], zmask_at(d), st);
+                    ++launches;
+                }
+                // all of the launch's tiles, or up to three that lie in one group after the wide ones
+                const int32_t nt = (nfull[d] - per * nw) * (32 / tw), c0 = 32 * per * nw;
+                const int32_t one = 1 << 30;
+                if (nt > 0) {
+                    launch_pull(dgl, Bm + Lb.base(c0), Lb.rpitch(0), Lb.tile_stride(), nw > 0 ? one : Lb.tile_sub(tw),
+                                A + La.base(c0), La.rpitch(0), La.tile_stride(), nw > 0 ? one : La.tile_sub(tw), nt, wide,
+                                g->tune_bps[wide], zmask_at(d) ? zmask_at(d) + c0 / 32 : nullptr, st);
+                    ++launches;
+                }
             }
             if (ws->profiling) {
                 PS_CUDA(cudaEventRecord(e1, st));

@@ -13,6 +13,11 @@ namespace ps {
 // floats per lane per in-neighbour row; pieces are ordered longest first so the groups of a warp run
 // similar trip counts.  Column indices are loaded eight at a time and broadcast within the group, so
 // eight row gathers are in flight per lane.
+// What bounds it: the L1's data pipe (88 % of its wavefront peak at T = 128), then the instructions around the gathers.
+// At T = 128 (kPullWide) a warp owns one piece, so the piece's record, indices and loop serve 128 columns instead of 32:
+// two eps = 0.05 queries on R-MAT 2^18 39.0 -> 33.5 ms (64 columns: 35.3).  At T = 64 (kPullMid) the gathered rows of a
+// graph of a million nodes still mostly fit the L2: the headline query 20.4 -> 19.9 ms (128 columns: 20.0, with 9.1 GB
+// read from DRAM by the longest launch against 6.4).
 // ------------------------------------------------------------------------------------------------
 template <int VEC>
 struct VecT;
@@ -87,7 +92,7 @@ __device__ __forceinline__ void pull_gather(const int32_t (&mine)[PER], unsigned
 // T = tile width; NT = tiles per pass (2: the 32-column tiles 2y and 2y + 1 in one pass, so every in-list and piece
 // record is read once for both, with half the in-neighbours per chunk to keep the same gathers in flight)
 template <int T, int NT>
-__global__ void __launch_bounds__(256, (NT == 1 && (T == 32 || T <= 2)) ? 4 : 3) k_pull(const int32_t *__restrict__ piece_v, const int64_t *__restrict__ piece_beg,
+__global__ void __launch_bounds__(256, (NT == 1 && (T >= 32 || T <= 2)) ? 4 : 3) k_pull(const int32_t *__restrict__ piece_v, const int64_t *__restrict__ piece_beg,
                                               const int32_t *__restrict__ piece_len, int64_t n_pieces,
                                               const int32_t *__restrict__ in_col, const float *__restrict__ w,
                                               const float *__restrict__ D, int32_t dpitch, float *__restrict__ MD,
@@ -196,7 +201,7 @@ void launch_pull(const DeviceGraph &g, const float *D, int32_t dpitch, int64_t d
                  int32_t pitch, int64_t mts, int32_t msub, int32_t ntiles, int32_t tile, int32_t blocks_per_sm,
                  const uint32_t *zmask, cudaStream_t s) {
     if (ntiles <= 0) return;
-    const int T = tile == kPullPairs ? 32 : tile;
+    const int T = tile == kPullPairs ? 32 : (tile == kPullMid ? 64 : tile);
     const int NT = tile == kPullPairs ? 2 : 1;
     const int L = T >= 4 ? T / 4 : 1;
     const int64_t threads_needed = g.n_pieces * L;
@@ -212,6 +217,8 @@ void launch_pull(const DeviceGraph &g, const float *D, int32_t dpitch, int64_t d
         case 8: PS_PULL(8, 1); break;
         case 16: PS_PULL(16, 1); break;
         case kPullPairs: PS_PULL(32, 2); break;
+        case kPullWide: PS_PULL(128, 1); break;
+        case kPullMid: PS_PULL(64, 1); break;
         default: PS_PULL(32, 1); break;
     }
 #undef PS_PULL

@@ -340,8 +340,8 @@ class Graph:
         return {"wide_tile": wide.value, "blocks_per_sm": {1 << i: bps[i] for i in range(6)}}
 
     def set_tuning(self, wide_tile, blocks_per_sm=None):
-        """Sets the pull's launch shape by hand (probesim_set_tuning): wide_tile 16, 32, 64 (32-column tiles two per
-        pass) or 96 (32-column tiles gathered by the TMA); blocks_per_sm, if given, 8 values for tile widths 1..32,
+        """Sets the pull's launch shape by hand (probesim_set_tuning): wide_tile 16, 32 (the default: wider tiles
+        where a depth has enough), 64 (32-column tiles two per pass) or 96 (32-column tiles gathered by the TMA); blocks_per_sm, if given, 8 values for tile widths 1..32,
         the pairs and the TMA launch."""
         arr = None
         if blocks_per_sm is not None:
