@@ -65,19 +65,6 @@ __device__ __forceinline__ uint32_t mix32(uint32_t h) {
     return h ^ (h >> 16);
 }
 
-// tree slots of depth >= 2: the probes
-__global__ void k_fr_list(TrieTable t, int32_t *slot, int32_t *count) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool take = e < t.cap && t.key[e] != kEmptyKey && t.depth[e] >= 2;
-    const unsigned m = __ballot_sync(0xffffffffu, take);
-    if (!m) return;
-    const int lane = threadIdx.x & 31;
-    int32_t base = 0;
-    if (lane == 0) base = atomicAdd(count, __popc(m));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (take) slot[base + __popc(m & ((1u << lane) - 1u))] = (int32_t)e;
-}
-
 // Rule 2 keeps an entry of score val at level j of a probe of length q when val * sqrt(c)^(q-j-1) > eps_p
 __device__ __forceinline__ bool rule2_keeps(float val, const float *pw, float eps_p, int32_t q, int32_t j) {
     return eps_p <= 0.f || val * pw[q - j - 1] > eps_p;
@@ -674,9 +661,6 @@ cudaError_t launch_table(const DeviceGraph &g, const TrieTable &t, const Frontie
 
 }  // namespace
 
-void launch_fr_list(TrieTable t, int32_t *slot, int32_t *count, cudaStream_t s) {
-    k_fr_list<<<blocks_for(t.cap), kThreads, 0, s>>>(t, slot, count);
-}
 void launch_fr_init(TrieTable t, FrontierProbes P, const int64_t *out_off, const float *pw, float eps_p,
                     FrontierEntry *list, cudaStream_t s) {
     if (P.P > 0) k_fr_init<<<blocks_for(P.P), kThreads, 0, s>>>(t, P, out_off, pw, eps_p, list);

@@ -113,6 +113,8 @@ struct TrieTable {
     float *gamma = nullptr;    // normalised weight minus the excluded score (see probe_level.cu)
     float *G = nullptr;        // sum of the children's gamma
     int32_t *walk_slot = nullptr;  // optional [W][l_max]: slot of the prefix of length i of walk w at [w][i-1]
+    int32_t *probes = nullptr;     // optional: the slots of depth >= 2 and their count, about in walk order, so that the
+    int32_t *probe_count = nullptr;  // probes of one query stay together and its estimate row in the L2
 };
 
 constexpr unsigned long long kEmptyKey = 0xFFFFFFFFFFFFFFFFull;
@@ -315,7 +317,6 @@ struct FrontierLevel {
     float eps_p = 0.f;
     int32_t j = 0;
 };
-void launch_fr_list(TrieTable t, int32_t *slot, int32_t *count, cudaStream_t s);
 void launch_fr_init(TrieTable t, FrontierProbes P, const int64_t *out_off, const float *pw, float eps_p,
                     FrontierEntry *list, cudaStream_t s);
 // switches the probes of [p0, p1) whose next frontier is certain to exceed the limit (no Rule 2; segments in src)

@@ -1105,15 +1105,16 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
     PS_CUDA(cudaMemsetAsync(t.height, 0, 4 * cap, st));
     PS_CUDA(cudaMemsetAsync(t_sw, 0, cap, st));
     LaunchCounters *d_ctr = ws->ctr.as<LaunchCounters>();
-    launch_trie_insert(dg, qb, P.W, L, ws->walks.as<int32_t>(), ws->lens.as<int32_t>(), t, d_ctr, st);
     // the probes: tree nodes of depth >= 2
     PS_ALLOC(ws->f_slot.ensure(sizeof(int32_t) * std::max<int64_t>(1, walk_nodes)));
     PS_ALLOC(ws->f_misc.ensure(512));
     int32_t *d_np = ws->f_misc.as<int32_t>();
     unsigned long long *d_fctr = reinterpret_cast<unsigned long long *>(ws->f_misc.as<char>() + 8);
     PS_CUDA(cudaMemsetAsync(d_np, 0, 512, st));
-    launch_fr_list(t, ws->f_slot.as<int32_t>(), d_np, st);
-    launches += 2;
+    t.probes = ws->f_slot.as<int32_t>();
+    t.probe_count = d_np;
+    launch_trie_insert(dg, qb, P.W, L, ws->walks.as<int32_t>(), ws->lens.as<int32_t>(), t, d_ctr, st);
+    ++launches;
     LaunchCounters *h_ctr = ws->pin_s.as<LaunchCounters>();
     long long *h_ll = reinterpret_cast<long long *>(ws->pin_s.as<char>() + 32768);
     PS_CUDA(cudaMemcpyAsync(h_ctr, d_ctr, sizeof(LaunchCounters), cudaMemcpyDeviceToHost, st));

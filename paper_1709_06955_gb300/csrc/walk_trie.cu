@@ -121,8 +121,16 @@ __global__ void __launch_bounds__(256) k_trie_insert(QueryBatch q, int32_t W, in
         t.parent[s] = (int32_t)p;
         t.depth[s] = i;
         t.query[s] = b;
-        atomicAdd(&t.weight[s], 1);
+        const int32_t through = atomicAdd(&t.weight[s], 1);
         atomicMax(&t.height[s], len - i);
+        if (t.probes && through == 0 && i >= 2) {  // the first walk through a prefix lists it as a probe
+            const unsigned mask = __activemask();
+            const int lane = threadIdx.x & 31, leader = __ffs(mask) - 1;
+            int32_t base = 0;
+            if (lane == leader) base = atomicAdd(t.probe_count, __popc(mask));
+            base = __shfl_sync(mask, base, leader);
+            t.probes[base + __popc(mask & ((1u << lane) - 1u))] = (int32_t)s;
+        }
         p = s;
     }
 }
