@@ -119,7 +119,7 @@ struct Workspace {
     DevBuf counts, offs, node_list, col_export, sched;  // level schedule: exported column nodes, uploaded plan
     DevBuf md_a, md_b, out_stage;                       // the two score buffers; host-output staging
     DevBuf r_part, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
-    DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_vals, tk_qk;
+    DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_qk, tk_short;
     // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, deferral stack, tasks, global tables,
     // estimates
     DevBuf f_wslot, f_tsw, f_slot, f_misc, f_pr32, f_pr64, f_acc, f_tab, f_list[2], f_stack, f_tasks, f_keys;
@@ -151,7 +151,7 @@ struct Workspace {
                           &t_height, &t_slot, &t_gamma, &t_G, &counts, &offs, &node_list, &col_export,
                           &sched, &md_a, &md_b, &out_stage, &r_part, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
                           &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
-                          &tk_cid, &tk_cval, &tk_ids, &tk_vals, &tk_qk, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_pr32, &f_pr64, &f_acc,
+                          &tk_cid, &tk_cval, &tk_ids, &tk_qk, &tk_short, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_pr32, &f_pr64, &f_acc,
                           &f_tab, &f_list[0], &f_list[1], &f_stack, &f_tasks, &f_keys, &pm_in, &pm_meets, &pull_err};
         for (DevBuf *b : bufs) b->release();
         f_table_clean = false;

@@ -259,6 +259,12 @@ int topk_blocks_per_query(int32_t n);
 void launch_topk(int32_t n, int32_t B, const float *scores, const int32_t *qnode, const int32_t *qk, int32_t kmax,
                  TopkScratch sc, int32_t *ids, float *vals, cudaStream_t s, int64_t *launches);
 cudaError_t topk_preload();
+// the same through a short candidate list, for kmax <= kShortMaxK (topk.cu); *over (device) != 0 afterwards when a
+// query's candidates did not fit: the batch's results are then not all written
+constexpr int kShortCap = 4096, kShortMaxK = 1024;
+size_t topk_short_bytes(int32_t n, int32_t B);
+void launch_topk_short(int32_t n, int32_t B, const float *scores, const int32_t *qnode, const int32_t *qk, int32_t kmax,
+                       void *scratch, int32_t *ids, float *vals, int32_t *over, cudaStream_t s, int64_t *launches);
 
 // frontier PROBE engine (frontier.cu): each walk prefix probed on its own, with Pruning Rule 2 and the switch
 constexpr int kFixShift = 44;  // scores and estimates accumulate as int64 multiples of 2^-44

@@ -1787,37 +1787,64 @@ probesim_status ps::topk_core(probesim_graph *g, Workspace *ws, const std::share
     PS_CUDA(ws->tk_cid.ensure(sizeof(int32_t) * (size_t)kmax * chunk));
     PS_CUDA(ws->tk_cval.ensure(sizeof(float) * (size_t)kmax * chunk));
     PS_CUDA(ws->tk_qk.ensure(sizeof(int32_t) * 2 * chunk));
+    // the short way's candidate lists are as large as 8,192 scores a query: within the scores' share of the budget only
+    const bool use_short = kmax <= kShortMaxK && topk_short_bytes(n, chunk) <= budget_of(g, ws) / 8;
+    if (use_short) PS_CUDA(ws->tk_short.ensure(topk_short_bytes(n, chunk)));
     const bool dev_ids = is_device_ptr(ids), dev_vals = is_device_ptr(vals);
-    if (!dev_ids) PS_CUDA(ws->tk_ids.ensure(sizeof(int32_t) * (size_t)kmax * chunk));
-    if (!dev_vals) PS_CUDA(ws->tk_vals.ensure(sizeof(float) * (size_t)kmax * chunk));
-    std::vector<int32_t> hq(2 * chunk);
+    // the lists of a chunk on the device: ids, scores, then the flag of the short way.  Short lists for host memory come
+    // back in one copy through pinned memory (each pageable copy waits for the device, about 10 us)
+    const size_t list = (size_t)kmax * chunk;
+    const bool pinned = list <= ((size_t)1 << 20);
+    const size_t pin_bytes = sizeof(int32_t) * std::max(pinned ? 2 * list + 1 : (size_t)1, 2 * (size_t)chunk);
+    PS_CUDA(ws->tk_ids.ensure(sizeof(int32_t) * (2 * list + 1)));
     for (int32_t done = 0; done < nq; done += chunk) {
         const int32_t B = std::min(chunk, nq - done);
         PS_TRY(run_queries(g, ws, q + done, B, ws->out_stage.as<float>(), st));
+        PS_CUDA(ws->pin_q.ensure(pin_bytes));
+        int32_t *h = ws->pin_q.as<int32_t>();
         for (int32_t b = 0; b < B; ++b) {
-            hq[b] = q[done + b].node;
-            hq[chunk + b] = q[done + b].k;
+            h[b] = q[done + b].node;
+            h[B + b] = q[done + b].k;
         }
-        int32_t *d_qn = ws->tk_qk.as<int32_t>(), *d_qk = d_qn + chunk;
-        PS_CUDA(cudaMemcpyAsync(d_qn, hq.data(), sizeof(int32_t) * B, cudaMemcpyHostToDevice, st));
-        PS_CUDA(cudaMemcpyAsync(d_qk, hq.data() + chunk, sizeof(int32_t) * B, cudaMemcpyHostToDevice, st));
+        int32_t *d_qn = ws->tk_qk.as<int32_t>(), *d_qk = d_qn + B;
+        PS_CUDA(cudaMemcpyAsync(d_qn, h, sizeof(int32_t) * 2 * B, cudaMemcpyHostToDevice, st));
         TopkScratch sc;
         sc.hist = ws->tk_hist.as<unsigned>();
         sc.state = ws->tk_state.as<unsigned>();
         sc.tiecnt = ws->tk_tie.as<unsigned>();
         sc.cand_id = ws->tk_cid.as<int32_t>();
         sc.cand_val = ws->tk_cval.as<float>();
-        int32_t *oi = dev_ids ? ids + (int64_t)done * kmax : ws->tk_ids.as<int32_t>();
-        float *ov = dev_vals ? vals + (int64_t)done * kmax : ws->tk_vals.as<float>();
-        launch_topk(n, B, ws->out_stage.as<float>(), d_qn, d_qk, kmax, sc, oi, ov, st, &ws->stats.kernel_launches);
-        PS_CUDA(cudaGetLastError());
-        if (!dev_ids)
-            PS_CUDA(cudaMemcpyAsync(ids + (int64_t)done * kmax, oi, sizeof(int32_t) * (size_t)B * kmax,
-                                    cudaMemcpyDeviceToHost, st));
-        if (!dev_vals)
-            PS_CUDA(cudaMemcpyAsync(vals + (int64_t)done * kmax, ov, sizeof(float) * (size_t)B * kmax,
-                                    cudaMemcpyDeviceToHost, st));
-        PS_CUDA(cudaStreamSynchronize(st));
+        const size_t LB = (size_t)B * kmax;
+        int32_t *stage = ws->tk_ids.as<int32_t>(), *d_over = stage + 2 * LB;
+        int32_t *oi = dev_ids ? ids + (int64_t)done * kmax : stage;
+        float *ov = dev_vals ? vals + (int64_t)done * kmax : reinterpret_cast<float *>(stage + LB);
+        // brings what belongs in host memory back, and the short way's flag
+        auto finish = [&](bool flag) -> probesim_status {
+            PS_CUDA(cudaGetLastError());
+            const size_t from = !pinned ? 2 * LB : (!dev_ids ? 0 : (!dev_vals ? LB : 2 * LB)), to = 2 * LB + (flag ? 1 : 0);
+            int32_t *hp = h + (pinned ? from : 0);
+            if (to > from)
+                PS_CUDA(cudaMemcpyAsync(hp, stage + from, sizeof(int32_t) * (to - from), cudaMemcpyDeviceToHost, st));
+            if (!pinned && !dev_ids)
+                PS_CUDA(cudaMemcpyAsync(ids + (int64_t)done * kmax, oi, sizeof(int32_t) * LB, cudaMemcpyDeviceToHost, st));
+            if (!pinned && !dev_vals)
+                PS_CUDA(cudaMemcpyAsync(vals + (int64_t)done * kmax, ov, sizeof(float) * LB, cudaMemcpyDeviceToHost, st));
+            PS_CUDA(cudaStreamSynchronize(st));
+            if (pinned && !dev_ids) std::memcpy(ids + (int64_t)done * kmax, h, sizeof(int32_t) * LB);
+            if (pinned && !dev_vals) std::memcpy(vals + (int64_t)done * kmax, h + LB, sizeof(float) * LB);
+            return PROBESIM_OK;
+        };
+        bool full = !use_short;
+        if (use_short) {
+            launch_topk_short(n, B, ws->out_stage.as<float>(), d_qn, d_qk, kmax, ws->tk_short.p, oi, ov, d_over, st,
+                              &ws->stats.kernel_launches);
+            PS_TRY(finish(true));
+            full = h[pinned ? 2 * LB : 0] != 0;
+        }
+        if (full) {
+            launch_topk(n, B, ws->out_stage.as<float>(), d_qn, d_qk, kmax, sc, oi, ov, st, &ws->stats.kernel_launches);
+            PS_TRY(finish(false));
+        }
     }
     return PROBESIM_OK;
 }
