@@ -20,6 +20,11 @@ struct DevBuf {
     void *p = nullptr;
     size_t cap = 0;
     bool pooled = false;  // from the stream-ordered pool (cudaMallocAsync): freed with cudaFreeAsync
+    bool view = false;    // a part of another buffer: nothing to free
+    void set_view(void *q, size_t bytes) {
+        release();
+        p = q, cap = bytes, view = true;
+    }
     // allocates exactly `bytes` from the device's stream-ordered pool on stream s (no device-wide synchronisation,
     // unlike cudaMalloc / cudaFree); for buffers that are written once, such as a new version of the graph store
     cudaError_t alloc_pooled(size_t bytes, cudaStream_t s) {
@@ -34,12 +39,13 @@ struct DevBuf {
         pooled = true;
         return cudaSuccess;
     }
-    cudaError_t ensure(size_t bytes) {
+    cudaError_t ensure(size_t bytes) { return bytes <= cap && p ? cudaSuccess : ensure_exact(bytes + bytes / 8); }
+    cudaError_t ensure_exact(size_t bytes) {
         if (bytes <= cap && p) return cudaSuccess;
         if (p) cudaFree(p);
         p = nullptr;
         cap = 0;
-        const size_t nb = std::max<size_t>(256, bytes + bytes / 8);
+        const size_t nb = std::max<size_t>(256, bytes);
         cudaError_t e = cudaMalloc(&p, nb);
         if (e == cudaSuccess) cap = nb; else cudaGetLastError();
         return e;
@@ -64,13 +70,13 @@ struct DevBuf {
     // A pooled buffer returns to the pool on the calling thread's default stream, without waiting: its readers
     // have synchronised their own streams before they let go of it.
     void release() {
-        if (p) {
+        if (p && !view) {
             if (pooled) cudaFreeAsync(p, cudaStreamPerThread);
             else cudaFree(p);
         }
         p = nullptr;
         cap = 0;
-        pooled = false;
+        pooled = view = false;
     }
     template <class T>
     T *as() const { return static_cast<T *>(p); }
@@ -102,12 +108,13 @@ struct PinnedBuf {
 // version beside it and publishes it, so queries never wait for updates nor updates for queries, and a version's
 // device memory is freed when its last reader lets go.
 struct StoreVersion {
+    DevBuf arena;  // the first version: one allocation that the arrays below are parts of
     DevBuf in_off, in_col, out_off, out_col, w, rec, piece_v, piece_beg, piece_len, split_v;
     std::shared_ptr<StoreVersion> base;  // set when this version reuses base's arrays (an update that changed nothing)
     ps::DeviceGraph dg;
     uint64_t epoch = 0;
     ~StoreVersion() {
-        for (DevBuf *b : {&in_off, &in_col, &out_off, &out_col, &w, &rec, &piece_v, &piece_beg, &piece_len, &split_v})
+        for (DevBuf *b : {&in_off, &in_col, &out_off, &out_col, &w, &rec, &piece_v, &piece_beg, &piece_len, &split_v, &arena})
             b->release();
     }
 };
@@ -184,9 +191,8 @@ struct probesim_graph {
         std::lock_guard<std::mutex> lk(store_ptr_mu);
         store.swap(v);  // the old version is released outside the lock, by whichever reader holds it last
     }
-    std::vector<int32_t> h_ext2int;  // host copy of the id map (update batches are sorted by internal ids)
     // update scratch
-    DevBuf u_batch, u_valid, u_vpre, u_delta, u_deg, u_part, u_hist, u_bounds;
+    DevBuf u_batch, u_valid, u_vpre, u_delta, u_deg, u_part, u_hist, u_bounds, u_raw, u_keys[3], u_sort;
     uint64_t epoch = 0;
     Workspace ws0;
     std::atomic<size_t> budget{0};  // device memory one call's working buffers may take (set while calls run)

@@ -2,14 +2,16 @@
 // for the sqrt(c)-walks and PROBE's weights, out-lists O(x) for the probes' pushes).  A graph of 10^9 edges is
 // sorted and laid out on the GPU in about a second, where a host sort takes minutes.
 //
-//   1. a key per edge, (destination << bs) | source in the caller's ids; a loop gets the key n << bs, which sorts
-//      after every edge; an id outside [0, n) raises a flag the host reads
+//   1. a key per edge, (destination << bs) | source in the caller's ids; a loop gets the key of all ones (2 bs
+//      bits), which no edge has; an id outside [0, n) raises a flag the host reads
 //   2. an LSD radix sort of the keys (below)
 //   3. repeats and loops dropped: a flag per key, its prefix sums, a compaction
 //   4. the caller-id in-list offsets (run boundaries of the sorted keys) and out-degrees; the renumbering by
-//      descending out-degree, ties by caller id, as a radix sort of n keys ((m - outdeg) << bs | id)
+//      descending out-degree, ties by caller id, as a radix sort of n keys ((m - outdeg) << bs | id), by the upper half alone: the
+//      keys start in id order and the sort is stable
 //   5. the in-lists per internal row in the caller's source order (each row's run of sorted keys mapped through
-//      ext2int), and the out-lists from a radix sort of (source << bs | destination) in internal ids
+//      ext2int), and the out-lists from a radix sort of (source << bs | destination) in internal ids, by the source alone: the
+//      keys start in destination order
 // w and the pull pieces then come from the kernels the update path uses.
 //
 // Radix sort: 8-bit digits, least significant first, tiles of 4096 keys.  Per digit pass, one kernel counts
@@ -33,24 +35,36 @@ static_assert(kRadixThreads == kRadix, "the digit scans use one thread per digit
 
 int64_t radix_tiles(int64_t count) { return (count + kRadixTile - 1) / kRadixTile; }
 
+// Each warp counts into its own table; its lanes that share the first lane's digit add once, which takes the load off
+// the one counter of a skewed digit.  (11 million keys: 55 to 78 us a pass with a match over the warp's 32 digits, 15 to 25 now.)
 __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint64_t *__restrict__ keys, int64_t count,
                                                               int shift, long long *__restrict__ counts,
                                                               int64_t ntiles) {
-    __shared__ unsigned int h[kRadix];
-    h[threadIdx.x] = 0;
+    __shared__ unsigned int h[kRadixWarps][kRadix];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int w = 0; w < kRadixWarps; ++w) h[w][threadIdx.x] = 0;
     __syncthreads();
-    const int lane = threadIdx.x & 31;
     const int64_t base = blockIdx.x * (int64_t)kRadixTile;
-#pragma unroll 4
-    for (int r = 0; r < kRadixKPT; ++r) {
-        const int64_t i = base + (int64_t)r * kRadixThreads + threadIdx.x;
-        const uint32_t d = i < count ? (uint32_t)(keys[i] >> shift) & (kRadix - 1) : kRadix;
-        // lanes with the same digit add once (skewed digits would otherwise serialise on one counter)
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        if (d < kRadix && (peers >> lane) == 1u) atomicAdd(&h[d], (unsigned)__popc(peers));
+#pragma unroll
+    for (int r0 = 0; r0 < kRadixKPT; r0 += 8) {
+        uint32_t d[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int64_t i = base + (int64_t)(r0 + r) * kRadixThreads + threadIdx.x;
+            d[r] = i < count ? (uint32_t)(keys[i] >> shift) & (kRadix - 1) : kRadix;
+        }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const uint32_t first = __shfl_sync(0xffffffffu, d[r], 0);
+            const unsigned same = __ballot_sync(0xffffffffu, d[r] == first);
+            if (d[r] < kRadix && (d[r] != first || lane == 0))
+                atomicAdd(&h[warp][d[r]], d[r] == first ? (unsigned)__popc(same) : 1u);
+        }
     }
     __syncthreads();
-    counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    unsigned sum = 0;
+    for (int w = 0; w < kRadixWarps; ++w) sum += h[w][threadIdx.x];
+    counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = sum;
 }
 
 // exclusive prefix sum of one value per thread over a block of kRadixThreads threads
@@ -129,12 +143,12 @@ __global__ void __launch_bounds__(kRadixThreads, 3) k_radix_scatter(const uint64
     }
 }
 
-uint64_t *radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t count, int bits, long long *counts,
+uint64_t *radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t count, int lo, int bits, long long *counts,
                          long long *offsets, long long *partial, cudaStream_t s) {
     if (count <= 1) return keys;
     const int64_t nt = radix_tiles(count);
     uint64_t *a = keys, *b = tmp;
-    for (int shift = 0; shift < bits; shift += 8) {
+    for (int shift = lo; shift < bits; shift += 8) {
         k_radix_hist<<<(unsigned)nt, kRadixThreads, 0, s>>>(a, count, shift, counts, nt);
         launch_scan64(counts, (int64_t)kRadix * nt, partial, offsets, s);
         k_radix_scatter<<<(unsigned)nt, kRadixThreads, 0, s>>>(a, b, count, shift, offsets, nt);
@@ -152,7 +166,7 @@ static unsigned build_blocks(int64_t work, int threads) {
 
 __global__ void k_build_keys(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, int64_t m, int32_t n,
                              int bs, uint64_t *__restrict__ keys, int32_t *bad) {
-    const uint64_t loop_key = (uint64_t)(uint32_t)n << bs;
+    const uint64_t loop_key = ((uint64_t)1 << 2 * bs) - 1;  // only a loop has both halves all ones
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t s = src[i], d = dst[i];
         if ((uint32_t)s >= (uint32_t)n || (uint32_t)d >= (uint32_t)n) {
@@ -245,6 +259,55 @@ __global__ void k_build_out_col(const uint64_t *__restrict__ okeys, int64_t mu, 
                                 int32_t *__restrict__ out_col) {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < mu; e += (int64_t)gridDim.x * blockDim.x)
         out_col[e] = (int32_t)(okeys[e] & smask);
+}
+
+// ------------------------------------------------------------------------------------------------
+// update batches: the batch's edges in the two row orders (keys as above, in-lists by (internal destination, caller's
+// source); a loop gets 1 << 2 bs)
+// ------------------------------------------------------------------------------------------------
+__global__ void k_batch_keys(const int32_t *__restrict__ src, const int32_t *__restrict__ dst, int64_t k, int32_t n,
+                             int bs, const int32_t *__restrict__ ext2int, uint64_t *__restrict__ keys, int32_t *bad) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= k) return;
+    const int32_t s = src[i], d = dst[i];
+    uint64_t key = (uint64_t)1 << 2 * bs;
+    if ((uint32_t)s >= (uint32_t)n || (uint32_t)d >= (uint32_t)n) atomicOr(bad, 1);
+    else if (s != d) key = ((uint64_t)(uint32_t)ext2int[d] << bs) | (uint32_t)s;
+    keys[i] = key;
+}
+
+__global__ void k_batch_in(const uint64_t *__restrict__ ukeys, int64_t k, int bs, const int32_t *__restrict__ ext2int,
+                           int32_t *__restrict__ in_dst, int32_t *__restrict__ in_src, int32_t *__restrict__ in_src_ext,
+                           uint64_t *__restrict__ okeys) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= k) return;
+    const int32_t d = (int32_t)(ukeys[i] >> bs), s = (int32_t)(ukeys[i] & (((uint64_t)1 << bs) - 1));
+    const int32_t x = ext2int[s];
+    in_dst[i] = d;
+    in_src[i] = x;
+    in_src_ext[i] = s;
+    okeys[i] = ((uint64_t)(uint32_t)x << bs) | (uint32_t)d;
+}
+
+__global__ void k_batch_out(const uint64_t *__restrict__ okeys, int64_t k, int bs, int32_t *__restrict__ out_src,
+                            int32_t *__restrict__ out_dst) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= k) return;
+    out_src[i] = (int32_t)(okeys[i] >> bs);
+    out_dst[i] = (int32_t)(okeys[i] & (((uint64_t)1 << bs) - 1));
+}
+
+void launch_batch_keys(const int32_t *src, const int32_t *dst, int64_t k, int32_t n, int bs, const int32_t *ext2int,
+                       uint64_t *keys, int32_t *bad, cudaStream_t s) {
+    if (k > 0) k_batch_keys<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(src, dst, k, n, bs, ext2int, keys, bad);
+}
+void launch_batch_in(const uint64_t *ukeys, int64_t k, int bs, const int32_t *ext2int, int32_t *in_dst, int32_t *in_src,
+                     int32_t *in_src_ext, uint64_t *okeys, cudaStream_t s) {
+    if (k > 0)
+        k_batch_in<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(ukeys, k, bs, ext2int, in_dst, in_src, in_src_ext, okeys);
+}
+void launch_batch_out(const uint64_t *okeys, int64_t k, int bs, int32_t *out_src, int32_t *out_dst, cudaStream_t s) {
+    if (k > 0) k_batch_out<<<(unsigned)((k + 255) / 256), 256, 0, s>>>(okeys, k, bs, out_src, out_dst);
 }
 
 __global__ void k_active_rows(const int64_t *__restrict__ out_off, int32_t n, int32_t *res) {

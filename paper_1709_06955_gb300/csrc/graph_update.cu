@@ -95,7 +95,7 @@ __global__ void k_upd_bounds(int64_t k, const int32_t *__restrict__ rows, const 
 // valid batch entries before an entry are counted with a binary search in the row's batch range and the prefix sums of
 // the validity flags.  Keys compare in the row's order: the caller's source id for in-lists, the internal destination id
 // for out-lists.  What bounds it: reading and writing the list.  Two batches of 10,000 edges and a query on R-MAT 2^21
-// took 10.9 ms with a warp per row, which searched the batch for every row (1.4 ms a list); 5.6 ms now (0.08 to
+// took 10.9 ms with a warp per row, which searched the batch for every row (1.4 ms a list); 5.6 ms by tiles (0.08 to
 // 0.2 ms a list).  Rows of fewer than 32 entries in a row of touched ones are taken 32 entries at a time, each lane
 // finding its own: inserted edges of nodes that had none leave thousands of such rows side by side (1.6 ms a list
 // without that).

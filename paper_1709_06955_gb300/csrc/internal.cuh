@@ -421,10 +421,10 @@ void launch_i64_copy(const long long *a, int64_t *b, int64_t count, cudaStream_t
 
 // device-side initial build of the graph store (graph_build.cu)
 int64_t radix_tiles(int64_t count);
-// Stable LSD radix sort of count keys by their low `bits` bits (8 per pass); tmp holds count keys, counts
+// Stable LSD radix sort of count keys by their bits lo .. bits - 1 (8 per pass); tmp holds count keys, counts
 // 256 * radix_tiles(count) entries, offsets one more, partial scan64_partials_needed(that).  Returns the buffer
 // (keys or tmp) that holds the sorted keys.
-uint64_t *radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t count, int bits, long long *counts,
+uint64_t *radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t count, int lo, int bits, long long *counts,
                          long long *offsets, long long *partial, cudaStream_t s);
 void launch_build_keys(const int32_t *src, const int32_t *dst, int64_t m, int32_t n, int bs, uint64_t *keys,
                        int32_t *bad, cudaStream_t s);
@@ -443,6 +443,14 @@ void launch_build_in_col(int32_t n, const int32_t *int2ext, const long long *ext
                          const uint64_t *ukeys, uint32_t smask, const int32_t *ext2int, int bs, int32_t *in_col,
                          uint64_t *okeys, cudaStream_t s);
 void launch_build_out_col(const uint64_t *okeys, int64_t mu, uint32_t smask, int32_t *out_col, cudaStream_t s);
+// an update batch: keys (internal destination << bs | caller's source; 1 << 2 bs for loops; *bad set for an id outside
+// [0, n)); the arrays of the sorted distinct keys in in-list order and their (source << bs | destination) keys; those
+// keys, sorted, as the arrays in out-list order
+void launch_batch_keys(const int32_t *src, const int32_t *dst, int64_t k, int32_t n, int bs, const int32_t *ext2int,
+                       uint64_t *keys, int32_t *bad, cudaStream_t s);
+void launch_batch_in(const uint64_t *ukeys, int64_t k, int bs, const int32_t *ext2int, int32_t *in_dst, int32_t *in_src,
+                     int32_t *in_src_ext, uint64_t *okeys, cudaStream_t s);
+void launch_batch_out(const uint64_t *okeys, int64_t k, int bs, int32_t *out_src, int32_t *out_dst, cudaStream_t s);
 // *res = 1 + the largest v with out-edges (0 if none); *res must be 0 before the launch
 void launch_active_rows(const int64_t *out_off, int32_t n, int32_t *res, cudaStream_t s);
 

@@ -103,27 +103,39 @@ static bool is_device_ptr(const void *p) {
 // internal ids in ascending order; ext2int / int2ext map at the boundary.
 static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *d_src, const int32_t *d_dst, int64_t m,
                                    cudaStream_t st) {
-    struct Scratch {  // the build's temporaries, freed on every return
+    struct Scratch {  // the build's temporaries: parts of one allocation, freed on every return
+        DevBuf slab;
         DevBuf ka, kb, kc, cnt, off, part, ext_off, outdeg, rka, rkb, indeg_i, outdeg_i, hist, flag;
-        ~Scratch() {
-            for (DevBuf *b : {&ka, &kb, &kc, &cnt, &off, &part, &ext_off, &outdeg, &rka, &rkb, &indeg_i, &outdeg_i,
-                              &hist, &flag})
-                b->release();
-        }
+        ~Scratch() { slab.release(); }
     } t;
+    // parts of 256-byte multiples out of one allocation (an allocation and its release cost the host some 70 us)
+    auto carve = [](DevBuf &slab, const std::vector<std::pair<DevBuf *, size_t>> &parts) -> cudaError_t {
+        size_t total = 0;
+        for (auto &x : parts) total += (x.second + 255) / 256 * 256;
+        const cudaError_t e = slab.ensure_exact(total);
+        if (e != cudaSuccess) return e;
+        char *at = slab.as<char>();
+        for (auto &x : parts) {
+            x.first->set_view(at, x.second);
+            at += (x.second + 255) / 256 * 256;
+        }
+        return cudaSuccess;
+    };
     auto bitlen = [](uint64_t x) { int b = 0; while (x) { ++b; x >>= 1; } return b; };
     const int bs = std::max(1, bitlen((uint64_t)std::max(1, n - 1)));  // bits of a node id
     const uint32_t smask = (uint32_t)(((uint64_t)1 << bs) - 1);
-    const uint64_t end_key = (uint64_t)(uint32_t)n << bs;
+    const uint64_t end_key = ((uint64_t)1 << 2 * bs) - 1;
     const int64_t M = std::max<int64_t>(1, m);
     const int64_t big = std::max<int64_t>(M, n);
     const int64_t ntiles = radix_tiles(big);
-    PS_CUDA(t.ka.ensure(8 * (size_t)(M + 1)));
-    PS_CUDA(t.kb.ensure(8 * (size_t)(M + 1)));
-    PS_CUDA(t.cnt.ensure(8 * (size_t)(256 * ntiles)));
-    PS_CUDA(t.off.ensure(8 * (size_t)(256 * ntiles + 1)));
-    PS_CUDA(t.part.ensure(8 * (size_t)scan64_partials_needed(std::max<int64_t>(256 * ntiles, big + 1))));
-    PS_CUDA(t.flag.ensure(sizeof(int32_t)));
+    const int nb = 2 * (kPiece + 1);  // piece buckets: rows with out-edges, then the others, by length
+    const size_t n8 = 8 * (size_t)n;
+    PS_CUDA(carve(t.slab, {{&t.ka, 8 * (size_t)(M + 1)}, {&t.kb, 8 * (size_t)(M + 1)}, {&t.kc, 8 * (size_t)M},
+                           {&t.cnt, 8 * (size_t)(256 * ntiles)}, {&t.off, 8 * (size_t)(256 * ntiles + 1)},
+                           {&t.part, 8 * (size_t)scan64_partials_needed(std::max<int64_t>(256 * ntiles, big + 1))},
+                           {&t.flag, sizeof(int32_t)}, {&t.ext_off, n8 + 8}, {&t.outdeg, n8}, {&t.rka, n8}, {&t.rkb, n8},
+                           {&t.indeg_i, n8}, {&t.outdeg_i, n8},
+                           {&t.hist, sizeof(unsigned long long) * (2 * (size_t)nb + 2)}}));
     long long *cnt = t.cnt.as<long long>(), *off = t.off.as<long long>(), *part = t.part.as<long long>();
     // 1-3: sorted unique edge keys (dst << bs | src, caller's ids)
     PS_CUDA(cudaMemsetAsync(t.flag.p, 0, sizeof(int32_t), st));
@@ -132,7 +144,7 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     PS_CUDA(cudaMemcpyAsync(&bad, t.flag.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaStreamSynchronize(st));
     if (bad) return fail(PROBESIM_E_RANGE, "edge id outside [0, n)");
-    uint64_t *sorted = radix_sort_u64(t.ka.as<uint64_t>(), t.kb.as<uint64_t>(), m, bs + bitlen(n), cnt, off, part, st);
+    uint64_t *sorted = radix_sort_u64(t.ka.as<uint64_t>(), t.kb.as<uint64_t>(), m, 0, 2 * bs, cnt, off, part, st);
     long long *pre = reinterpret_cast<long long *>(sorted == t.ka.as<uint64_t>() ? t.kb.p : t.ka.p);
     launch_build_flags(sorted, m, end_key, pre, st);
     launch_scan64(pre, m, part, pre, st);  // in place: pre[m] = the number of distinct edges
@@ -140,16 +152,9 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     PS_CUDA(cudaMemcpyAsync(&mu_ll, pre + std::max<int64_t>(0, m), sizeof(long long), cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaStreamSynchronize(st));
     const int64_t mu = m > 0 ? (int64_t)mu_ll : 0;
-    PS_CUDA(t.kc.ensure(8 * (size_t)std::max<int64_t>(1, mu)));
     uint64_t *ukeys = t.kc.as<uint64_t>();
     launch_build_compact(sorted, m, end_key, pre, ukeys, st);
     // 4: in-list offsets and out-degrees by caller id, then the renumbering
-    PS_CUDA(t.ext_off.ensure(8 * ((size_t)n + 1)));
-    PS_CUDA(t.outdeg.ensure(8 * (size_t)n));
-    PS_CUDA(t.rka.ensure(8 * (size_t)n));
-    PS_CUDA(t.rkb.ensure(8 * (size_t)n));
-    PS_CUDA(t.indeg_i.ensure(8 * (size_t)n));
-    PS_CUDA(t.outdeg_i.ensure(8 * (size_t)n));
     long long *ext_off = t.ext_off.as<long long>();
     unsigned long long *outdeg = t.outdeg.as<unsigned long long>();
     PS_CUDA(cudaMemsetAsync(outdeg, 0, 8 * (size_t)n, st));
@@ -157,37 +162,32 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     launch_build_outdeg(ukeys, mu, smask, outdeg, st);
     launch_build_rank_keys(outdeg, n, mu, bs, t.rka.as<uint64_t>(), st);
     const uint64_t *rk =
-        radix_sort_u64(t.rka.as<uint64_t>(), t.rkb.as<uint64_t>(), n, bs + bitlen((uint64_t)mu), cnt, off, part, st);
+        radix_sort_u64(t.rka.as<uint64_t>(), t.rkb.as<uint64_t>(), n, bs, bs + bitlen((uint64_t)mu), cnt, off, part, st);
     PS_CUDA(g->ext2int.ensure(sizeof(int32_t) * n));
     PS_CUDA(g->int2ext.ensure(sizeof(int32_t) * n));
     launch_build_perm(rk, n, smask, ext_off, outdeg, g->int2ext.as<int32_t>(), g->ext2int.as<int32_t>(),
                       t.indeg_i.as<long long>(), t.outdeg_i.as<long long>(), st);
     // 5: the CSR arrays in internal ids
     auto sv = std::make_shared<StoreVersion>();
-    PS_CUDA(sv->in_off.ensure(sizeof(int64_t) * ((size_t)n + 1)));
-    PS_CUDA(sv->out_off.ensure(sizeof(int64_t) * ((size_t)n + 1)));
-    PS_CUDA(sv->in_col.ensure(sizeof(int32_t) * std::max<int64_t>(1, mu)));
-    PS_CUDA(sv->out_col.ensure(sizeof(int32_t) * std::max<int64_t>(1, mu)));
+    const int64_t cap_pieces = (int64_t)n + mu / kPiece + 1;
+    const size_t off_bytes = sizeof(int64_t) * ((size_t)n + 1), col_bytes = sizeof(int32_t) * std::max<int64_t>(1, mu);
+    PS_CUDA(carve(sv->arena, {{&sv->in_off, off_bytes}, {&sv->out_off, off_bytes}, {&sv->in_col, col_bytes},
+                              {&sv->out_col, col_bytes}, {&sv->w, sizeof(float) * (size_t)n},
+                              {&sv->rec, sizeof(int4) * (size_t)n}, {&sv->piece_v, sizeof(int32_t) * (size_t)cap_pieces},
+                              {&sv->piece_beg, sizeof(int64_t) * (size_t)cap_pieces},
+                              {&sv->piece_len, sizeof(int32_t) * (size_t)cap_pieces},
+                              {&sv->split_v, sizeof(int32_t) * (size_t)n}}));
     launch_scan64(t.indeg_i.as<long long>(), n, part, sv->in_off.as<long long>(), st);
     launch_scan64(t.outdeg_i.as<long long>(), n, part, sv->out_off.as<long long>(), st);
     uint64_t *okeys = t.ka.as<uint64_t>();  // the edge-key buffers are free again (the unique keys live in kc)
     launch_build_in_col(n, g->int2ext.as<int32_t>(), ext_off, sv->in_off.as<int64_t>(), ukeys, smask,
                         g->ext2int.as<int32_t>(), bs, sv->in_col.as<int32_t>(), okeys, st);
-    const uint64_t *osorted = radix_sort_u64(okeys, t.kb.as<uint64_t>(), mu, 2 * bs, cnt, off, part, st);
+    const uint64_t *osorted = radix_sort_u64(okeys, t.kb.as<uint64_t>(), mu, bs, 2 * bs, cnt, off, part, st);
     launch_build_out_col(osorted, mu, smask, sv->out_col.as<int32_t>(), st);
     // w and the pull pieces (in-lists cut into at most kPiece edges, longest first)
-    const int64_t cap_pieces = (int64_t)n + mu / kPiece + 1;
-    PS_CUDA(sv->w.ensure(sizeof(float) * n));
-    PS_CUDA(sv->rec.ensure(sizeof(int4) * n));
-    PS_CUDA(sv->piece_v.ensure(sizeof(int32_t) * cap_pieces));
-    PS_CUDA(sv->piece_beg.ensure(sizeof(int64_t) * cap_pieces));
-    PS_CUDA(sv->piece_len.ensure(sizeof(int32_t) * cap_pieces));
-    PS_CUDA(sv->split_v.ensure(sizeof(int32_t) * (size_t)n));
-    PS_CUDA(t.hist.ensure(sizeof(unsigned long long) * (4 * (kPiece + 1) + 2)));
     launch_upd_w(n, sv->in_off.as<long long>(), sv->in_col.as<int32_t>(), (float)std::sqrt(g->cfg.c),
                  g->int2ext.as<int32_t>(), rec_shift_for(n), sv->w.as<float>(), sv->rec.as<int4>(),
                  t.indeg_i.as<long long>(), st);
-    const int nb = 2 * (kPiece + 1);  // piece buckets: rows with out-edges, then the others, by length
     unsigned long long *hist = t.hist.as<unsigned long long>(), *cursor = hist + nb, *nsplit = cursor + nb;
     PS_CUDA(cudaMemsetAsync(t.flag.p, 0, sizeof(int32_t), st));
     launch_active_rows(sv->out_off.as<int64_t>(), n, t.flag.as<int32_t>(), st);
@@ -201,8 +201,6 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     PS_CUDA(cudaMemcpyAsync(hh.data() + nb, nsplit, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaMemcpyAsync(&ends[0], sv->in_off.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaMemcpyAsync(&ends[1], sv->out_off.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
-    g->h_ext2int.resize(n);
-    PS_CUDA(cudaMemcpyAsync(g->h_ext2int.data(), g->ext2int.p, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaGetLastError());
     PS_CUDA(cudaStreamSynchronize(st));
     if (ends[0] != mu || ends[1] != mu) return fail(PROBESIM_E_CUDA, "internal: the built lists disagree on m");
@@ -239,18 +237,6 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
 // Device memory one call on workspace ws may take (a server gives each worker a share of the graph's budget).
 static size_t budget_of(const probesim_graph *g, const Workspace *ws) {
     return ws->budget ? ws->budget : g->budget.load();
-}
-
-// Copies an int32 array that may live on the device to the host.
-static probesim_status fetch_ids(const int32_t *p, int64_t k, std::vector<int32_t> &out) {
-    out.resize(std::max<int64_t>(1, k));
-    if (k == 0) return PROBESIM_OK;
-    if (is_device_ptr(p)) {
-        PS_CUDA(cudaMemcpy(out.data(), p, sizeof(int32_t) * k, cudaMemcpyDeviceToHost));
-    } else {
-        std::memcpy(out.data(), p, sizeof(int32_t) * k);
-    }
-    return PROBESIM_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1517,7 +1503,8 @@ probesim_status probesim_graph_destroy(probesim_graph *g) {
     if (!g) return PROBESIM_OK;
     g->store.reset();
     DevBuf *bufs[] = {&g->ext2int, &g->int2ext, &g->u_batch, &g->u_valid,
-                      &g->u_vpre, &g->u_delta, &g->u_deg, &g->u_part, &g->u_hist, &g->u_bounds};
+                      &g->u_vpre, &g->u_delta, &g->u_deg, &g->u_part, &g->u_hist, &g->u_bounds,
+                      &g->u_raw, &g->u_keys[0], &g->u_keys[1], &g->u_keys[2], &g->u_sort};
     for (DevBuf *b : bufs) b->release();
     g->ws0.release();
     delete g;
@@ -1541,24 +1528,9 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     if (k < 0 || (k > 0 && (!src || !dst))) return fail(PROBESIM_E_INVALID, "bad update batch");
     std::lock_guard<std::mutex> lk(g->update_mu);
     g_last_error.clear();
-    std::vector<int32_t> hs, hd;
-    PS_TRY(fetch_ids(src, k, hs));
-    PS_TRY(fetch_ids(dst, k, hd));
     const int32_t n = g->n;
     const std::shared_ptr<StoreVersion> old = g->current();  // read only; queries may be reading it too
-    for (int64_t e = 0; e < k; ++e)
-        if (hs[e] < 0 || hs[e] >= n || hd[e] < 0 || hd[e] >= n) return fail(PROBESIM_E_RANGE, "edge id outside [0, n)");
-    // the batch without loops and repeats, in the two row orders
-    std::vector<uint64_t> in_keys, out_keys;
-    in_keys.reserve(k);
-    for (int64_t e = 0; e < k; ++e) {
-        if (hs[e] == hd[e]) continue;
-        in_keys.push_back(((uint64_t)(uint32_t)g->h_ext2int[hd[e]] << 32) | (uint32_t)hs[e]);  // (dst int, src ext)
-    }
-    std::sort(in_keys.begin(), in_keys.end());
-    in_keys.erase(std::unique(in_keys.begin(), in_keys.end()), in_keys.end());
-    const int64_t K = (int64_t)in_keys.size();
-    if (K == 0) {  // nothing changes but the epoch: the next version shares the current one's arrays
+    auto unchanged = [&]() -> probesim_status {  // nothing but the epoch: the next version shares the arrays
         auto nv = std::make_shared<StoreVersion>();
         nv->base = old;
         nv->dg = old->dg;
@@ -1566,36 +1538,58 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
         g->publish(nv);
         if (applied) *applied = 0;
         return PROBESIM_OK;
+    };
+    if (k == 0) return unchanged();
+    // the batch on the device, without loops and repeats, in the two row orders (sorted there: the host's two sorts of
+    // 10,000 edges took 0.7 ms of an update)
+    const int32_t *d_src = src, *d_dst = dst;
+    if (!is_device_ptr(src) || !is_device_ptr(dst)) {
+        PS_CUDA(g->u_raw.ensure(2 * sizeof(int32_t) * (size_t)k));
+        PS_CUDA(cudaMemcpyAsync(g->u_raw.p, src, sizeof(int32_t) * (size_t)k, cudaMemcpyDefault, st));
+        PS_CUDA(cudaMemcpyAsync(g->u_raw.as<int32_t>() + k, dst, sizeof(int32_t) * (size_t)k, cudaMemcpyDefault, st));
+        d_src = g->u_raw.as<int32_t>();
+        d_dst = d_src + k;
     }
-    out_keys.resize(K);
-    std::vector<int32_t> hb(5 * K);
-    int32_t *in_dst = hb.data(), *in_src = in_dst + K, *in_src_ext = in_src + K, *out_src = in_src_ext + K,
-            *out_dst = out_src + K;
-    for (int64_t e = 0; e < K; ++e) {
-        const int32_t d_int = (int32_t)(in_keys[e] >> 32), s_ext = (int32_t)(in_keys[e] & 0xffffffffu);
-        const int32_t s_int = g->h_ext2int[s_ext];
-        in_dst[e] = d_int;
-        in_src[e] = s_int;
-        in_src_ext[e] = s_ext;
-        out_keys[e] = ((uint64_t)(uint32_t)s_int << 32) | (uint32_t)d_int;
-    }
-    std::sort(out_keys.begin(), out_keys.end());
-    for (int64_t e = 0; e < K; ++e) {
-        out_src[e] = (int32_t)(out_keys[e] >> 32);
-        out_dst[e] = (int32_t)(out_keys[e] & 0xffffffffu);
-    }
+    int bs = 1;  // bits of a node id
+    while (((int64_t)(n - 1) >> bs) > 0) ++bs;
+    const int64_t ntiles = radix_tiles(k);
+    PS_CUDA(g->u_hist.ensure(sizeof(unsigned long long) * (4 * (kPiece + 1) + 2)));
+    for (DevBuf &b : g->u_keys) PS_CUDA(b.ensure(8 * (size_t)(k + 1)));
+    PS_CUDA(g->u_sort.ensure(8 * (size_t)(2 * 256 * ntiles + 1)));
+    PS_CUDA(g->u_part.ensure(sizeof(long long) * scan64_partials_needed(std::max<int64_t>({k, n, 256 * ntiles}))));
+    uint64_t *ka = g->u_keys[0].as<uint64_t>(), *kb = g->u_keys[1].as<uint64_t>(), *kc = g->u_keys[2].as<uint64_t>();
+    long long *cnt = g->u_sort.as<long long>(), *coff = cnt + 256 * ntiles, *part = g->u_part.as<long long>();
+    int32_t *d_bad = g->u_hist.as<int32_t>();
+    const int32_t *ext2int = g->ext2int.as<int32_t>();
+    const uint64_t end_key = (uint64_t)1 << 2 * bs;
+    PS_CUDA(cudaMemsetAsync(d_bad, 0, sizeof(int32_t), st));
+    launch_batch_keys(d_src, d_dst, k, n, bs, ext2int, ka, d_bad, st);
+    uint64_t *sorted = radix_sort_u64(ka, kb, k, 0, 2 * bs + 1, cnt, coff, part, st);
+    long long *pre = reinterpret_cast<long long *>(sorted == ka ? kb : ka);
+    launch_build_flags(sorted, k, end_key, pre, st);
+    launch_scan64(pre, k, part, pre, st);  // in place: pre[k] = the number of distinct edges
+    launch_build_compact(sorted, k, end_key, pre, kc, st);
+    long long hk = 0;
+    int32_t bad = 0;
+    PS_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    PS_CUDA(cudaMemcpyAsync(&hk, pre + k, sizeof(long long), cudaMemcpyDeviceToHost, st));
+    PS_CUDA(cudaGetLastError());
+    PS_CUDA(cudaStreamSynchronize(st));
+    if (bad) return fail(PROBESIM_E_RANGE, "edge id outside [0, n)");
+    const int64_t K = (int64_t)hk;
+    if (K == 0) return unchanged();
+    PS_CUDA(g->u_batch.ensure(sizeof(int32_t) * 5 * K));
+    int32_t *db = g->u_batch.as<int32_t>();
+    launch_batch_in(kc, K, bs, ext2int, db, db + K, db + 2 * K, ka, st);
+    const uint64_t *osorted = radix_sort_u64(ka, kb, K, bs, 2 * bs, cnt, coff, part, st);  // they start in destination order
+    launch_batch_out(osorted, K, bs, db + 3 * K, db + 4 * K, st);
     const DeviceGraph &dg = old->dg;
     auto nv = std::make_shared<StoreVersion>();  // the next version, built beside the current one
-    PS_CUDA(g->u_batch.ensure(sizeof(int32_t) * 5 * K));
     PS_CUDA(g->u_bounds.ensure(upd_bounds_bytes(K)));
     PS_CUDA(g->u_valid.ensure(sizeof(long long) * 2 * K));
     PS_CUDA(g->u_vpre.ensure(sizeof(long long) * 2 * (K + 1)));
     PS_CUDA(g->u_delta.ensure(sizeof(long long) * 2 * (size_t)n));
     PS_CUDA(g->u_deg.ensure(sizeof(long long) * 2 * ((size_t)n + 1)));
-    PS_CUDA(g->u_part.ensure(sizeof(long long) * scan64_partials_needed(std::max<int64_t>(K, n))));
-    PS_CUDA(g->u_hist.ensure(sizeof(unsigned long long) * (4 * (kPiece + 1) + 2)));
-    PS_CUDA(cudaMemcpyAsync(g->u_batch.p, hb.data(), sizeof(int32_t) * 5 * K, cudaMemcpyHostToDevice, st));
-    int32_t *db = g->u_batch.as<int32_t>();
     UpdateBatchArgs a;
     a.k = K;
     a.in_dst = db; a.in_src = db + K; a.in_src_ext = db + 2 * K; a.out_src = db + 3 * K; a.out_dst = db + 4 * K;
