@@ -180,6 +180,30 @@ inline int grid_for(int64_t work, int threads, int per_sm) {
     return (int)(blocks < 1 ? 1 : blocks);
 }
 
+// Launch whose blocks may be scheduled before the kernel ahead of it in the stream has finished; the kernel calls
+// pdl_wait() before it touches memory, which waits for that kernel, and so hides its own launch.  A depth of the level
+// loop is a chain of five to seven short kernels, with 2 to 3 us between two of them otherwise (one query on 1,000 nodes,
+// with the single stream of small graphs: 0.94 -> 0.74 ms; three on 30,000 nodes 2.46 -> 2.28).  What the kernel ahead
+// writes is read with plain loads: the read-only path (and a compiler that takes it as invariant) may look too early.
+__device__ __forceinline__ void pdl_wait() {
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+template <class... P, class... A>
+inline cudaError_t pdl_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Launchers (each launches one kernel on `s`).
 // ---------------------------------------------------------------------------------------------
@@ -192,13 +216,16 @@ void launch_sched_export(TrieTable t, int32_t *out, int32_t *count, cudaStream_t
 void launch_node_lists(TrieTable t, const int32_t *node_off, int32_t *ncur, int32_t *node_list, cudaStream_t s);
 void launch_set_slots(TrieTable t, const int32_t *pairs, int32_t count, cudaStream_t s);
 // scatters the gammas of the tree nodes two depths down into B, and zeroes B's spare row and A's split rows over the
-// pulled columns
+// pulled columns, and (zw > 0) columns [z0, z0 + zw) of A's rows below zrows
 void launch_prepare_pull(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *B, ColLayout Lb,
-                         float *A, ColLayout La, int32_t width, cudaStream_t s);
-// inherited = false: push nodes whose column is in the push block (slot >= h0); true: those whose column
-// was inherited from the parent (slot < h0)
+                         float *A, ColLayout La, int32_t width, int32_t zrows, int32_t z0, int32_t zw, cudaStream_t s);
+// which = 0: push nodes whose column is in the push block (slot >= h0); 1: those whose column was inherited from the
+// parent (slot < h0); 2: both
 void launch_push_h2(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *MD, ColLayout L,
-                    int32_t h0, bool inherited, cudaStream_t s);
+                    int32_t h0, int32_t which, cudaStream_t s);
+// Graphs of at most kSmallRows rows run a depth on one stream, with all its zeroing in the prepare launch and one push
+// launch: there the second stream's events cost more than it hides (see run_batch).
+constexpr int32_t kSmallRows = 1 << 16;
 // Parts of at most four sources: p1 (the first part of every group: bit 30 of the destination = set, else add)
 // then p2 (later parts: add).  Sources are -1 where absent.
 // W = the columns of a row of B that hold data (a multiple of 4), nsrc = the sources of all parts.

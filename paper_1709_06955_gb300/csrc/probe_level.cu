@@ -71,7 +71,9 @@ __device__ __forceinline__ bool is_push_node(const TrieTable &t, int32_t e) { re
 __global__ void __launch_bounds__(256) k_prepare_pull(const int32_t *__restrict__ nodes, int32_t cnt, int32_t blocks_sc,
                                                       TrieTable t, float *B, ColLayout Lb,
                                                       const int32_t *__restrict__ rows, int32_t nrows, float *A,
-                                                      ColLayout La, int32_t width) {
+                                                      ColLayout La, int32_t width, int32_t zrows, int32_t z0,
+                                                      int32_t zw) {
+    pdl_wait();
     if ((int32_t)blockIdx.x < blocks_sc) {
         const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
         if (i >= cnt) return;
@@ -90,21 +92,27 @@ __global__ void __launch_bounds__(256) k_prepare_pull(const int32_t *__restrict_
         if (r < nrows) A[La.at(rows[r], c)] = 0.f;
         else B[Lb.at(Lb.n, c)] = 0.f;
     }
+    const int64_t block = (int64_t)zrows * zw;
+    for (int64_t i = (int64_t)(blockIdx.x - blocks_sc) * blockDim.x + threadIdx.x; i < block; i += step) {
+        const int64_t r = i / zw;
+        A[La.at(r, z0 + (int32_t)(i - r * zw))] = 0.f;
+    }
 }
 
 // nodes: the tree nodes two depths down (cnt may be 0); width: the columns pulled
 void launch_prepare_pull(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *B, ColLayout Lb,
-                         float *A, ColLayout La, int32_t width, cudaStream_t s) {
+                         float *A, ColLayout La, int32_t width, int32_t zrows, int32_t z0, int32_t zw, cudaStream_t s) {
     const int bs = (std::max(0, cnt) + 255) / 256;
-    const int bz = grid_for(((int64_t)g.n_split + 1) * std::max(1, width), 256, 8);
-    k_prepare_pull<<<bs + bz, 256, 0, s>>>(nodes, cnt, bs, t, B, Lb, g.split_v, g.n_split, A, La, width);
+    const int bz = grid_for(std::max(((int64_t)g.n_split + 1) * std::max(1, width), (int64_t)zrows * zw), 256, 8);
+    pdl_launch(k_prepare_pull, dim3(bs + bz), dim3(256), 0, s, nodes, cnt, bs, t, B, Lb, g.split_v, g.n_split, A, La, width,
+               zrows, z0, zw);
 }
 
 // ------------------------------------------------------------------------------------------------
 // push: for every tree node g at depth t+2 whose grandparent p is a push node:
 // MD[x][slot(p)] += sqrt(c)/|I(x)| * gamma_g for every x in O(a_g).  A push node's column is either in the
-// push block of its depth (slot >= h0) or the column it inherited from its parent (slot < h0); one launch
-// serves one of the two kinds.  One block per node g: an out-list can hold tens of thousands of edges
+// push block of its depth (slot >= h0) or the column it inherited from its parent (slot < h0); a launch
+// serves one of the two kinds or both.  One block per node g: an out-list can hold tens of thousands of edges
 // (hubs), so the block's threads split it and a hub does not hold up the launch.
 // ------------------------------------------------------------------------------------------------
 // A block per node waits for its longest list: few nodes get larger blocks, so a hub's list takes fewer rounds.
@@ -115,12 +123,13 @@ static int list_threads(int32_t cnt) {
 
 __global__ void __launch_bounds__(512) k_push_h2(const int64_t *__restrict__ out_off, const int32_t *__restrict__ out_col,
                                                  const float *__restrict__ w, const int32_t *__restrict__ nodes,
-                                                 TrieTable t, float *MD, ColLayout L, int32_t h0, int32_t inherited,
+                                                 TrieTable t, float *MD, ColLayout L, int32_t h0, int32_t which,
                                                  int32_t rows) {
+    pdl_wait();
     const int32_t e = nodes[blockIdx.x];
     const int32_t p = t.parent[t.parent[e]];  // the height-2 node
     const int32_t sl = t.slot[p];
-    if (sl < 0 || !is_push_node(t, p) || (sl < h0) != (inherited != 0)) return;
+    if (sl < 0 || !is_push_node(t, p) || (which != 2 && (sl < h0) != (which == 1))) return;
     const int32_t a = t.node[e];
     const float g = t.gamma[e];
     const int64_t beg = out_off[a], end = out_off[a + 1];
@@ -143,10 +152,10 @@ __global__ void __launch_bounds__(512) k_push_h2(const int64_t *__restrict__ out
 }
 
 void launch_push_h2(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *MD, ColLayout L,
-                    int32_t h0, bool inherited, cudaStream_t s) {
+                    int32_t h0, int32_t which, cudaStream_t s) {
     if (cnt <= 0) return;
-    k_push_h2<<<(unsigned)cnt, list_threads(cnt), 0, s>>>(g.out_off, g.out_col, g.w, nodes, t, MD, L, h0,
-                                                          inherited ? 1 : 0, g.n_active);
+    pdl_launch(k_push_h2, dim3(cnt), dim3(list_threads(cnt)), 0, s, g.out_off, g.out_col, g.w, nodes, t, MD, L, h0, which,
+               g.n_active);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -168,6 +177,7 @@ constexpr int kAccRows = 4;
 template <bool LATER>
 __global__ void __launch_bounds__(256) k_accumulate(int32_t n, float *B, ColLayout L, const int32_t *__restrict__ pdst,
                                                     const int4 *__restrict__ psrc, int32_t np) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int32_t pi = blockIdx.y * 32 + lane;
     const bool on = pi < np;
@@ -232,6 +242,7 @@ __global__ void __launch_bounds__(kStageThreads) k_accumulate_rows(int32_t n, fl
                                                                    const int32_t *__restrict__ p2dst,
                                                                    const int4 *__restrict__ p2src, int32_t np2) {
     extern __shared__ __align__(16) float rows[];
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const uint32_t rows_s = (uint32_t)__cvta_generic_to_shared(rows);
     auto part = [&](const float *row, int4 sc) {
@@ -298,9 +309,8 @@ static cudaError_t accumulate_rows(int32_t n, float *B, const ColLayout &L, int3
                                                (int)bytes);
     if (e != cudaSuccess) return e;
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, kStageBytes / std::max<size_t>(1, bytes)));
-    k_accumulate_rows<R><<<grid_for(((int64_t)n + R - 1) / R, 1, per_sm), kStageThreads, bytes, s>>>(
-        n, B, L, W, p1dst, p1src, np1, p2dst, p2src, np2);
-    return cudaSuccess;
+    return pdl_launch(k_accumulate_rows<R>, dim3(grid_for(((int64_t)n + R - 1) / R, 1, per_sm)), dim3(kStageThreads), bytes,
+                      s, n, B, L, W, p1dst, p1src, np1, p2dst, p2src, np2);
 }
 
 // W: the columns of a row that hold data; nsrc: the sources of all parts.  In place, a row costs a sector per source and
@@ -323,9 +333,10 @@ cudaError_t launch_accumulate(int32_t n, float *B, ColLayout L, int32_t W, int64
         const int x = grid_for((int64_t)(n + kAccRows - 1) / kAccRows * 32, 256, 8);
         return dim3((unsigned)std::max(1, std::min(x, 8 * 152 / y + 1)), (unsigned)y);
     };
-    k_accumulate<false><<<grid(np1), 256, 0, s>>>(n, B, L, p1dst, p1src, np1);
-    if (np2 > 0) k_accumulate<true><<<grid(np2), 256, 0, s>>>(n, B, L, p2dst, p2src, np2);
-    return cudaSuccess;
+    cudaError_t e = pdl_launch(k_accumulate<false>, grid(np1), dim3(256), 0, s, n, B, L, p1dst, p1src, np1);
+    if (e == cudaSuccess && np2 > 0)
+        e = pdl_launch(k_accumulate<true>, grid(np2), dim3(256), 0, s, n, B, L, p2dst, p2src, np2);
+    return e;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -338,8 +349,9 @@ cudaError_t launch_accumulate(int32_t n, float *B, ColLayout L, int32_t W, int64
 __global__ void __launch_bounds__(512) k_gamma(const int64_t *__restrict__ in_off, const int32_t *__restrict__ in_col,
                                                const float *__restrict__ w, const int32_t *__restrict__ nodes,
                                                TrieTable t, const float *__restrict__ inv_nr,
-                                               const float *__restrict__ MD, ColLayout Lc) {
+                                               const float *MD, ColLayout Lc) {
     __shared__ float part[16];
+    pdl_wait();
     const int32_t e = nodes[blockIdx.x];
     const int32_t a = t.node[e];
     const int32_t sl = t.slot[e];
@@ -353,12 +365,12 @@ __global__ void __launch_bounds__(512) k_gamma(const int64_t *__restrict__ in_of
         for (; k + 3 * T < end; k += 4 * T) {
             const int32_t x0 = __ldg(in_col + k), x1 = __ldg(in_col + k + T);
             const int32_t x2 = __ldg(in_col + k + 2 * T), x3 = __ldg(in_col + k + 3 * T);
-            sum += __ldg(col + (int64_t)x0 * rp);
-            s1 += __ldg(col + (int64_t)x1 * rp);
-            s2 += __ldg(col + (int64_t)x2 * rp);
-            s3 += __ldg(col + (int64_t)x3 * rp);
+            sum += col[(int64_t)x0 * rp];
+            s1 += col[(int64_t)x1 * rp];
+            s2 += col[(int64_t)x2 * rp];
+            s3 += col[(int64_t)x3 * rp];
         }
-        for (; k < end; k += T) sum += __ldg(col + (int64_t)__ldg(in_col + k) * rp);
+        for (; k < end; k += T) sum += col[(int64_t)__ldg(in_col + k) * rp];
         sum += s1 + s2 + s3;
     }
     for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -378,7 +390,7 @@ __global__ void __launch_bounds__(512) k_gamma(const int64_t *__restrict__ in_of
 void launch_gamma(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, const float *inv_nr,
                   const float *MD, ColLayout L, cudaStream_t s) {
     if (cnt <= 0) return;
-    k_gamma<<<(unsigned)cnt, list_threads(cnt), 0, s>>>(g.in_off, g.in_col, g.w, nodes, t, inv_nr, MD, L);
+    pdl_launch(k_gamma, dim3(cnt), dim3(list_threads(cnt)), 0, s, g.in_off, g.in_col, g.w, nodes, t, inv_nr, MD, L);
 }
 
 // ------------------------------------------------------------------------------------------------

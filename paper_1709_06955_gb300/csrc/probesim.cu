@@ -703,7 +703,9 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
     // Without profiling, the push block and the tail tile of a depth run on a second stream beside the
     // accumulate and the full-tile pull: they write other columns of A than the full tiles do.  With
     // profiling everything stays on the caller's stream, so the phase times do not overlap.
-    const bool overlap = !ws->profiling;
+    // On a small graph the kernels are a few us long and the events between the streams cost more than they hide.
+    const bool small = dg.n_active <= kSmallRows;
+    const bool overlap = !ws->profiling && !small;
     auto zmask_at = [&](int32_t d) -> const uint32_t * {
         return zany[d] ? reinterpret_cast<const uint32_t *>(d_sched + o_zmask + zoff[d]) : nullptr;
     };
@@ -723,13 +725,15 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
             PS_CUDA(cudaEventRecord(ws->ev_start, st));
             PS_CUDA(cudaStreamWaitEvent(ss, ws->ev_start, 0));
         }
-        if (H > 0) {  // height-2 columns: zero, then push from the grandchildren's gamma
-            // zeroed: the push block, and the inherited columns outside the pulled tiles (the pull writes 0 into
-            // those inside them); inherited columns are pushed after the pull, below
-            const int32_t z0 = hinh[d] > 0 ? dw[d] : h0v[d];
+        // height-2 columns: zero, then push from the grandchildren's gamma.  Zeroed: the push block, and the inherited
+        // columns outside the pulled tiles (the pull writes 0 into those inside them); inherited columns are pushed
+        // after the pull, below.  On a small graph the prepare launch zeroes them and all are pushed after the pull.
+        const int32_t z0 = hinh[d] > 0 ? dw[d] : h0v[d];
+        const bool late = small && S > 0;
+        if (H > 0 && !late) {
             ph.begin(6);
             launch_zero_cols(rows, A, La, z0, rpv[d] - z0, ss);
-            launch_push_h2(dg, node_list + node_off[d + 2], ncount[d + 2], t, A, La, h0v[d], false, ss);
+            launch_push_h2(dg, node_list + node_off[d + 2], ncount[d + 2], t, A, La, h0v[d], 0, ss);
             ph.end();
             launches += 2;
         }
@@ -745,7 +749,8 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
             ++launches;
             ph.begin(3);  // gamma scatter into D; the spare row and the split rows zeroed for the pull
             launch_prepare_pull(dg, d + 2 <= Dmax ? node_list + node_off[d + 2] : nullptr,
-                                d + 2 <= Dmax ? ncount[d + 2] : 0, t, Bm, Lb, A, La, dw[d], st);
+                                d + 2 <= Dmax ? ncount[d + 2] : 0, t, Bm, Lb, A, La, dw[d], rows, z0,
+                                late && H > 0 ? rpv[d] - z0 : 0, st);
             ph.end();
             ++launches;
             cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -807,9 +812,9 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
             PS_CUDA(cudaEventRecord(ws->ev_side, ss));
             PS_CUDA(cudaStreamWaitEvent(st, ws->ev_side, 0));
         }
-        if (hinh[d] > 0) {  // push nodes in inherited columns: after the pull has written those columns as 0
+        if (late ? H > 0 : hinh[d] > 0) {  // push nodes in inherited columns: after the pull has written those columns as 0
             ph.begin(6);
-            launch_push_h2(dg, node_list + node_off[d + 2], ncount[d + 2], t, A, La, h0v[d], true, st);
+            launch_push_h2(dg, node_list + node_off[d + 2], ncount[d + 2], t, A, La, h0v[d], late ? 2 : 1, st);
             ph.end();
             ++launches;
         }

@@ -14,18 +14,20 @@ namespace ps {
 
 namespace {
 
+// plain loads: the kernel ahead, which may still run when this one starts, writes what is gathered, so the read-only
+// path is not for it
 template <int VEC>
 struct Vec {
     float a[VEC];
     __device__ __forceinline__ void load(const float *p) {
         if (VEC == 4) {
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
+            const float4 v = *reinterpret_cast<const float4 *>(p);
             a[0] = v.x, a[1 % VEC] = v.y, a[2 % VEC] = v.z, a[3 % VEC] = v.w;
         } else if (VEC == 2) {
-            const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+            const float2 v = *reinterpret_cast<const float2 *>(p);
             a[0] = v.x, a[1 % VEC] = v.y;
         } else {
-            a[0] = __ldg(p);
+            a[0] = *p;
         }
     }
 };
@@ -36,8 +38,9 @@ __global__ void __launch_bounds__(256) k_pull_narrow(const int32_t *__restrict__
                                                      const int64_t *__restrict__ piece_beg,
                                                      const int32_t *__restrict__ piece_len, int64_t n_pieces,
                                                      const int32_t *__restrict__ in_col, const float *__restrict__ w,
-                                                     const float *__restrict__ D, int32_t dpitch, float *__restrict__ MD,
+                                                     const float *D, int32_t dpitch, float *MD,
                                                      int32_t pitch, int32_t zrow, const uint32_t *__restrict__ zmask) {
+    pdl_wait();
     constexpr int VEC = T >= 4 ? 4 : T, LPE = T > 4 ? T / 4 : 1, EPS = 8 / LPE;  // lanes an entry, entries a step
     const int lane = threadIdx.x & 31, lig = lane & 7, sub = lig % LPE, slot = lig / LPE;
     const unsigned gmask = 0xffu << (lane - lig);
@@ -124,8 +127,8 @@ void launch_pull_narrow(const DeviceGraph &g, const float *D, int32_t dpitch, fl
                         int32_t blocks_per_sm, const uint32_t *zmask, cudaStream_t s) {
     const int blocks = grid_for(g.n_pieces * 8, 256, blocks_per_sm > 0 ? blocks_per_sm : 8);
 #define PS_NARROW(T, U)                                                                                               \
-    k_pull_narrow<T, U><<<blocks, 256, 0, s>>>(g.piece_v, g.piece_beg, g.piece_len, g.n_pieces, g.in_col, g.w, D, dpitch, \
-                                               MD, pitch, g.n, zmask)
+    pdl_launch(k_pull_narrow<T, U>, dim3(blocks), dim3(256), 0, s, g.piece_v, g.piece_beg, g.piece_len, g.n_pieces,   \
+               g.in_col, g.w, D, dpitch, MD, pitch, g.n, zmask)
     switch (tile) {
         case 1: PS_NARROW(1, 2); break;
         case 2: PS_NARROW(2, 2); break;

@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(kLevelThreads, 4) k_rand_level(DeviceGraph g, 
                                                               int32_t l_max,
                                                               const uint32_t *__restrict__ qkey, uint32_t seed,
                                                               uint32_t t_keep, RandLevel L) {
+    pdl_wait();  // the level before writes the lists and the counter
     const unsigned long long packed_in = *L.packed_in;
     const long long F = (long long)(packed_in & kRandCountMask), E = (long long)(packed_in >> kRandCountBits);
     if (F == 0 || F > L.cur.cap || E > L.max_items) return;  // the host grows the list, or runs the range again
@@ -362,7 +363,7 @@ void launch_add_i32(int32_t *a, const int32_t *b, int64_t count, cudaStream_t s)
 void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const uint32_t *qkey,
                        uint32_t seed, uint32_t t_keep, const RandLevel &L, int64_t E, cudaStream_t s) {
     const int blocks = grid_for(E, kLevelThreads, 8);
-    k_rand_level<<<blocks, kLevelThreads, 0, s>>>(g, walks, l_max, qkey, seed, t_keep, L);
+    pdl_launch(k_rand_level, dim3(blocks), dim3(kLevelThreads), 0, s, g, walks, l_max, qkey, seed, t_keep, L);
 }
 void launch_rand_finalize(int32_t n, int32_t B, const int32_t *qnode, const int32_t *counts, const float *inv_nr,
                           const int32_t *ext2int, float shift, float *out, cudaStream_t s) {
