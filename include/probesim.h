@@ -119,7 +119,8 @@ probesim_status probesim_graph_info(const probesim_graph *g, int32_t *n, int64_t
 /* Dynamic updates (the paper's index-free design needs no rebuild, Sec. 1): apply k edge insertions or
  * deletions as one batch that advances the epoch.  Inserting an existing edge, deleting an absent edge and
  * self-loops are skipped; *applied (may be NULL) receives the number of edges actually changed.  Queries
- * issued after the call returns see the new edge set. */
+ * issued after the call returns see the new edge set.  The batch runs on a stream of the graph's own and is
+ * complete on return; it waits for earlier work on `stream` only when an edge array lies in device or pinned memory. */
 probesim_status probesim_insert_edges(probesim_graph *g, const int32_t *src, const int32_t *dst, int64_t k,
                                       int64_t *applied, void *stream);
 probesim_status probesim_delete_edges(probesim_graph *g, const int32_t *src, const int32_t *dst, int64_t k,

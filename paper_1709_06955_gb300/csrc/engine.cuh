@@ -193,6 +193,18 @@ struct probesim_graph {
     }
     // update scratch
     DevBuf u_batch, u_valid, u_vpre, u_delta, u_deg, u_part, u_hist, u_bounds, u_raw, u_keys[3], u_sort;
+    // update batches run on a stream of their own (under update_mu), created on first use
+    cudaStream_t u_stream = nullptr;
+    cudaEvent_t u_ready = nullptr;
+    cudaError_t ensure_update_stream() {
+        if (u_stream) return cudaSuccess;
+        int low = 0, high = 0;
+        cudaError_t e = cudaDeviceGetStreamPriorityRange(&low, &high);
+        if (e == cudaSuccess && !u_ready) e = cudaEventCreateWithFlags(&u_ready, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&u_stream, cudaStreamNonBlocking, high);
+        if (e != cudaSuccess) u_stream = nullptr;
+        return e;
+    }
     uint64_t epoch = 0;
     Workspace ws0;
     std::atomic<size_t> budget{0};  // device memory one call's working buffers may take (set while calls run)

@@ -66,3 +66,33 @@ def test_batches_equal_a_fresh_build(n, m):
     assert G.insert_edges([1, 2, 3], [0, 1, 0]) == 3
     _same(G, n, np.array([n, 2 * n + 1, 3 * n], np.int64), nodes)
     G.close()
+
+
+@pytest.mark.parametrize("memory", ["device", "pinned", "host"])
+def test_update_reads_edges_that_the_callers_stream_writes(memory):
+    """A batch runs on the graph's own stream; edges in device or pinned memory are read after the work that the caller's
+    stream already holds, here products of two matrices and then the copies that write the edges."""
+    import torch
+    from paper_1709_06955_gb300 import probesim
+    n, rng = 3000, np.random.default_rng(12)
+    s, d = dedup(n, rng.integers(0, n, 20000), rng.integers(0, n, 20000))
+    keys = np.unique(s.astype(np.int64) * n + d)
+    es, ed = (rng.integers(0, n, 4000).astype(np.int32) for _ in range(2))
+    G = probesim.Graph(n, keys // n, keys % n, probe_mode=probesim.PROBE_RANDOMIZED)
+    stream = torch.cuda.Stream()
+    a = torch.randn(4096, 4096, device="cuda")
+    bufs = [torch.zeros(4000, dtype=torch.int32, device="cuda" if memory == "device" else "cpu",
+                        pin_memory=memory == "pinned") for _ in range(2)]
+    from_dev = [torch.tensor(x, device="cuda") for x in (es, ed)]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for _ in range(30):
+            a = (a @ a) * 1e-3
+        for b, f in zip(bufs, from_dev):
+            b.copy_(f, non_blocking=memory != "host")
+    args = bufs if memory == "device" else [b.numpy() for b in bufs]
+    G.insert_edges(args[0], args[1], stream=stream.cuda_stream)
+    torch.cuda.synchronize()
+    added = (es.astype(np.int64) * n + ed)[es != ed]
+    _same(G, n, np.union1d(keys, added), [1, 2, 3])
+    G.close()
