@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "level_plan.h"
 
 // ------------------------------------------------------------------------------------------------
 // device buffers that grow on demand and are freed with the graph
@@ -123,8 +124,9 @@ struct StoreVersion {
 struct Workspace {
     DevBuf qbuf, walks, lens, ctr;
     DevBuf t_key, t_node, t_parent, t_depth, t_query, t_weight, t_height, t_slot, t_gamma, t_G;
-    DevBuf counts, offs, node_list, col_export, sched;  // level schedule: exported column nodes, uploaded plan
-    DevBuf md_a, md_b, out_stage;                       // the two score buffers; host-output staging
+    DevBuf counts, node_list, sched;  // level schedule: node counts and lists per depth, uploaded plan
+    ps::LevelPlan plan;               // its host side
+    DevBuf md_a, md_b, out_stage;     // the two score buffers; host-output staging
     DevBuf r_part, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
     DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_qk, tk_short;
     // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, deferral stack, tasks, global tables,
@@ -133,7 +135,7 @@ struct Workspace {
     DevBuf pm_in, pm_meets;  // pairwise Monte Carlo: pairs and keys, meet counts
     DevBuf pull_err;         // set by the TMA pull when a stage's wait gives up
     bool f_table_clean = false;  // f_keys (the global tables) holds only empty slots (every sweep empties its slots)
-    PinnedBuf pin_q;  // query arrays of one batch
+    PinnedBuf pin_q;  // query arrays of one batch; exported tree nodes; the plan on its way up
     PinnedBuf pin_s;  // counters and schedule offsets (fixed size, allocated at creation)
     int profiling = 0;
     size_t budget = 0;  // device memory one call on this workspace may take; 0 = the graph's budget
@@ -155,7 +157,7 @@ struct Workspace {
     }
     void release() {
         DevBuf *bufs[] = {&qbuf, &walks, &lens, &ctr, &t_key, &t_node, &t_parent, &t_depth, &t_query, &t_weight,
-                          &t_height, &t_slot, &t_gamma, &t_G, &counts, &offs, &node_list, &col_export,
+                          &t_height, &t_slot, &t_gamma, &t_G, &counts, &node_list,
                           &sched, &md_a, &md_b, &out_stage, &r_part, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
                           &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
                           &tk_cid, &tk_cval, &tk_ids, &tk_qk, &tk_short, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_pr32, &f_pr64, &f_acc,

@@ -306,11 +306,6 @@ __global__ void __launch_bounds__(kPieceThreads) k_upd_piece_fill(int32_t n, con
     }
 }
 
-__global__ void k_i64_copy(const long long *__restrict__ a, int64_t *b, int64_t count) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < count) b[i] = a[i];
-}
-
 static unsigned blocks_for(int64_t work, int threads) { return (unsigned)((work + threads - 1) / threads); }
 
 void launch_upd_mark(const DeviceGraph &g, const UpdateBatchArgs &a, long long *in_delta, long long *out_delta,
@@ -361,10 +356,6 @@ void launch_upd_pieces(int32_t n, const long long *new_off, const int32_t *n_act
     k_upd_piece_hist<<<blocks, kPieceThreads, 0, s>>>(n, new_off, n_active, hist, split_v, n_split);
     k_upd_piece_starts<<<1, 32, 0, s>>>(hist, cursor);
     k_upd_piece_fill<<<blocks, kPieceThreads, 0, s>>>(n, new_off, n_active, cursor, pv, pb, pl);
-}
-
-void launch_i64_copy(const long long *a, int64_t *b, int64_t count, cudaStream_t s) {
-    if (count > 0) k_i64_copy<<<blocks_for(count, 256), 256, 0, s>>>(a, b, count);
 }
 
 }  // namespace ps

@@ -211,10 +211,9 @@ void launch_walks(const DeviceGraph &g, const QueryBatch &q, int32_t W, int32_t 
                   uint32_t seed, int32_t *walks, int32_t *lens, bool pad, LaunchCounters *ctr, cudaStream_t s);
 void launch_trie_insert(const DeviceGraph &g, const QueryBatch &q, int32_t W, int32_t l_max, const int32_t *walks,
                         const int32_t *lens, TrieTable t, LaunchCounters *ctr, cudaStream_t s);
-void launch_sched_count(TrieTable t, int32_t *ncount, int32_t *scount, int32_t *hcount, cudaStream_t s);
-void launch_sched_export(TrieTable t, int32_t *out, int32_t *count, cudaStream_t s);
-void launch_node_lists(TrieTable t, const int32_t *node_off, int32_t *ncur, int32_t *node_list, cudaStream_t s);
-void launch_set_slots(TrieTable t, const int32_t *pairs, int32_t count, cudaStream_t s);
+void launch_sched(TrieTable t, int32_t D1, int32_t *count, int32_t *cur, int32_t *node_list, int32_t *out, int64_t stride,
+                  cudaStream_t s);
+void launch_set_slots(TrieTable t, const int32_t *ent, const int32_t *col, int32_t count, cudaStream_t s);
 // scatters the gammas of the tree nodes two depths down into B, and zeroes B's spare row and A's split rows over the
 // pulled columns, and (zw > 0) columns [z0, z0 + zw) of A's rows below zrows
 void launch_prepare_pull(const DeviceGraph &g, const int32_t *nodes, int32_t cnt, TrieTable t, float *B, ColLayout Lb,
@@ -444,7 +443,6 @@ inline int32_t rec_shift_for(int32_t n) {  // ids below n, shifted, fit 8 bits
 void launch_upd_pieces(int32_t n, const long long *new_off, const int32_t *n_active, unsigned long long *hist,
                        unsigned long long *cursor, int32_t *split_v, unsigned long long *n_split, int32_t *pv,
                        int64_t *pb, int32_t *pl, cudaStream_t s);
-void launch_i64_copy(const long long *a, int64_t *b, int64_t count, cudaStream_t s);
 
 // device-side initial build of the graph store (graph_build.cu)
 int64_t radix_tiles(int64_t count);

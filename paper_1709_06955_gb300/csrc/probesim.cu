@@ -10,7 +10,6 @@
 #include <shared_mutex>
 #include <new>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
 #include "engine.cuh"
@@ -424,258 +423,64 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
     PS_CUDA(cudaMemsetAsync(t.G, 0, 4 * cap, st));
     launch_trie_insert(dg, qb, P.W, L, ws->walks.as<int32_t>(), ws->lens.as<int32_t>(), t, d_ctr, st);
     ++launches;
-    // 3. level schedule: nodes, dense columns (pulled) and push columns per depth
+    // 3. level schedule: the tree's nodes per depth, and the nodes that own a column (exported to pinned memory).  Every
+    // dense node's heir takes over its column one depth down, so along a chain of heirs the MD column of the child
+    // already is the D column of the parent and nothing is copied.  Push columns (height 2) sit in a block after the
+    // dense columns.
     const int32_t D1 = L + 2;
-    PS_CUDA(ws->counts.ensure(sizeof(int32_t) * 5 * D1));
-    int32_t *d_ncount = ws->counts.as<int32_t>(), *d_scount = d_ncount + D1, *d_hcount = d_ncount + 2 * D1,
-            *d_ncur = d_ncount + 3 * D1;
-    PS_CUDA(cudaMemsetAsync(d_ncount, 0, sizeof(int32_t) * 4 * D1, st));
-    launch_sched_count(t, d_ncount, d_scount, d_hcount, st);
+    const int64_t most = walk_nodes + B;  // tree nodes
+    PS_CUDA(ws->counts.ensure(sizeof(int32_t) * (4 * D1 + 1)));
+    PS_CUDA(ws->node_list.ensure(sizeof(int32_t) * most));
+    PS_CUDA(ws->pin_q.ensure(sizeof(int32_t) * 3 * (size_t)most));
+    int32_t *d_count = ws->counts.as<int32_t>();
+    const int32_t *h_exp = ws->pin_q.as<int32_t>();
+    PS_CUDA(cudaMemsetAsync(d_count, 0, sizeof(int32_t) * (4 * D1 + 1), st));
+    launch_sched(t, D1, d_count, d_count + 3 * D1, ws->node_list.as<int32_t>(), ws->pin_q.as<int32_t>(), most, st);
     ph.end();
-    ++launches;
+    launches += 2;
     int32_t *h_cnt = reinterpret_cast<int32_t *>(ws->pin_s.as<char>() + 256);
-    PS_CUDA(cudaMemcpyAsync(h_cnt, d_ncount, sizeof(int32_t) * 3 * D1, cudaMemcpyDeviceToHost, st));
+    PS_CUDA(cudaMemcpyAsync(h_cnt, d_count, sizeof(int32_t) * 3 * D1, cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaMemcpyAsync(h_ctr, d_ctr, sizeof(LaunchCounters), cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaStreamSynchronize(st));
     if (h_ctr->overflow) return fail(PROBESIM_E_CUDA, "internal: walk tree table overflow");
-    std::vector<int32_t> ncount(h_cnt, h_cnt + D1), scount(h_cnt + D1, h_cnt + 2 * D1),
-        hcount(h_cnt + 2 * D1, h_cnt + 3 * D1);
-    int32_t Dmax = 0;
-    for (int32_t d = 0; d < D1; ++d)
-        if (ncount[d] > 0) Dmax = d;
-    std::vector<int32_t> node_off(D1 + 1, 0), dw(D1, 0);
-    for (int32_t d = 0; d < D1; ++d) node_off[d + 1] = node_off[d] + ncount[d];
-    const int32_t total_nodes = node_off[D1];
-    ws->stats.tree_nodes += total_nodes;
-    for (int32_t d = 0; d < D1; ++d) ws->stats.vectors += scount[d] + hcount[d];
-    PS_CUDA(ws->offs.ensure(sizeof(int32_t) * (D1 + 1)));
-    int32_t *d_node_off = ws->offs.as<int32_t>();
-    int32_t *h_offs = h_cnt + 3 * D1;
-    std::memcpy(h_offs, node_off.data(), sizeof(int32_t) * (D1 + 1));
-    PS_CUDA(cudaMemcpyAsync(d_node_off, h_offs, sizeof(int32_t) * (D1 + 1), cudaMemcpyHostToDevice, st));
-    PS_CUDA(ws->node_list.ensure(sizeof(int32_t) * std::max(1, total_nodes)));
-    ph.begin(1);
-    launch_node_lists(t, d_node_off, d_ncur, ws->node_list.as<int32_t>(), st);
-    // columns.  Every dense node's "heir" (its dense child with the deepest chain below it) takes over its
-    // column one depth down, so along a chain of heirs the MD column of the child already is the D column of
-    // the parent and nothing is copied.  Push columns (height 2) sit in a block after the dense columns.
-    int32_t ncol_nodes = 0;
-    for (int32_t d = 0; d < D1; ++d) ncol_nodes += scount[d] + hcount[d];
-    PS_CUDA(ws->col_export.ensure(sizeof(int32_t) * (5 * (size_t)std::max(1, ncol_nodes) + 1)));
-    int32_t *d_exp = ws->col_export.as<int32_t>(), *d_expn = d_exp + 5 * (size_t)std::max(1, ncol_nodes);
-    PS_CUDA(cudaMemsetAsync(d_expn, 0, sizeof(int32_t), st));
-    launch_sched_export(t, d_exp, d_expn, st);
-    ph.end();
-    launches += 2;
-    PS_CUDA(ws->pin_q.ensure(sizeof(int32_t) * (5 * (size_t)std::max(1, ncol_nodes) + 64)));
-    int32_t *h_exp = ws->pin_q.as<int32_t>();
-    PS_CUDA(cudaMemcpyAsync(h_exp, d_exp, sizeof(int32_t) * 5 * (size_t)ncol_nodes, cudaMemcpyDeviceToHost, st));
-    PS_CUDA(cudaStreamSynchronize(st));
     const auto host0 = std::chrono::steady_clock::now();  // the host-side schedule starts (the device waits)
-    // export rows: 0 entry, 1 depth, 2 parent entry, 3 dense, 4 query
-    std::vector<std::vector<int32_t>> dense_at(D1), push_at(D1);
-    for (int32_t i = 0; i < ncol_nodes; ++i) (h_exp[5 * i + 3] ? dense_at : push_at)[h_exp[5 * i + 1]].push_back(i);
-    // the export row of every node's parent (-1: none).  Tree entries are slots of the table, so a flat array
-    // indexes them unless the table is much larger than the exported set
-    std::vector<int32_t> prow(ncol_nodes, -1);
-    if (t.cap <= 32 * (int64_t)ncol_nodes + 65536) {
-        std::vector<int32_t> row_of((size_t)t.cap, -1);
-        for (int32_t i = 0; i < ncol_nodes; ++i) row_of[h_exp[5 * i]] = i;
-        for (int32_t i = 0; i < ncol_nodes; ++i) {
-            const int32_t pe = h_exp[5 * i + 2];
-            if (pe >= 0) prow[i] = row_of[pe];
-        }
-    } else {
-        std::unordered_map<int32_t, int32_t> row_of;
-        row_of.reserve(2 * (size_t)ncol_nodes + 1);
-        for (int32_t i = 0; i < ncol_nodes; ++i) row_of[h_exp[5 * i]] = i;
-        for (int32_t i = 0; i < ncol_nodes; ++i) {
-            const auto it = row_of.find(h_exp[5 * i + 2]);
-            if (it != row_of.end()) prow[i] = it->second;
-        }
+    std::vector<int32_t> ncount(D1), node_off(D1 + 1, 0);
+    const int32_t *scount = h_cnt + D1, *hcount = h_cnt + 2 * D1;
+    int32_t Dmax = 0, ncol_nodes = 0;
+    for (int32_t d = 0; d < D1; ++d) {
+        ncount[d] = h_cnt[d] + scount[d] + hcount[d];
+        node_off[d + 1] = node_off[d] + ncount[d];
+        ncol_nodes += scount[d] + hcount[d];
+        if (ncount[d] > 0) Dmax = d;
     }
-    // heights are not exported; the heir is the dense child with the deepest dense descendant chain, found
-    // bottom-up, ties to the smaller entry
-    std::vector<int32_t> chain(ncol_nodes, 0), heir(ncol_nodes, -1), col(ncol_nodes, -1);
-    for (int32_t d = Dmax; d >= 1; --d)
-        for (int32_t i : dense_at[d]) {
-            const int32_t pr = prow[i];
-            if (pr < 0) continue;
-            const int32_t h = heir[pr];
-            if (h < 0 || chain[i] > chain[h] || (chain[i] == chain[h] && h_exp[5 * i] < h_exp[5 * h])) heir[pr] = i;
-            chain[pr] = std::max(chain[pr], chain[i] + 1);
-        }
-    // a dense node without a dense heir takes its first push child (smallest entry) as "push heir": that
-    // child's pushed column is then the node's D column, in place, and the accumulate has nothing to copy
-    std::vector<int32_t> pheir(ncol_nodes, -1);
-    for (int32_t d = 1; d <= Dmax; ++d)
-        for (int32_t i : push_at[d]) {
-            const int32_t pr = prow[i];
-            if (pr < 0 || heir[pr] >= 0) continue;
-            if (pheir[pr] < 0 || h_exp[5 * i] < h_exp[5 * pheir[pr]]) pheir[pr] = i;
-        }
-    std::vector<char> is_pheir(ncol_nodes, 0);
-    for (int32_t i = 0; i < ncol_nodes; ++i)
-        if (pheir[i] >= 0) is_pheir[pheir[i]] = 1;
-    // a chain is a maximal path of heirs (ending, possibly, in a push heir); all its nodes share one column.
-    // Chains are coloured deepest bottom
-    // first, each taking the smallest column whose chains all start more than one depth below its bottom
-    // (every chain coloured before it ends at least as deep, so that is "free over its depth range and the
-    // depth below"); the columns in use at a depth then stay close to the number of dense nodes there.
-    std::vector<char> is_heir(ncol_nodes, 0);
-    for (int32_t i = 0; i < ncol_nodes; ++i)
-        if (heir[i] >= 0) is_heir[heir[i]] = 1;
-    struct Chain {
-        int32_t head, top, bottom;
-    };
-    std::vector<Chain> chains;
-    for (int32_t d = 0; d <= Dmax; ++d)
-        for (int32_t i : dense_at[d]) {
-            if (is_heir[i]) continue;
-            int32_t x = i, bot = d;
-            while (heir[x] >= 0) x = heir[x], ++bot;
-            if (pheir[x] >= 0) ++bot;
-            chains.push_back({i, d, bot});
-        }
-    std::sort(chains.begin(), chains.end(), [&](const Chain &x, const Chain &y) {
-        if (x.bottom != y.bottom) return x.bottom > y.bottom;
-        if (x.top != y.top) return x.top < y.top;
-        return h_exp[5 * x.head] < h_exp[5 * y.head];
-    });
-    // per column: the smallest top depth of the chains holding it, kept in a max segment tree over the
-    // columns (columns not opened yet hold INT32_MAX) so the first column above a depth is found in log time
-    int32_t seg_leaves = 1;
-    while (seg_leaves < std::max<int32_t>(1, (int32_t)chains.size())) seg_leaves <<= 1;
-    std::vector<int32_t> top_min(2 * (size_t)seg_leaves, INT32_MAX);
-    for (const Chain &ch : chains) {
-        // a column whose chain ends at depth d stays unused at depth d+1 too: there the accumulate sets it to
-        // the chain bottom's D, while other groups may still read what a chain starting at d+1 left in it.
-        // The chain takes the first column all of whose chains start below ch.bottom + 1.
-        int32_t i = 1;
-        while (i < seg_leaves) i = top_min[2 * i] > ch.bottom + 1 ? 2 * i : 2 * i + 1;
-        const int32_t c = i - seg_leaves;
-        top_min[i] = std::min(top_min[i], ch.top);
-        for (i >>= 1; i >= 1; i >>= 1) top_min[i] = std::max(top_min[2 * i], top_min[2 * i + 1]);
-        int32_t last = ch.head;
-        for (int32_t x = ch.head; x >= 0; x = heir[x]) col[x] = c, last = x;
-        if (pheir[last] >= 0) col[pheir[last]] = c;
-    }
-    std::vector<int32_t> width(D1, 0), rho(B, -1);
-    for (int32_t d = 0; d <= Dmax; ++d) {
-        int32_t w = 0;
-        for (int32_t i : dense_at[d]) w = std::max(w, col[i] + 1);
-        width[d] = w;
-        if (d == 0)
-            for (int32_t i : dense_at[0]) rho[h_exp[5 * i + 4]] = col[i];
-    }
-    // pull tiles per depth: full 32-column tiles (or 16-column halves, if the tuner prefers them) and one
-    // narrower tail tile of 1..16 columns; dw = the columns the pull covers
-    std::vector<int32_t> nfull(D1, 0), tail(D1, 0);
-    for (int32_t d = 0; d <= Dmax; ++d) {
-        int32_t full = width[d] / 32, rem = width[d] - 32 * full;
-        if (rem > 16) ++full, rem = 0;
-        nfull[d] = full;
-        tail[d] = rem > 0 ? pull_tile_for(rem, 16) : 0;
-        dw[d] = 32 * full + tail[d];
-    }
-    // push nodes of a depth that keep a column of their own (the others inherited their parent's)
-    std::vector<int32_t> hinh(D1, 0);
-    for (int32_t d = 0; d <= Dmax; ++d) {
-        std::vector<int32_t> &pa = push_at[d];
-        const size_t before = pa.size();
-        pa.erase(std::remove_if(pa.begin(), pa.end(), [&](int32_t x) { return is_pheir[x] != 0; }), pa.end());
-        hinh[d] = (int32_t)(before - pa.size());
-    }
-    // MD of depth d is read in place as D of depth d-1, so its matrix holds the columns of both depths:
-    // max(dw[d-1], dw[d]) dense columns (inherited push columns among them), then the push block at h0[d]
-    std::vector<int32_t> h0v(D1, 0), rpv(D1, 0);
+    ws->stats.tree_nodes += node_off[D1];
+    ws->stats.vectors += ncol_nodes;
+    LevelPlan &plan = ws->plan;
+    if (!plan.build(ncol_nodes, h_exp, h_exp + most, h_exp + 2 * most, t.cap, B, D1,
+                    [](int32_t rem) { return pull_tile_for(rem, 16); }))
+        return fail(PROBESIM_E_CUDA, "internal: a tree node without its parent");
+    const std::vector<int32_t> &nfull = plan.nfull, &tail = plan.tail, &dw = plan.dw, &hinh = plan.hinh, &h0v = plan.h0,
+                               &rpv = plan.cols, &zoff = plan.zoff, &zany = plan.zany, &p1_at = plan.p1_at,
+                               &p2_at = plan.p2_at;
+    const std::vector<int64_t> &acc_src = plan.acc_src;
     std::vector<ColLayout> lay(D1);
     int64_t max_floats = 4 * (int64_t)n;
     for (int32_t d = 0; d <= Dmax; ++d) {
-        const int32_t dense_w = std::max(dw[d], d >= 1 ? dw[d - 1] : 0);
-        h0v[d] = round_up(std::max(dense_w, 1), 4);
-        rpv[d] = round_up(h0v[d] + (int32_t)push_at[d].size(), 4);
         lay[d] = make_layout(n, rpv[d]);
         max_floats = std::max<int64_t>(max_floats, lay[d].size());
         ws->stats.max_columns = std::max<int64_t>(ws->stats.max_columns, rpv[d]);
-    }
-    // push columns of a depth: grouped by parent (in parent column order), so a parent's push children are
-    // adjacent for the accumulate
-    for (int32_t d = 0; d <= Dmax; ++d) {
-        std::vector<int32_t> &pa = push_at[d];
-        auto pcol = [&](int32_t x) { return d >= 1 && prow[x] >= 0 ? col[prow[x]] : -1; };
-        std::sort(pa.begin(), pa.end(), [&](int32_t x, int32_t y) {
-            const int32_t px = pcol(x), py = pcol(y);
-            return px != py ? px < py : h_exp[5 * x] < h_exp[5 * y];
-        });
-        for (size_t r = 0; r < pa.size(); ++r) col[pa[r]] = h0v[d] + (int32_t)r;
     }
     const size_t level_bytes2 = 2 * (size_t)max_floats * sizeof(float);
     if (level_bytes2 > budget_of(g, ws)) {
         *too_big = B > 1;
         return fail(PROBESIM_E_NOMEM, "score vectors of one query exceed the workspace budget");
     }
-    // accumulate groups per depth d (dense parents at d): dst = parent column (| set flag when it has no heir
-    // of either kind), srcs = columns (at d+1) of its children other than the heir
-    std::vector<std::vector<int32_t>> kids(ncol_nodes);
-    for (int32_t i = 0; i < ncol_nodes; ++i) {
-        const int32_t pr = prow[i];
-        if (pr >= 0 && heir[pr] != i && pheir[pr] != i) kids[pr].push_back(col[i]);
-    }
-    // Each group is cut into parts of at most four sources, stored as a destination (bit 30: set, for a node
-    // without heir) and an int4 of sources (-1 = none).  The first part of every group runs in the
-    // accumulate's first phase, the others add in a second phase (so one node with many children does not
-    // hold up a block).  Records of depth d: first parts [p1_at[d], p1_at[d+1]), later parts likewise.
-    std::vector<int32_t> pairs, p1dst, p1src, p2dst, p2src, p1_at(D1 + 1, 0), p2_at(D1 + 1, 0);
-    std::vector<int64_t> acc_src(D1, 0);  // sources of a depth's parts
-    pairs.reserve(2 * (size_t)ncol_nodes);
-    for (int32_t i = 0; i < ncol_nodes; ++i) {
-        pairs.push_back(h_exp[5 * i]);
-        pairs.push_back(col[i]);
-    }
-    auto put_part = [](std::vector<int32_t> &dst, std::vector<int32_t> &src, int32_t dcol, const std::vector<int32_t> &k,
-                       size_t from) {
-        dst.push_back(dcol);
-        for (size_t j = 0; j < 4; ++j) src.push_back(from + j < k.size() ? k[from + j] : -1);
-    };
-    for (int32_t d = 0; d < D1; ++d) {
-        p1_at[d] = (int32_t)p1dst.size();
-        p2_at[d] = (int32_t)p2dst.size();
-        if (d > Dmax) continue;
-        // groups in destination order, sources ascending
-        std::sort(dense_at[d].begin(), dense_at[d].end(), [&](int32_t x, int32_t y) { return col[x] < col[y]; });
-        for (int32_t i : dense_at[d]) {
-            std::sort(kids[i].begin(), kids[i].end());
-            const bool own = heir[i] < 0 && pheir[i] < 0;  // no heir of any kind: the column is set
-            if (kids[i].empty() && !own) continue;            // its column already is its heir's MD
-            acc_src[d] += (int64_t)kids[i].size();
-            put_part(p1dst, p1src, col[i] | (own ? (1 << 30) : 0), kids[i], 0);
-            for (size_t f = 4; f < kids[i].size(); f += 4) put_part(p2dst, p2src, col[i], kids[i], f);
-        }
-    }
-    p1_at[D1] = (int32_t)p1dst.size();
-    p2_at[D1] = (int32_t)p2dst.size();
-    // zero masks of the pull at each depth: an inherited push column inside the pulled tiles is written as 0
-    // there (the push fills it afterwards); one 32-bit word per 32 columns, words of depth d at zoff[d]
-    std::vector<int32_t> zmask, zoff(D1 + 1, 0), zany(D1, 0);
-    for (int32_t d = 0; d < D1; ++d) {
-        zoff[d] = (int32_t)zmask.size();
-        zmask.resize(zmask.size() + (size_t)(dw[d] + 31) / 32, 0);
-    }
-    zoff[D1] = (int32_t)zmask.size();
-    for (int32_t i = 0; i < ncol_nodes; ++i) {
-        if (!is_pheir[i]) continue;
-        const int32_t d = h_exp[5 * i + 1], c = col[i];
-        if (c < dw[d]) {
-            zmask[zoff[d] + c / 32] |= (int32_t)(1u << (c % 32));
-            zany[d] = 1;
-        }
-    }
-    // upload: slot pairs, super-root columns, part destinations, zero masks, part sources (int4, 16-byte aligned)
-    const size_t sched_ints =
-        pairs.size() + B + p1dst.size() + p2dst.size() + zmask.size() + p1src.size() + p2src.size() + 8;
-    PS_CUDA(ws->sched.ensure(sizeof(int32_t) * std::max<size_t>(1, sched_ints)));
-    PS_CUDA(ws->pin_q.ensure(sizeof(int32_t) * std::max<size_t>(1, sched_ints)));
+    // upload: entries and their columns, super-root columns, part destinations, zero masks, part sources (int4, 16-byte
+    // aligned)
+    const size_t sched_ints = 2 * (size_t)ncol_nodes + B + plan.p1dst.size() + plan.p2dst.size() + plan.zmask.size() +
+                              plan.p1src.size() + plan.p2src.size() + 8;
+    PS_CUDA(ws->sched.ensure(sizeof(int32_t) * sched_ints));
+    PS_CUDA(ws->pin_q.ensure(sizeof(int32_t) * sched_ints));
     int32_t *h_sched = ws->pin_q.as<int32_t>();
     size_t o = 0;
     auto put = [&](const std::vector<int32_t> &v) {
@@ -684,14 +489,14 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
         o += v.size();
         return at;
     };
-    const size_t o_pairs = put(pairs), o_rho = put(rho), o_p1dst = put(p1dst), o_p2dst = put(p2dst),
-                 o_zmask = put(zmask);
+    const size_t o_ent = put(plan.ent), o_col = put(plan.col), o_rho = put(plan.rho), o_p1dst = put(plan.p1dst),
+                 o_p2dst = put(plan.p2dst), o_zmask = put(plan.zmask);
     o = (o + 3) / 4 * 4;
-    const size_t o_p1src = put(p1src), o_p2src = put(p2src);
+    const size_t o_p1src = put(plan.p1src), o_p2src = put(plan.p2src);
     int32_t *d_sched = ws->sched.as<int32_t>();
     PS_CUDA(cudaMemcpyAsync(d_sched, h_sched, sizeof(int32_t) * o, cudaMemcpyHostToDevice, st));
     ws->stats.phase_ms[9] += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - host0).count();
-    launch_set_slots(t, d_sched + o_pairs, (int32_t)(pairs.size() / 2), st);
+    launch_set_slots(t, d_sched + o_ent, d_sched + o_col, ncol_nodes, st);
     ++launches;
     const int32_t *d_rho = d_sched + o_rho;
     // 4. level loop, deepest depth first.  Two score buffers: A receives this depth's MD; B holds the depth

@@ -142,66 +142,101 @@ void launch_trie_insert(const DeviceGraph &g, const QueryBatch &q, int32_t W, in
     k_trie_insert<<<(W + 255) / 256, 256, 0, s>>>(q, W, l_max, walks, lens, t, ctr);
 }
 
-// Counts tree nodes and vector columns per depth.  A node owns a score-vector column when its subtree has
-// height >= 2: only then is the sum of its children's contributions more than a sparse set of nodes.
-// Height >= 3 nodes (and a super-root of height 2) get "dense" columns filled by the pull; height-2 nodes
-// get "push" columns filled from their grandchildren's few gamma terms.  Dense columns take local indices
-// 0.., push columns are encoded -2 - local until the host knows the dense width of the depth.
-__global__ void k_sched_count(TrieTable t, int32_t *ncount, int32_t *scount, int32_t *hcount) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= t.cap) return;
-    if (t.key[e] == kEmptyKey) return;
-    const int32_t d = t.depth[e], h = t.height[e];
-    atomicAdd(&ncount[d], 1);
-    if (h >= 3 || (d == 0 && h >= 2)) t.slot[e] = atomicAdd(&scount[d], 1);
-    else if (h == 2) t.slot[e] = -2 - atomicAdd(&hcount[d], 1);
-    else t.slot[e] = -1;
+// ------------------------------------------------------------------------------------------------
+// level schedule: two passes over the tree's table.  The first counts the nodes of each depth by class -- without a column,
+// dense (height >= 3, and a super-root of height 2), push (height 2) -- and leaves the class in the slot; the second
+// writes every node into its depth's list and exports the nodes that own a column (dense or push).  Both count in shared
+// memory and take one global add per block and counter: the counters are a few dozen addresses that every node would
+// queue on.  The export goes straight to the host's pinned memory, so one synchronisation brings the counts and the nodes.
+// (R-MAT 2^18, two queries at eps 0.05, 59,404 nodes: 46 us in three kernels, 19 in these two.)
+// ------------------------------------------------------------------------------------------------
+constexpr int kSchedThreads = 256, kSchedPer = 4;
+
+// count: [3][D1]
+__global__ void __launch_bounds__(kSchedThreads) k_sched_count(TrieTable t, int32_t D1, int32_t *count) {
+    extern __shared__ int32_t sh[];
+    for (int i = threadIdx.x; i < 3 * D1; i += kSchedThreads) sh[i] = 0;
+    __syncthreads();
+    const int64_t e0 = blockIdx.x * (int64_t)(kSchedThreads * kSchedPer) + threadIdx.x;
+#pragma unroll
+    for (int u = 0; u < kSchedPer; ++u) {
+        const int64_t e = e0 + u * kSchedThreads;
+        if (e >= t.cap || t.key[e] == kEmptyKey) continue;
+        const int32_t d = t.depth[e], h = t.height[e];
+        const int cls = h >= 3 || (d == 0 && h >= 2) ? 1 : (h == 2 ? 2 : 0);
+        t.slot[e] = cls == 1 ? 0 : (cls == 2 ? -2 : -1);
+        atomicAdd(&sh[cls * D1 + d], 1);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * D1; i += kSchedThreads)
+        if (sh[i] > 0) atomicAdd(&count[i], sh[i]);
 }
 
-void launch_sched_count(TrieTable t, int32_t *ncount, int32_t *scount, int32_t *hcount, cudaStream_t s) {
-    k_sched_count<<<(unsigned)((t.cap + 255) / 256), 256, 0, s>>>(t, ncount, scount, hcount);
+// cur: [D1 + 1], zero; cur[D1] counts the exported nodes.  out: three arrays of `stride`: entry, parent entry (-1 - query
+// at depth 0), 2 * depth + (1 if dense).
+__global__ void __launch_bounds__(kSchedThreads) k_sched_lists(TrieTable t, int32_t D1, const int32_t *__restrict__ count,
+                                                               int32_t *cur, int32_t *node_list, int32_t *out,
+                                                               int64_t stride) {
+    extern __shared__ int32_t sh[];
+    int32_t *s_n = sh, *s_at = sh + D1 + 1;
+    for (int i = threadIdx.x; i <= D1; i += kSchedThreads) s_n[i] = 0;
+    __syncthreads();
+    const int64_t e0 = blockIdx.x * (int64_t)(kSchedThreads * kSchedPer) + threadIdx.x;
+    int32_t dep[kSchedPer], pos[kSchedPer], slot[kSchedPer], at[kSchedPer];
+#pragma unroll
+    for (int u = 0; u < kSchedPer; ++u) {
+        const int64_t e = e0 + u * kSchedThreads;
+        dep[u] = -1;
+        if (e >= t.cap || t.key[e] == kEmptyKey) continue;
+        dep[u] = t.depth[e];
+        slot[u] = t.slot[e];
+        pos[u] = atomicAdd(&s_n[dep[u]], 1);
+        if (slot[u] != -1) at[u] = atomicAdd(&s_n[D1], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {  // the depths' offsets, and this block's place in each
+        int32_t base = 0;
+        for (int d0 = 0; d0 <= D1; d0 += 32) {
+            const int d = d0 + threadIdx.x;
+            int32_t x = d < D1 ? count[d] + count[D1 + d] + count[2 * D1 + d] : 0, sum = x;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t y = __shfl_up_sync(0xffffffffu, sum, o);
+                if ((int)threadIdx.x >= o) sum += y;
+            }
+            if (d <= D1) s_at[d] = (d < D1 ? base + sum - x : 0) + (s_n[d] > 0 ? atomicAdd(&cur[d], s_n[d]) : 0);
+            base += __shfl_sync(0xffffffffu, sum, 31);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kSchedPer; ++u) {
+        if (dep[u] < 0) continue;
+        const int64_t e = e0 + u * kSchedThreads;
+        node_list[s_at[dep[u]] + pos[u]] = (int32_t)e;
+        if (slot[u] == -1) continue;
+        const int64_t i = s_at[D1] + at[u];
+        out[i] = (int32_t)e;
+        out[stride + i] = dep[u] > 0 ? t.parent[e] : -1 - t.query[e];
+        out[2 * stride + i] = 2 * dep[u] + (slot[u] >= 0 ? 1 : 0);
+    }
 }
 
-// Exports every node that owns a column (dense or push): entry, depth, parent entry, dense flag, query.
-__global__ void k_sched_export(TrieTable t, int32_t *out, int32_t *count) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= t.cap) return;
-    if (t.key[e] == kEmptyKey) return;
-    const int32_t sl = t.slot[e];
-    if (sl == -1) return;
-    const int32_t i = atomicAdd(count, 1);
-    out[5 * i + 0] = (int32_t)e;
-    out[5 * i + 1] = t.depth[e];
-    out[5 * i + 2] = t.parent[e];
-    out[5 * i + 3] = sl >= 0 ? 1 : 0;
-    out[5 * i + 4] = t.query[e];
+void launch_sched(TrieTable t, int32_t D1, int32_t *count, int32_t *cur, int32_t *node_list, int32_t *out, int64_t stride,
+                  cudaStream_t s) {
+    const unsigned blocks = (unsigned)((t.cap + kSchedThreads * kSchedPer - 1) / (kSchedThreads * kSchedPer));
+    k_sched_count<<<blocks, kSchedThreads, 3 * D1 * sizeof(int32_t), s>>>(t, D1, count);
+    k_sched_lists<<<blocks, kSchedThreads, 2 * (D1 + 1) * sizeof(int32_t), s>>>(t, D1, count, cur, node_list, out, stride);
 }
 
-void launch_sched_export(TrieTable t, int32_t *out, int32_t *count, cudaStream_t s) {
-    k_sched_export<<<(unsigned)((t.cap + 255) / 256), 256, 0, s>>>(t, out, count);
-}
-
-// Node lists per depth (every tree node).
-__global__ void k_node_lists(TrieTable t, const int32_t *__restrict__ node_off, int32_t *ncur, int32_t *node_list) {
-    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= t.cap) return;
-    if (t.key[e] == kEmptyKey) return;
-    const int32_t d = t.depth[e];
-    node_list[node_off[d] + atomicAdd(&ncur[d], 1)] = (int32_t)e;
-}
-
-void launch_node_lists(TrieTable t, const int32_t *node_off, int32_t *ncur, int32_t *node_list, cudaStream_t s) {
-    k_node_lists<<<(unsigned)((t.cap + 255) / 256), 256, 0, s>>>(t, node_off, ncur, node_list);
-}
-
-// slot[pairs[2i]] = pairs[2i+1]
-__global__ void k_set_slots(TrieTable t, const int32_t *__restrict__ pairs, int32_t count) {
+// slot[ent[i]] = col[i]
+__global__ void k_set_slots(TrieTable t, const int32_t *__restrict__ ent, const int32_t *__restrict__ col, int32_t count) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) t.slot[pairs[2 * i]] = pairs[2 * i + 1];
+    if (i < count) t.slot[ent[i]] = col[i];
 }
 
-void launch_set_slots(TrieTable t, const int32_t *pairs, int32_t count, cudaStream_t s) {
-    if (count > 0) k_set_slots<<<(count + 255) / 256, 256, 0, s>>>(t, pairs, count);
+void launch_set_slots(TrieTable t, const int32_t *ent, const int32_t *col, int32_t count, cudaStream_t s) {
+    if (count > 0) k_set_slots<<<(count + 255) / 256, 256, 0, s>>>(t, ent, col, count);
 }
 
 }  // namespace ps
