@@ -179,26 +179,28 @@ typedef struct {
                                n_active below): 4m + 16 pieces + 4 rows + 4 S (n_active + rows) */
     int64_t kernel_launches;/* all kernels this library launched in the call */
     double phase_ms[12];    /* profiling on: CUDA-event time per phase of the deterministic path: 0 walks,
-                               1 walk tree and level schedule, 2 D accumulate, 3 gamma scatter and the
-                               zeroing the pull needs, 4 unused, 5 pull, 6 push columns, 7 gamma, 8 estimates.  9 (always recorded):
-                               host wall-clock time of the column schedule, during which the device waits;
-                               10-11 unused */
+                               1 walk tree and level schedule, 2 D accumulate, 3 gamma scatter and the zeroing
+                               the pull needs, 4 unused, 5 pull, 6 push columns, 7 gamma, 8 estimates.  9 (always
+                               recorded): host wall-clock time of the column schedule, during which the device
+                               waits; 10-11 unused */
     int64_t max_columns;    /* widest score matrix of the level loop, in columns (deterministic path) */
     int64_t probes;         /* walk prefixes probed one by one (Pruning Rule 2 or the switch) */
     int64_t switched;       /* of those, the probes the switch of Sec. 4.4 handed to Alg. 3 */
-    int64_t table_passes;   /* passes over the frontier engine's per-level tables (more than one per level when
-                               a table exceeds a quarter of the memory budget) */
-    int64_t max_table_slots;/* largest per-level table, in slots of 12 bytes */
+    int64_t table_passes;   /* rounds of the frontier engine that wrote a next frontier: one per level and range of
+                               probes (more ranges than one when the memory budget cuts a level) */
+    int64_t max_table_slots;/* slots of all tables of the largest round, in shared or device memory */
     int64_t deferred;       /* probe ranges the frontier engine set aside at a level and resumed later, so that
-                               one level's frontier stays within an eighth of the memory budget */
+                               one level's frontier stays within an eighth of the memory budget and
+                               its tables in device memory within a quarter */
 } probesim_stats;
 
 probesim_status probesim_set_profiling(probesim_graph *g, int32_t on);
 
 /* Device memory that one call's working buffers on this graph may take, in bytes (0 restores the default, 60%
  * of the device's memory at graph creation).  A call whose queries need more is cut into smaller batches; the
- * frontier engine (Pruning Rule 2, the switch) also cuts a level's table into passes of a quarter of it.  A
- * single query that still does not fit fails with PROBESIM_E_NOMEM.  Results do not depend on the budget. */
+ * frontier engine (Pruning Rule 2, the switch) also sets probes of a level aside, the randomized PROBE cuts its walks
+ * into ranges.  A single query that still does not fit fails with PROBESIM_E_NOMEM.  Results do not depend on the
+ * budget. */
 probesim_status probesim_set_memory_budget(probesim_graph *g, double bytes);
 
 /* Autotuner of the PROBE level kernel's launch shape on this graph.  It times the pull over the graph's own

@@ -55,8 +55,9 @@ __device__ __forceinline__ uint32_t node_hash(int32_t v) {
     return (uint32_t)(((unsigned long long)(uint32_t)v * 0x9E3779B97F4A7C15ull) >> 32);
 }
 
-// a bijection of 32 bits (xor-shifts and odd multiplies): the shared tables take their slot from its low bits and the
-// part from its high bits, and splitting a part always separates distinct nodes in the end
+// a bijection of 32 bits (xor-shifts and odd multiplies, the finaliser of A. Appleby's MurmurHash3): the shared tables
+// take their slot from its low bits and the part from its high bits, and splitting a part always separates distinct
+// nodes in the end
 __device__ __forceinline__ uint32_t mix32(uint32_t h) {
     h ^= h >> 16;
     h *= 0x85EBCA6Bu;

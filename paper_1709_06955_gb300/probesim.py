@@ -341,8 +341,8 @@ class Graph:
 
     def set_tuning(self, wide_tile, blocks_per_sm=None):
         """Sets the pull's launch shape by hand (probesim_set_tuning): wide_tile 16, 32 (the default: wider tiles
-        where a depth has enough), 64 (32-column tiles two per pass) or 96 (32-column tiles gathered by the TMA); blocks_per_sm, if given, 8 values for tile widths 1..32,
-        the pairs and the TMA launch."""
+        where a depth has enough), 64 (32-column tiles two per pass) or 96 (32-column tiles gathered by the TMA);
+        blocks_per_sm, if given, 8 values for tile widths 1..32, the pairs and the TMA launch."""
         arr = None
         if blocks_per_sm is not None:
             vals = [int(b) for b in blocks_per_sm]
