@@ -12,7 +12,8 @@
 //            applied to the sums as they are written (Rule 2 of level j + 1), and entries that are pruned or have no
 //            out-edges are not written at all
 // The classes, by the bound D = min(out-degree sum, n) on the next frontier:
-//   last     the probe's last level: pushes go straight into its query's estimate with weight w
+//   last     the probe's last level: pushes go straight into its query's estimate with weight w, or, for one query on a
+//            graph of a few slabs, through sums in shared memory (k_fr_last)
 //   single   one entry: its targets are distinct, so they are written as they come
 //   warp, block, mid, wide   a table in shared memory (up to kWarpD, kBlockD, kMidD, kPartD entries); a wide probe's
 //            targets are split by hash into up to kMaxParts parts, each a block that scans all of the probe's items and
@@ -162,9 +163,9 @@ __global__ void __launch_bounds__(kThreads) k_fr_plan(TrieTable t, FrontierProbe
         if (lane == 0) atomicAdd(totals + c, v);
     }
     const unsigned long long live = cls != kFrNone ? d : 0ull;
-    const unsigned long long vs[5] = {sweeps, D, slots, cls == kFrGlobal ? slots : 0ull, live};
-    const int at[5] = {kFrSweep, kFrTotD, kFrTotSlots, kFrTotGlobal, kFrTotItems};
-    for (int k = 0; k < 5; ++k) {
+    const unsigned long long vs[6] = {sweeps, D, slots, cls == kFrGlobal ? slots : 0ull, live, cls == kFrLast ? d : 0ull};
+    const int at[6] = {kFrSweep, kFrTotD, kFrTotSlots, kFrTotGlobal, kFrTotItems, kFrTotLast};
+    for (int k = 0; k < 6; ++k) {
         const unsigned long long v = warp_sum(vs[k]);
         if (lane == 0 && v) atomicAdd(totals + at[k], v);
     }
@@ -382,6 +383,47 @@ __global__ void __launch_bounds__(kThreads) k_fr_direct(DeviceGraph g, TrieTable
             }
             fr_append(beg, deg, sc, packed, out);
         });
+    }
+}
+
+// The last level of one query's call on a graph of at most kLastParts slabs: the estimates' 64-bit adds in the L2 (5e10 a
+// second) were the engine's largest part there, so a block sums a slab of the nodes (v = part mod parts) in shared memory
+// over its share of the tasks and adds the slab to the estimates once.  Every part reads every item, so it pays while the
+// parts are few and the items many (see launch_fr_level).
+constexpr int kLastThreads = 1024;
+__global__ void __launch_bounds__(kLastThreads) k_fr_last(DeviceGraph g, TrieTable t, FrontierProbes P, FrontierLevel a,
+                                                          int64_t task0, int64_t ntasks, uint32_t parts) {
+    extern __shared__ uint32_t smem[];
+    uint32_t *lo = smem, *hi = smem + kSlabN;
+    const uint32_t part = blockIdx.x % parts, size = ((uint32_t)g.n + parts - 1) / parts;
+    for (uint32_t i = threadIdx.x; i < size; i += kLastThreads) lo[i] = 0u, hi[i] = 0u;
+    __syncthreads();
+    const uint32_t inv = parts > 1 ? (uint32_t)((0x100000000ull + parts - 1) / parts) : 0u;
+    auto index = [&](uint32_t v) { return parts > 1 ? __umulhi(v, inv) : v; };  // v / parts, exact for v < 2^32 / parts
+    const int64_t step = (int64_t)(gridDim.x / parts) * (kLastThreads / 32);
+    for (int64_t i = (int64_t)(blockIdx.x / parts) * (kLastThreads / 32) + (threadIdx.x >> 5); i < ntasks; i += step) {
+        const FrontierTask tk = a.tasks[task0 + i];
+        const int32_t p = tk.p, ex = P.ex[p];
+        const unsigned long long pk = P.packed[p];
+        const uint32_t d = (uint32_t)(pk >> kFrCountBits), cnt = (uint32_t)(pk & kFrCountMask);
+        const uint32_t t0 = tk.part * (uint32_t)kFrChunk, t1 = min(d, t0 + (uint32_t)kFrChunk);
+        const long long w = t.weight[P.slot[p]];
+        fr_items(
+            g, a.src + P.beg[p], cnt, d, t0, t1,
+            [&](int32_t v) { return v != ex && (uint32_t)v - index((uint32_t)v) * parts == part; },
+            [&](int32_t v) { return __ldg(g.w + v); },
+            [&](bool on, int32_t v, float wv, float val) {
+                if (!on) return;
+                const unsigned long long c = (unsigned long long)(f_to_fx(wv * val) * w);
+                const uint32_t h = index((uint32_t)v), cl = (uint32_t)c, old = atomicAdd(lo + h, cl);
+                const uint32_t ch = (uint32_t)(c >> 32) + (old + cl < old ? 1u : 0u);
+                if (ch) atomicAdd(hi + h, ch);
+            });
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < size; i += kLastThreads) {
+        const unsigned long long c = ((unsigned long long)hi[i] << 32) | lo[i];
+        if (c) atomicAdd(a.acc + (int64_t)i * parts + part, c);  // a sum above 0 belongs to a node below n
     }
 }
 
@@ -696,7 +738,19 @@ cudaError_t launch_fr_level(const DeviceGraph &g, TrieTable t, FrontierProbes P,
     if (n(kFrSingle) > 0)
         k_fr_direct<false><<<blocks_for(32 * n(kFrSingle)), kThreads, 0, s>>>(g, t, P, a, base.at[kFrSingle],
                                                                               n(kFrSingle));
-    if (n(kFrLast) > 0)
+    // k_fr_last against k_fr_direct<true>, ms per query with Thm. 2's split of 0.1, 16 edges a node: 20,000 nodes (1 part)
+    // 3.6 against 9.0, 60,000 (3) 8.6 / 14.5, 100,000 (5) 11.9 / 15.4, 150,000 (7) 13.6 / 15.1, 200,000 (9) 20.4 / 22.0,
+    // 240,000 (10) 23.0 / 24.0.  Adding the slabs costs about as much as 4 million items' adds; tasks of few items cost
+    // their start once per part.
+    const uint32_t parts = ((uint32_t)g.n + kSlabN - 1) / kSlabN;
+    if (n(kFrLast) > 0 && a.one_query && parts <= kLastParts && ntasks[kFrTotLast] >= kLastItems &&
+        ntasks[kFrTotLast] >= kLastPerTask * ntasks[kFrLast]) {
+        constexpr int bytes = (int)kSlabN * 8;
+        e = cudaFuncSetAttribute(k_fr_last, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+        k_fr_last<<<parts * std::max(1u, 152u / parts), kLastThreads, bytes, s>>>(g, t, P, a, base.at[kFrLast],
+                                                                                  n(kFrLast), parts);
+    } else if (n(kFrLast) > 0)
         k_fr_direct<true><<<blocks_for(32 * n(kFrLast)), kThreads, 0, s>>>(g, t, P, a, base.at[kFrLast], n(kFrLast));
     if (n(kFrSweep) > 0) k_fr_sweep<<<(unsigned)n(kFrSweep), kThreads, 0, s>>>(g, t, P, a, base.at[kFrSweep]);
     return cudaSuccess;

@@ -302,12 +302,15 @@ constexpr unsigned long long kFrCountMask = (1ull << kFrCountBits) - 1;
 // classes of a probe at a level (see frontier.cu), then the sweep of the global tables, then the range's totals
 enum {
     kFrNone = 0, kFrLast, kFrSingle, kFrWarp, kFrBlock, kFrMid, kFrWide, kFrSlab, kFrGlobal, kFrSweep, kFrClasses,
-    kFrTotD = kFrClasses, kFrTotSlots, kFrTotGlobal, kFrTotItems, kFrTotEntries, kFrTotals
+    kFrTotD = kFrClasses, kFrTotSlots, kFrTotGlobal, kFrTotItems, kFrTotLast, kFrTotEntries, kFrTotals
 };
 // bounds on the next frontier for the tables in shared memory: three quarters of their slots (half of the warp table's)
 constexpr unsigned kWarpD = 128, kBlockD = 1536, kMidD = 6144, kPartD = 12288;
 constexpr unsigned kSlabN = 24576, kSlabParts = 6;  // nodes of a slab part
 constexpr unsigned kMaxParts = 6;
+// k_fr_last serves the last level: nodes in at most kLastParts slabs, items of a level and items per task at least
+constexpr unsigned kLastParts = 10;
+constexpr unsigned long long kLastItems = 1ull << 22, kLastPerTask = 256;
 constexpr unsigned kFrChunk = 2048;                              // work items per warp task
 struct FrontierProbes {
     int32_t P = 0;
@@ -348,6 +351,7 @@ struct FrontierLevel {
     const float *pw = nullptr;            // sqrt(c)^k
     float eps_p = 0.f;
     int32_t j = 0;
+    bool one_query = false;               // acc has one row
 };
 void launch_fr_init(TrieTable t, FrontierProbes P, const int64_t *out_off, const float *pw, float eps_p,
                     FrontierEntry *list, cudaStream_t s);

@@ -1076,6 +1076,7 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
         a.pw = d_pw;
         a.eps_p = g->cfg.eps_p;
         a.j = R.j;
+        a.one_query = B == 1;
         PS_CUDA(launch_fr_level(dg, t, of_parity(R.cur), a, base, h_tot, st, &launches));
         PS_CUDA(cudaGetLastError());
         if (G > 0) ws->f_table_clean = true;

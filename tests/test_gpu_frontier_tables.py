@@ -141,3 +141,24 @@ def test_scores_that_round_to_zero_stay_members():
             want += sum(len(out[x]) for x in frontier)
             frontier = {v for x in frontier for v in out[x] if v != pre[len(pre) - j - 2]}
     assert pushes == want
+
+
+@pytest.mark.parametrize("n", [7001, 24576, 24577, 98305, 245760, 245761])
+def test_last_level_summed_in_shared_memory(n):
+    """One query's last-level pushes are summed in slabs of 24,576 nodes in shared memory (on a graph of at most ten of
+    them), several queries' straight in the estimates: the sums are exact, so the estimates are equal bit for bit."""
+    from paper_1709_06955_gb300 import probesim
+    rng = np.random.default_rng(n)
+    m = 16 * n
+    s = rng.permutation(n)[(n * rng.random(m) ** 3).astype(np.int64)]
+    d = rng.permutation(n)[(n * rng.random(m) ** 2).astype(np.int64)]
+    s, d = dedup(n, s, d)
+    sp = probesim.split_error(0.1, c=0.6, shift=True)
+    G = probesim.Graph(n, s, d, l_max=sp["l_max"], eps_p=sp["eps_p"], shift=sp["shift"])
+    nodes = [int(x) for x in rng.choice(np.unique(d), 2, replace=False)]
+    ids = np.array([5, 6])
+    both = G.single_source(probesim.make_queries(nodes, eps=sp["eps"], query_ids=ids))
+    for i in range(2):
+        alone = G.single_source(probesim.make_queries(nodes[i:i + 1], eps=sp["eps"], query_ids=ids[i:i + 1]))
+        assert np.array_equal(alone[0], both[i])
+    G.close()
