@@ -25,11 +25,13 @@
 // Why: a global table costs an item two random sectors, and its sweeps read every slot; with one table per level in
 // device memory the expansion and its compaction were 90 % of this engine's time.  Scanning a probe's items again costs
 // a coalesced read and a hash; at six parts the two cost the same (Thm. 2's split on 150,000 nodes, ms per query: 16.9 at
-// 6 parts, 18.2 at 8, 51.7 at 16; at 4 parts 17.3).  What bounds it now: the last level's 64-bit atomics on the
-// estimates (5e10 a second), then the tables' shared-memory atomics.
+// 6 parts, 18.2 at 8, 51.7 at 16; at 4 parts 17.3).  What bounds it now: the
+// tables' scans of items (issue slots), and for batches and large graphs the last level's 64-bit atomics on the estimates
+// (5e10 a second).
 // Measured, before and after (one table per level in device memory): one eps_a = 0.1 query with Rule 2, 150,000 nodes
-// 24.4 -> 14.8 ms, 10,000 nodes 21.7 -> 9.6; 64 mixed-eps switch queries on R-MAT 2^22: expansion, compaction and
-// scans 405 -> 18 ms (the early switch: 95 of the 123 ms left without it).
+// 24.4 -> 14.8 ms (k_fr_last: another query 16.5 -> 14.4), 10,000 nodes 21.7 -> 9.6 (without k_fr_last); 64 mixed-eps
+// switch queries on R-MAT 2^22: expansion, compaction and scans 405 -> 18 ms (the early switch: 95 of the 123 ms left
+// without it).
 //
 // Scores are FP32 products accumulated in 2^-44 fixed point (64-bit sums; in shared memory a 32-bit low half whose
 // carries go to the high half).  The sums are exact whatever order the adds land in, so the frontier sets, the pruning
