@@ -13,6 +13,7 @@
 
 #include "internal.cuh"
 #include "level_plan.h"
+#include "rand_lists.h"
 
 // ------------------------------------------------------------------------------------------------
 // device buffers that grow on demand and are freed with the graph

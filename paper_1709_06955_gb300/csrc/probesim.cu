@@ -717,10 +717,8 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
         l.cap = (long long)std::min(ws->r_ent[k].cap / sizeof(RandEntry), ws->r_first[k].cap / sizeof(long long));
         return l;
     };
-    // the work items whose members are taken to fit a list: `need` below gives at least that many entries
-    auto items_of = [&](const RandList &l) -> long long {
-        return l.cap <= 1024 ? l.cap : (long long)((double)(l.cap - 1) / list_share);
-    };
+    // the work items of the levels that a list is sized for (rand_lists.h)
+    auto items_of = [&](const RandList &l) -> long long { return rand_list_items(list_share, l.cap); };
     PS_ALLOC_RANGE(ws->r_ent[0].ensure(sizeof(RandEntry) * ni));
     PS_ALLOC_RANGE(ws->r_first[0].ensure(sizeof(long long) * ni));
     // counters of levels 0 .. 255 and their checks
@@ -745,7 +743,7 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
             *too_short = true;
             return fail(PROBESIM_E_NOMEM, "internal: a randomized PROBE level outgrew its list");
         }
-        const int64_t need = std::max<int64_t>(1024, (int64_t)(list_share * (double)E) + 1);
+        const int64_t need = std::max<int64_t>(kRandListMin, rand_list_entries(list_share, E));
         // an overflowed counter, or lists beyond the budget: a smaller walk range needs less
         if (h_ctr[256 + j] != (unsigned long long)E ||
             ((sizeof(RandEntry) + sizeof(long long)) * (size_t)need > budget_of(g, ws) / 4 && W > 1)) {
@@ -754,7 +752,7 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
         }
         PS_ALLOC_RANGE(ws->r_ent[nx].ensure(sizeof(RandEntry) * need));
         PS_ALLOC_RANGE(ws->r_first[nx].ensure(sizeof(long long) * need));
-        const int32_t end = std::min(max_len - 1, j + group);
+        const int32_t begin = j, end = std::min(max_len - 1, j + group);
         for (int32_t t = j; t < end; ++t) {
             RandLevel Lv;
             Lv.cur = list_of(t & 1);
@@ -779,6 +777,7 @@ static probesim_status rand_range(probesim_graph *g, Workspace *ws, const QueryB
             ws->stats.levels += 1;
             ++j;
         }
+        if (j == begin) return fail(PROBESIM_E_CUDA, "internal: a randomized PROBE level did not run");
         group = std::min(8, 2 * group);
     }
     return PROBESIM_OK;
