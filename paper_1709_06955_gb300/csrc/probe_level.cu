@@ -305,8 +305,9 @@ static cudaError_t accumulate_rows(int32_t n, float *B, const ColLayout &L, int3
                                    const int4 *p1src, int32_t np1, const int32_t *p2dst, const int4 *p2src, int32_t np2,
                                    cudaStream_t s) {
     const size_t bytes = (size_t)R * W * sizeof(float);
+    // the same for every call: the attribute belongs to the kernel, and calls of other threads launch it with other sizes
     const cudaError_t e = cudaFuncSetAttribute(k_accumulate_rows<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)bytes);
+                                               (int)kStageBytes);
     if (e != cudaSuccess) return e;
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, kStageBytes / std::max<size_t>(1, bytes)));
     return pdl_launch(k_accumulate_rows<R>, dim3(grid_for(((int64_t)n + R - 1) / R, 1, per_sm)), dim3(kStageThreads), bytes,
