@@ -1058,11 +1058,11 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
         PS_ALLOC(ws->f_list[nx].ensure(sizeof(FrontierEntry) * std::max<long long>(1, D)));
         PS_ALLOC(ws->f_tasks.ensure(sizeof(FrontierTask) * std::max<long long>(1, nt)));
         if (G > 0) {
-            const void *k0 = ws->f_keys.p;
-            PS_ALLOC(ws->f_keys.ensure(sizeof(FrontierSlot) * G));
-            if (ws->f_keys.p != k0 || !ws->f_table_clean)  // new memory, or a failed call left slots behind
-                PS_CUDA(cudaMemsetAsync(ws->f_keys.p, 0, ws->f_keys.cap, st));
-            ws->f_table_clean = false;  // until this level's sweep has emptied its slots
+            bool fresh = false;
+            PS_ALLOC(ws->f_keys.ensure(sizeof(FrontierSlot) * G, &fresh));
+            const bool clear = fresh || !ws->f_table_clean;  // new memory, or a failed call left slots behind
+            ws->f_table_clean = false;                       // until this level's sweep has emptied its slots
+            if (clear) PS_CUDA(cudaMemsetAsync(ws->f_keys.p, 0, ws->f_keys.cap, st));
         }
         launch_fr_tasks(of_parity(R.cur), R.p0, R.p1, n, base, d_cursor, ws->f_tasks.as<FrontierTask>(), st);
         ++launches;
