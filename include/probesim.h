@@ -190,8 +190,8 @@ typedef struct {
                                probes (more ranges than one when the memory budget cuts a level) */
     int64_t max_table_slots;/* slots of all tables of the largest round, in shared or device memory */
     int64_t deferred;       /* probe ranges the frontier engine set aside at a level and resumed later, so that
-                               one level's frontier stays within an eighth of the memory budget and
-                               its tables in device memory within a quarter */
+                               one level's frontier stays within an eighth of the memory budget, its
+                               tables in device memory within a quarter and its tasks within a sixteenth */
 } probesim_stats;
 
 probesim_status probesim_set_profiling(probesim_graph *g, int32_t on);

@@ -973,14 +973,19 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
     }
     const float *d_pw = ws->f_tab.as<float>();
     const long long *d_thr = sw_mode ? reinterpret_cast<const long long *>(ws->f_tab.as<char>() + 256 * sizeof(float)) : nullptr;
-    // The deterministic rounds work on probe ranges [p0, p1) at a level j.  A range whose next frontiers or global tables
-    // might not fit their part of the budget keeps as many of its first probes as the bounds allow and defers the
+    // The deterministic rounds work on probe ranges [p0, p1) at a level j.  A range whose next frontiers, global tables or
+    // task lists might not fit their part of the budget keeps as many of its first probes as the bounds allow and defers the
     // others, with their level-j segments, to a stack; they resume once the kept probes have run out.  Every probe's
     // last-level pushes land in the estimate exactly once, whatever the split.
     const long long slot_cap =
         std::max<long long>((long long)n, (long long)(budget_of(g, ws) / 4 / sizeof(FrontierSlot)));
     const long long list_cap =
         std::max<long long>((long long)n, (long long)(budget_of(g, ws) / 8 / sizeof(FrontierEntry)));
+    // tasks of a level (a last-level or single-entry probe has one per kFrChunk items and no next frontier or table to be
+    // held back by); one probe's fit n or 2^31 / kFrChunk, and a class's number is a grid size
+    const long long task_cap = std::min<long long>(
+        ((long long)1 << 31) - 1,
+        std::max<long long>((long long)n, (long long)(budget_of(g, ws) / 16 / sizeof(FrontierTask))));
     struct Range {
         int32_t p0, p1, j;
         int cur;
@@ -1020,9 +1025,12 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
             live = false;
             continue;
         }
-        if ((D > list_cap || G > slot_cap) && R.p1 - R.p0 > 1) {  // defer the range's last probes
-            const double keep = 0.9 * std::min(D > 0 ? (double)list_cap / (double)D : 1.0,
-                                               G > 0 ? (double)slot_cap / (double)G : 1.0);
+        long long nt = 0;
+        for (int c = kFrNone + 1; c < kFrClasses; ++c) nt += (long long)h_tot[c];
+        if ((D > list_cap || G > slot_cap || nt > task_cap) && R.p1 - R.p0 > 1) {  // defer the range's last probes
+            const double keep = 0.9 * std::min({D > 0 ? (double)list_cap / (double)D : 1.0,
+                                                G > 0 ? (double)slot_cap / (double)G : 1.0,
+                                                nt > 0 ? (double)task_cap / (double)nt : 1.0});
             const int32_t pm = R.p0 + std::max(1, (int32_t)std::min<double>(keep * (R.p1 - R.p0), R.p1 - R.p0 - 1));
             Range tail{pm, R.p1, R.j, R.cur, true, R.on_stack ? R.at : stack_top};
             if (!R.on_stack) {
@@ -1048,12 +1056,7 @@ static probesim_status run_batch_frontier(probesim_graph *g, Workspace *ws, cons
         if (D > 0) ws->stats.table_passes += 1;
         ws->stats.max_table_slots = std::max<int64_t>(ws->stats.max_table_slots, (int64_t)h_tot[kFrTotSlots]);
         FrontierBases base;
-        long long nt = 0;
-        for (int c = kFrNone + 1; c < kFrClasses; ++c) {
-            base.at[c] = nt;
-            nt += (long long)h_tot[c];
-            if (h_tot[c] >= ((unsigned long long)1 << 31)) return fail(PROBESIM_E_INVALID, "too much work in one call");
-        }
+        for (int c = kFrLast; c < kFrSweep; ++c) base.at[c + 1] = base.at[c] + (long long)h_tot[c];
         const int nx = R.cur ^ 1;
         PS_ALLOC(ws->f_list[nx].ensure(sizeof(FrontierEntry) * std::max<long long>(1, D)));
         PS_ALLOC(ws->f_tasks.ensure(sizeof(FrontierTask) * std::max<long long>(1, nt)));
