@@ -12,12 +12,15 @@ struct DevBuf {
     size_t cap = 0;
     bool pooled = false;  // from the stream-ordered pool (cudaMallocAsync): freed with cudaFreeAsync
     bool view = false;    // a part of another buffer: nothing to free
+    bool writing = false;             // pooled: work on `writer` may still be writing it
+    cudaStream_t writer = nullptr;    // pooled: the stream it was allocated on
     void set_view(void *q, size_t bytes) {
         release();
         p = q, cap = bytes, view = true;
     }
     // allocates exactly `bytes` from the device's stream-ordered pool on stream s (no device-wide synchronisation,
-    // unlike cudaMalloc / cudaFree); for buffers that are written once, such as a new version of the graph store
+    // unlike cudaMalloc / cudaFree); for buffers that are written once, such as a new version of the graph store, by work
+    // on s, until settle()
     cudaError_t alloc_pooled(size_t bytes, cudaStream_t s) {
         release();
         cudaError_t e = cudaMallocAsync(&p, std::max<size_t>(256, bytes), s);
@@ -27,9 +30,11 @@ struct DevBuf {
             return e;
         }
         cap = std::max<size_t>(256, bytes);
-        pooled = true;
+        pooled = writing = true;
+        writer = s;
         return cudaSuccess;
     }
+    void settle() { writing = false; }  // the work on `writer` is complete
     cudaError_t ensure(size_t bytes) { return bytes <= cap && p ? cudaSuccess : ensure_exact(bytes + bytes / 8); }
     // the same; *fresh tells whether the memory is newly allocated, and so holds anything.  The address does not tell: an
     // allocation that replaces a smaller one may come back at the same place.
@@ -65,15 +70,16 @@ struct DevBuf {
         return e;
     }
     // A pooled buffer returns to the pool on the calling thread's default stream, without waiting: its readers
-    // have synchronised their own streams before they let go of it.
+    // have synchronised their own streams before they let go of it.  Before it has settled (an update that fails half-way)
+    // it returns in the order of the stream whose kernels may still be writing it.
     void release() {
         if (p && !view) {
-            if (pooled) cudaFreeAsync(p, cudaStreamPerThread);
+            if (pooled) cudaFreeAsync(p, writing ? writer : cudaStreamPerThread);
             else cudaFree(p);
         }
         p = nullptr;
         cap = 0;
-        pooled = view = false;
+        pooled = view = writing = false;
     }
     template <class T>
     T *as() const { return static_cast<T *>(p); }

@@ -25,6 +25,10 @@ struct StoreVersion {
     std::shared_ptr<StoreVersion> base;  // set when this version reuses base's arrays (an update that changed nothing)
     ps::DeviceGraph dg;
     uint64_t epoch = 0;
+    void settle() {  // every array is written
+        for (DevBuf *b : {&in_off, &in_col, &out_off, &out_col, &w, &rec, &piece_v, &piece_beg, &piece_len, &split_v})
+            b->settle();
+    }
     ~StoreVersion() {
         for (DevBuf *b : {&in_off, &in_col, &out_off, &out_col, &w, &rec, &piece_v, &piece_beg, &piece_len, &split_v, &arena})
             b->release();

@@ -1497,6 +1497,7 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
         npieces += (int64_t)hh[k];
         if (k <= kPiece) npieces_active += (int64_t)hh[k];
     }
+    nv->settle();
     // publish the new version: queries that start from now on read it, those in flight keep the old one
     DeviceGraph &ng = nv->dg;
     ng = dg;

@@ -11,6 +11,7 @@ RUNTIME = r"""
 #include <cstdio>
 #include <cstdlib>
 static char place[1 << 20];
+static cudaStream_t freed_on;
 static size_t limit = sizeof(place);  // larger allocations fail
 extern "C" {
 // every allocation comes back at the same place, as it may when one that was just freed is replaced
@@ -19,7 +20,7 @@ cudaError_t cudaFree(void *) { return cudaSuccess; }
 cudaError_t cudaMallocHost(void **p, size_t n) { return cudaMalloc(p, n); }
 cudaError_t cudaFreeHost(void *) { return cudaSuccess; }
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) { return cudaMalloc(p, n); }
-cudaError_t cudaFreeAsync(void *, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaFreeAsync(void *, cudaStream_t s) { return freed_on = s, cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *, const void *, size_t, cudaMemcpyKind, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { return cudaSuccess; }
@@ -57,4 +58,20 @@ def test_new_memory_is_told_by_the_allocation_not_by_its_address(tmp_path):
     CHECK(b.ensure(10, &fresh) == cudaSuccess && fresh && b.p == before);
     CHECK(b.ensure(2 << 20, &fresh) != cudaSuccess && b.p == nullptr);
     CHECK(b.ensure(10, &fresh) == cudaSuccess && fresh);
+    """)
+
+
+def test_memory_still_being_written_is_freed_in_its_writers_order(tmp_path):
+    run(tmp_path, r"""
+    const cudaStream_t writer = (cudaStream_t)0x1234;
+    DevBuf b;
+    CHECK(b.alloc_pooled(1000, writer) == cudaSuccess);
+    b.release();  // an update that failed half-way: kernels on `writer` may be at it
+    CHECK(freed_on == writer);
+    CHECK(b.alloc_pooled(1000, writer) == cudaSuccess);
+    b.settle();  // written and published; the last reader lets go, on whatever thread
+    b.release();
+    CHECK(freed_on == cudaStreamPerThread);
+    CHECK(b.alloc_pooled(2000, writer) == cudaSuccess && b.alloc_pooled(1000, writer) == cudaSuccess);
+    CHECK(freed_on == writer);
     """)
