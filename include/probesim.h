@@ -170,13 +170,15 @@ typedef struct {
     int64_t tree_nodes;     /* reverse-reachability tree nodes (Alg. 4), the virtual super-roots included */
     int64_t vectors;        /* dense score vectors pushed (tree nodes with a subtree of height >= 2) */
     int64_t levels;         /* level-loop iterations */
-    int64_t edge_gathers;   /* (edge, vector) pairs processed by the PROBE level kernel */
+    int64_t edge_gathers;   /* (edge, vector) pairs processed by the PROBE level kernel (below depth 0 it runs over the
+                               in-lists of nodes with out-edges only: nobody reads the other rows) */
     int64_t probe_launches; /* launches of the PROBE level kernel */
     double probe_ms;        /* their summed CUDA-event duration (profiling on), else 0 */
     double probe_bytes;     /* algorithmic bytes of those launches: per launch 4 per in-edge index, 16 per in-list piece
                                record, 4 per row's weight, and for each of the launch's S columns 4 per row read (the
-                               n_active rows of nodes with out-edges) and 4 per row written (all n at depth 0, those
-                               n_active below): 4m + 16 pieces + 4 rows + 4 S (n_active + rows) */
+                               n_active rows of nodes with out-edges) and 4 per row written.  Rows: all n at depth 0,
+                               the n_active below, and the edges and pieces of their in-lists: 4 edges + 16 pieces +
+                               4 rows + 4 S (n_active + rows) */
     int64_t kernel_launches;/* all kernels this library launched in the call */
     double phase_ms[12];    /* profiling on: CUDA-event time per phase of the deterministic path: 0 walks,
                                1 walk tree and level schedule, 2 D accumulate, 3 gamma scatter and the zeroing

@@ -59,6 +59,7 @@ struct DeviceGraph {
     float *w = nullptr;
     int64_t n_pieces = 0;
     int64_t n_pieces_active = 0;   // the first of them: those of the rows below n_active
+    int64_t m_active = 0;          // the edges of those rows' in-lists
     int32_t *piece_v = nullptr;
     int64_t *piece_beg = nullptr;
     int32_t *piece_len = nullptr;  // length | (split ? 1 << 31 : 0)

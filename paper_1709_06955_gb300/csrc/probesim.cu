@@ -214,10 +214,10 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     PS_CUDA(cudaGetLastError());
     PS_CUDA(cudaStreamSynchronize(st));
     if (ends[0] != mu || ends[1] != mu) return fail(PROBESIM_E_CUDA, "internal: the built lists disagree on m");
-    int64_t npieces = 0, npieces_active = 0;
+    int64_t npieces = 0, npieces_active = 0, m_active = 0;
     for (int k = 0; k < nb; ++k) {
         npieces += (int64_t)hh[k];
-        if (k <= kPiece) npieces_active += (int64_t)hh[k];
+        if (k <= kPiece) npieces_active += (int64_t)hh[k], m_active += k * (int64_t)hh[k];  // bucket k: pieces of k edges
     }
     DeviceGraph &d = sv->dg;
     d.n = n;
@@ -231,6 +231,7 @@ static probesim_status build_graph(probesim_graph *g, int32_t n, const int32_t *
     d.rec_shift = rec_shift_for(n);
     d.n_pieces = npieces;
     d.n_pieces_active = npieces_active;
+    d.m_active = m_active;
     d.piece_v = sv->piece_v.as<int32_t>();
     d.piece_beg = sv->piece_beg.as<int64_t>();
     d.piece_len = sv->piece_len.as<int32_t>();
@@ -621,8 +622,9 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
                 marks.push_back({e0, e1});
             }
             ws->stats.probe_launches += 1;
-            ws->stats.edge_gathers += dg.m * (int64_t)S;
-            ws->stats.probe_bytes += 4.0 * dg.m + 16.0 * dgl.n_pieces + 4.0 * rows + 4.0 * ((double)dg.n_active + rows) * S;
+            const int64_t edges = d > 0 ? dg.m_active : dg.m;  // of the rows pulled
+            ws->stats.edge_gathers += edges * S;
+            ws->stats.probe_bytes += 4.0 * edges + 16.0 * dgl.n_pieces + 4.0 * rows + 4.0 * ((double)dg.n_active + rows) * S;
         }
         if (overlap && side_work) {  // the gamma of this depth (and every later step) waits for the side work
             PS_CUDA(cudaEventRecord(ws->ev_side, ss));
@@ -1492,10 +1494,10 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     PS_CUDA(cudaMemcpyAsync(&n_active, d_active, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     PS_CUDA(cudaGetLastError());
     PS_CUDA(cudaStreamSynchronize(st));
-    int64_t npieces = 0, npieces_active = 0;
+    int64_t npieces = 0, npieces_active = 0, m_active = 0;
     for (int k = 0; k < nb; ++k) {
         npieces += (int64_t)hh[k];
-        if (k <= kPiece) npieces_active += (int64_t)hh[k];
+        if (k <= kPiece) npieces_active += (int64_t)hh[k], m_active += k * (int64_t)hh[k];  // bucket k: pieces of k edges
     }
     nv->settle();
     // publish the new version: queries that start from now on read it, those in flight keep the old one
@@ -1510,6 +1512,7 @@ probesim_status ps::apply_updates(probesim_graph *g, const int32_t *src, const i
     ng.rec = nv->rec.as<int4>();
     ng.n_pieces = npieces;
     ng.n_pieces_active = npieces_active;
+    ng.m_active = m_active;
     ng.piece_v = nv->piece_v.as<int32_t>();
     ng.piece_beg = nv->piece_beg.as<int64_t>();
     ng.piece_len = nv->piece_len.as<int32_t>();
