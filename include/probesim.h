@@ -205,16 +205,15 @@ probesim_status probesim_set_profiling(probesim_graph *g, int32_t on);
  * budget. */
 probesim_status probesim_set_memory_budget(probesim_graph *g, double bytes);
 
-/* Autotuner of the PROBE level kernel's launch shape on this graph.  It times the pull over the graph's own
- * in-lists for tile widths {1,2,4,8,16,32} columns and {2,4,8,16} blocks per SM (a constant-filled 64-column
- * score matrix, CUDA events, three runs after a warm-up), keeps the fastest shape per width and, for the
- * 32-column tiles of wide matrices, whichever of 32-column tiles, 16-column halves, 32-column tiles taken two
- * per pass (one read of the in-lists for both) and 32-column tiles gathered by the TMA takes less time.
- * Later queries on the graph use the choice.  Takes about a second; results do not depend on it (only the
- * summation order). */
+/* Autotuner of the PROBE level kernel's launch shape on this graph.  It times the pulls that the level loop launches
+ * below depth 0 -- the kernel of each tail width {1,2,4,8,16}, the wide and the 32-column full tiles -- over the graph's
+ * own in-lists for {2,4,8,16} blocks per SM (a constant-filled score matrix of four wide tiles where 1 GB and half the
+ * memory budget hold them, CUDA events, the best of three runs after a warm-up), and for the full tiles the other shapes of
+ * probesim_set_tuning.  What is faster than the default by more than 2 % is kept.  Later queries on the graph use the
+ * choice.  Takes well under a second; results do not depend on it (only the summation order). */
 probesim_status probesim_autotune(probesim_graph *g, void *stream);
 /* The current choice: *wide_tile in {16, 32, 64, 96} (see probesim_set_tuning); blocks_per_sm[6] for tile widths
- * 1, 2, 4, 8, 16, 32. */
+ * 1, 2, 4, 8, 16 and the full tiles (32: of the wide tiles). */
 probesim_status probesim_get_tuning(const probesim_graph *g, int32_t *wide_tile, int32_t *blocks_per_sm);
 /* Sets the launch shape by hand: wide_tile in {16, 32, 64, 96} (32: 32-column tiles, four or two of them taken as one
  * 128- or 64-column tile where a depth has enough of them; 64: 32-column tiles two per pass; 96: 32-column

@@ -126,10 +126,7 @@ struct probesim_graph {
     Workspace ws0;
     std::atomic<size_t> budget{0};  // device memory one call's working buffers may take (set while calls run)
     size_t budget0 = 0;  // the default: 60% of device memory at creation
-    // pull launch shape chosen by probesim_autotune (defaults until then)
-    int32_t tune_wide = 32;       // full tiles: 16, 32, kPullPairs (32-column tiles two per pass) or kPullTma
-    int32_t tune_bps[128] = {0};  // blocks per SM per tile width, kPullPairs / kPullTma for those (0 = default)
-    int32_t tuned = 0;
+    ps::PullTuning tune;  // the pull's launch shape: probesim_autotune, probesim_set_tuning (defaults until then)
 };
 
 

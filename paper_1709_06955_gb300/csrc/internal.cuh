@@ -7,6 +7,7 @@
 #include <string>
 
 #include "../../include/probesim.h"
+#include "pull_shape.h"
 
 namespace ps {
 
@@ -240,28 +241,17 @@ void launch_zero_cols(int32_t n, float *MD, ColLayout L, int32_t c0, int32_t wid
 // Row n of D (the spare row) must be zero over the pulled columns.
 // zmask (may be null): bit i of word k set = column 32k + i of the launch's columns is written as 0.
 // tile = kPullPairs: 32-column tiles (ntiles of them, strides as for tile 32) taken two per pass.
-constexpr int32_t kPullPairs = 64;
-// tile = kPullWide: 128-column tiles; kPullMid: 64-column tiles.  The level loop takes full 32-column tiles four at a time
-// the first way while the rows its gathers read (n_active of them) fit the L2 at 128 columns, else two at a time; and one
-// at a time when the wide tiles would not fill the chip (a warp or half a warp per piece and tile: kPullWideWarps) -- on
-// a graph of 1,000 nodes they left most of it idle and cost a launch (1.02 -> 1.04 ms a query).
-constexpr int32_t kPullWide = 128, kPullMid = 192;
-constexpr int64_t kPullWideWarps = 2 * 152 * 32;
-constexpr int64_t kPullWideRows = (128ll << 20) / 512;
+// (tile codes: pull_shape.h)
 void launch_pull(const DeviceGraph &g, const float *D, int32_t dpitch, int64_t dts, int32_t dsub, float *MD,
                  int32_t pitch, int64_t mts, int32_t msub, int32_t ntiles, int32_t tile, int32_t blocks_per_sm,
                  const uint32_t *zmask, cudaStream_t s);
-// the same over one tile of 1, 2, 4, 8 or 16 columns (pull_narrow.cu), for graphs of at most kNarrowPieces pieces: four
-// times the threads the chip holds at eight lanes a piece (beyond that both kernels are bound by the gathers: 78 us
-// against 82 for one column of R-MAT 2^20, where 22 against 5 on 30,000 nodes)
-constexpr int64_t kNarrowPieces = 4ll * 152 * 2048 / 8;
+// the same over one tile of 1, 2, 4, 8 or 16 columns (pull_narrow.cu)
 void launch_pull_narrow(const DeviceGraph &g, const float *D, int32_t dpitch, float *MD, int32_t pitch, int32_t tile,
                         int32_t blocks_per_sm, const uint32_t *zmask, cudaStream_t s);
 // The pull over ntiles full 32-column tiles with TMA row gathers (pull_tma.cu); D's tiles as for launch_pull, plus
 // dcols = the columns of one row of D's layout (its pitch, or a group's width).  *err is set when a stage's wait
 // gives up.  Not available (cudaErrorNotSupported) when the driver gives no tensor-map encoder.
 constexpr int32_t kTmaMaxGroups = 8;   // groups of D one launch addresses (one tensor map each)
-constexpr int32_t kPullTma = 96;       // the tuner's name for this launch shape
 bool pull_tma_available();
 cudaError_t launch_pull_tma(const DeviceGraph &g, const float *D, int32_t dpitch, int32_t dcols, int64_t dts,
                             int32_t dsub, float *MD, int32_t pitch, int64_t mts, int32_t msub, int32_t ntiles,

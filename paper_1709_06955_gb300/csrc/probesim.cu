@@ -358,6 +358,46 @@ struct PhaseTimer {
     }
 };
 
+// The pull of a depth's nfull full 32-column tiles, from column 0 of B and A, in the tuning's shape (pull_shape.h); the
+// level loop and the tuner launch it.  err: the TMA shape's error flag.
+static cudaError_t pull_full(const DeviceGraph &g, const PullTuning &t, const float *B, const ColLayout &Lb, float *A,
+                             const ColLayout &La, int32_t nfull, const uint32_t *zmask, int32_t *err, int64_t *launches,
+                             cudaStream_t st) {
+    if (nfull <= 0) return cudaSuccess;
+    if (t.shape == kPullTma) {
+        ++*launches;
+        return launch_pull_tma(g, B, Lb.rpitch(0), Lb.K > 0 ? kGroup : Lb.R, Lb.tile_stride(), Lb.tile_sub(32), A,
+                               La.rpitch(0), La.tile_stride(), La.tile_sub(32), nfull, t.bps[kPullTma], zmask, err, st);
+    }
+    const int32_t tw = t.shape == 16 ? 16 : 32;
+    FullTiles f{32, 1, 0, nfull};
+    if (t.shape == 32) f = full_tiles(nfull, g.n_pieces, g.n_active);
+    if (f.wide > 0) {
+        launch_pull(g, B, Lb.rpitch(0), Lb.tile_stride(), Lb.tile_sub(32 * f.per), A, La.rpitch(0), La.tile_stride(),
+                    La.tile_sub(32 * f.per), f.wide, f.tile, t.bps[f.tile], zmask, st);
+        ++*launches;
+    }
+    // all of the launch's tiles, or up to three that lie in one group after the wide ones
+    const int32_t c0 = 32 * f.per * f.wide, one = 1 << 30;
+    if (f.rest > 0) {
+        launch_pull(g, B + Lb.base(c0), Lb.rpitch(0), Lb.tile_stride(), f.wide > 0 ? one : Lb.tile_sub(tw),
+                    A + La.base(c0), La.rpitch(0), La.tile_stride(), f.wide > 0 ? one : La.tile_sub(tw),
+                    f.rest * (32 / tw), t.shape, t.bps[t.shape], zmask ? zmask + c0 / 32 : nullptr, st);
+        ++*launches;
+    }
+    return cudaSuccess;
+}
+
+// The pull of a tail tile of `tail` columns that starts at column c (it lies inside one group, or row, of each layout).
+static void pull_tail(const DeviceGraph &g, const PullTuning &t, const float *B, const ColLayout &Lb, float *A,
+                      const ColLayout &La, int32_t c, int32_t tail, const uint32_t *zmask, cudaStream_t st) {
+    if (narrow_tail(g.n_pieces))
+        launch_pull_narrow(g, B + Lb.base(c), Lb.rpitch(c), A + La.base(c), La.rpitch(c), tail, t.narrow[tail], zmask, st);
+    else
+        launch_pull(g, B + Lb.base(c), Lb.rpitch(c), 0, 1 << 30, A + La.base(c), La.rpitch(c), 0, 1 << 30, 1, tail,
+                    t.bps[tail], zmask, st);
+}
+
 // Runs the query path for one batch into d_out ([B][n] on the device).  Returns PROBESIM_E_NOMEM with
 // *too_big set when the level buffers of this batch would exceed the workspace budget.
 static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesim_query *q, int32_t B, float *d_out,
@@ -506,12 +546,9 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
     PS_CUDA(ws->md_b.ensure((size_t)max_floats * sizeof(float)));
     float *A = ws->md_a.as<float>(), *Bm = ws->md_b.as<float>();
     const int32_t *node_list = ws->node_list.as<int32_t>();
-    // the full tiles' launch: 32-column tiles, their 16-column halves, 32-column tiles two per pass, or 32-column
-    // tiles gathered by the TMA
-    const int32_t wide = g->tune_wide == 16 || g->tune_wide == kPullPairs || g->tune_wide == kPullTma ? g->tune_wide : 32;
-    const int32_t tw = wide == 16 ? 16 : 32;
+    const PullTuning tune = g->tune;
     int32_t *d_pull_err = nullptr;
-    if (wide == kPullTma) {
+    if (tune.shape == kPullTma) {
         PS_CUDA(ws->pull_err.ensure(sizeof(int32_t)));
         d_pull_err = ws->pull_err.as<int32_t>();
         PS_CUDA(cudaMemsetAsync(d_pull_err, 0, sizeof(int32_t), st));
@@ -576,47 +613,16 @@ static probesim_status run_batch(probesim_graph *g, Workspace *ws, const probesi
                 e1 = tm.get();
                 PS_CUDA(cudaEventRecord(e0, st));
             }
-            if (tail[d] > 0) {  // the tail tile lies inside one group (or row) of each layout
+            const uint32_t *zm = zmask_at(d);
+            if (tail[d] > 0) {
                 if (overlap) {
                     PS_CUDA(cudaEventRecord(ws->ev_ready, st));
                     PS_CUDA(cudaStreamWaitEvent(ss, ws->ev_ready, 0));
                 }
-                const int32_t c = 32 * nfull[d];
-                const uint32_t *zm = zmask_at(d) ? zmask_at(d) + nfull[d] : nullptr;
-                if (dgl.n_pieces <= kNarrowPieces)
-                    launch_pull_narrow(dgl, Bm + Lb.base(c), Lb.rpitch(c), A + La.base(c), La.rpitch(c), tail[d],
-                                       g->tune_bps[tail[d]], zm, ss);
-                else
-                    launch_pull(dgl, Bm + Lb.base(c), Lb.rpitch(c), 0, 1 << 30, A + La.base(c), La.rpitch(c), 0, 1 << 30,
-                                1, tail[d], g->tune_bps[tail[d]], zm, ss);
+                pull_tail(dgl, tune, Bm, Lb, A, La, 32 * nfull[d], tail[d], zm ? zm + nfull[d] : nullptr, ss);
                 ++launches;
             }
-            if (nfull[d] > 0 && wide == kPullTma) {  // 32-column tiles, rows gathered by the TMA
-                PS_CUDA(launch_pull_tma(dgl, Bm, Lb.rpitch(0), Lb.K > 0 ? kGroup : Lb.R, Lb.tile_stride(), Lb.tile_sub(32),
-                                        A, La.rpitch(0), La.tile_stride(), La.tile_sub(32), nfull[d],
-                                        g->tune_bps[kPullTma], zmask_at(d), d_pull_err, st));
-                ++launches;
-            } else if (nfull[d] > 0) {  // 32-column tiles (or their 16-column halves, or pairs of them)
-                // tiles of 128 or 64 columns first (see kPullWide), then what is left
-                const int32_t per = dg.n_active <= kPullWideRows ? 4 : 2;
-                int32_t nw = wide == 32 ? nfull[d] / per : 0;
-                if (dgl.n_pieces * nw * per / 4 < kPullWideWarps) nw = 0;
-                if (nw > 0) {
-                    launch_pull(dgl, Bm, Lb.rpitch(0), Lb.tile_stride(), Lb.tile_sub(32 * per), A, La.rpitch(0),
-                                La.tile_stride(), La.tile_sub(32 * per), nw, per == 4 ? kPullWide : kPullMid,
-                                g->tune_bps[32], zmask_at(d), st);
-                    ++launches;
-                }
-                // all of the launch's tiles, or up to three that lie in one group after the wide ones
-                const int32_t nt = (nfull[d] - per * nw) * (32 / tw), c0 = 32 * per * nw;
-                const int32_t one = 1 << 30;
-                if (nt > 0) {
-                    launch_pull(dgl, Bm + Lb.base(c0), Lb.rpitch(0), Lb.tile_stride(), nw > 0 ? one : Lb.tile_sub(tw),
-                                A + La.base(c0), La.rpitch(0), La.tile_stride(), nw > 0 ? one : La.tile_sub(tw), nt, wide,
-                                g->tune_bps[wide], zmask_at(d) ? zmask_at(d) + c0 / 32 : nullptr, st);
-                    ++launches;
-                }
-            }
+            PS_CUDA(pull_full(dgl, tune, Bm, Lb, A, La, nfull[d], zm, d_pull_err, &launches, st));
             if (ws->profiling) {
                 PS_CUDA(cudaEventRecord(e1, st));
                 marks.push_back({e0, e1});
@@ -1709,86 +1715,98 @@ probesim_status probesim_topk(probesim_graph *g, const probesim_query *q, int32_
     return topk_core(g, &g->ws0, g->current(), q, nq, kmax, ids, vals, (cudaStream_t)stream);
 }
 
-// Times the pull on this graph's in-lists for every tile width in {1, 2, 4, 8, 16, 32} and blocks-per-SM in
-// {2, 4, 8, 16} over a random score matrix, keeps the fastest shape per width, and picks the full tiles' launch
-// (16-column halves, 32-column tiles, or 32-column tiles two per pass) by time per column.  The choice is stored in the graph and used by every later query.
+// Times the pulls that the level loop launches below depth 0 (pull_full, pull_tail: the same kernels, chosen by the same
+// rules, over the same pieces) for {2, 4, 8, 16} blocks per SM, keeps the fastest number for each kernel, and picks the
+// full tiles' shape.  What is not faster than the default by more than kTunerGain stays at the default: a choice within
+// the timings' noise must not make a tuned graph slower than an untuned one.  The choice is stored in the graph and used by
+// every later query.  (Timing 32-column tiles alone over 64 columns, as this did, gave the wide tiles 2 blocks per SM: a
+// query of two on 50,000 nodes and 5 million edges 8.4 ms untuned, 9.2 tuned; R-MAT 2^18 at eps 0.05 31.2 and 32.4.)
 probesim_status probesim_autotune(probesim_graph *g, void *stream) {
     if (!g) return fail(PROBESIM_E_INVALID, "graph is null");
     std::lock_guard<std::mutex> lk(g->mu);
     const std::shared_ptr<StoreVersion> snap = g->current();
     g_last_error.clear();
     cudaStream_t st = (cudaStream_t)stream;
-    const DeviceGraph &dg = snap->dg;
-    const int32_t n = dg.n, P = 64;
+    DeviceGraph dg = snap->dg;
+    dg.n_pieces = dg.n_pieces_active;
+    if (dg.n_pieces == 0) return PROBESIM_OK;  // no edges: nothing is pulled below depth 0
+    const int32_t n = dg.n, nt = tuner_tiles(n, dg.n_pieces, dg.n_active, budget_of(g, &g->ws0) / 2);
+    const ColLayout L = make_layout(n, 32 * nt);
     Workspace *ws = &g->ws0;
-    PS_CUDA(ws->md_a.ensure((size_t)(n + 1) * P * sizeof(float)));  // a spare row after the n rows
-    PS_CUDA(ws->md_b.ensure((size_t)(n + 1) * P * sizeof(float)));
-    PS_CUDA(cudaMemsetAsync(ws->md_a.p, 0x3c, (size_t)(n + 1) * P * sizeof(float), st));  // any finite values
-    const int32_t tiles[] = {1, 2, 4, 8, 16}, bpss[] = {2, 4, 8, 16};
+    const size_t bytes = sizeof(float) * (size_t)L.size();
+    PS_CUDA(ws->md_a.ensure(bytes));
+    PS_CUDA(ws->md_b.ensure(bytes));
+    PS_CUDA(cudaMemsetAsync(ws->md_a.p, 0x3c, bytes, st));  // any finite values
+    PS_CUDA(cudaMemsetAsync(ws->md_b.p, 0, bytes, st));
+    PS_CUDA(ws->pull_err.ensure(sizeof(int32_t)));
+    PS_CUDA(cudaMemsetAsync(ws->pull_err.p, 0, sizeof(int32_t), st));
+    const float *D = ws->md_a.as<float>();
+    float *M = ws->md_b.as<float>();
     Timer tm{ws, st};
-    // times one configuration: three runs after a warm-up run, in ms
+    const cudaEvent_t e0 = tm.get(), e1 = tm.get();
+    PullTuning t = g->tune;
+    int64_t launches = 0;
+    cudaError_t le = cudaSuccess;
+    // the shortest of three runs after a warm-up run, in ms
     auto time_pull = [&](auto &&launch) -> float {
-        float total = 0.f;
+        float best = 1e30f;
         for (int rep = 0; rep < 4; ++rep) {
-            cudaEvent_t e0 = tm.get(), e1 = tm.get();
             cudaEventRecord(e0, st);
             launch();
             cudaEventRecord(e1, st);
-            cudaEventSynchronize(e1);
+            if (cudaEventSynchronize(e1) != cudaSuccess) return 1e30f;
             float ms = 0.f;
             cudaEventElapsedTime(&ms, e0, e1);
-            if (rep > 0) total += ms;
+            if (rep > 0) best = std::min(best, ms);
         }
-        return total;
+        return best;
     };
-    float *Da = ws->md_a.as<float>(), *Mb = ws->md_b.as<float>();
+    const float kTunerGain = 0.98f;
+    // blocks per SM of one kernel, into `slot`; returns its time
+    auto tune_blocks = [&](int32_t &slot, auto &&launch) -> float {
+        int32_t pick = slot = kPullBlocks;
+        float best = time_pull(launch);
+        for (int32_t bps : {2, 4, 16}) {
+            slot = bps;
+            const float ms = time_pull(launch);
+            if (ms < kTunerGain * best) best = ms, pick = bps;
+        }
+        slot = pick;
+        return best;
+    };
     // tail tiles: one narrow tile over a compact [n][T] block
-    for (int32_t T : tiles) {
-        float best = 1e30f;
-        for (int32_t bps : bpss) {
-            const float ms = time_pull([&] { launch_pull(dg, Da, T, 0, 1, Mb, T, 0, 1, 1, T, bps, nullptr, st); });
-            if (ms < best) best = ms, g->tune_bps[T] = bps;
-        }
+    for (int32_t T : {1, 2, 4, 8, 16}) {
+        const ColLayout LT = make_layout(n, T);
+        tune_blocks(narrow_tail(dg.n_pieces) ? t.narrow[T] : t.bps[T],
+                    [&] { pull_tail(dg, t, D, LT, M, LT, 0, T, nullptr, st); });
     }
-    // wide tiles: two 32-column tiles of a node-major [n][64] matrix, as 32-column tiles, 16-column halves, or one
-    // pass over both
-    double per_col[kPullTma + 1] = {0};
-    int32_t wide_bps[kPullTma + 1] = {0};
-    for (int32_t T : {16, 32, kPullPairs}) {
-        float best = 1e30f;
-        for (int32_t bps : bpss) {
-            const int32_t nt = T == 16 ? 4 : 2;
-            const float ms =
-                time_pull([&] { launch_pull(dg, Da, P, 0, 1 << 30, Mb, P, 0, 1 << 30, nt, T, bps, nullptr, st); });
-            if (ms < best) best = ms, wide_bps[T] = bps;
-        }
-        per_col[T] = best / 3.0 / 64.0;
+    // full tiles, each shape over the same nt tiles: with 32 the wide tiles, and the 32-column ones left over or alone
+    auto full = [&](int32_t tiles) {
+        const cudaError_t e =
+            pull_full(dg, t, D, L, M, L, tiles, nullptr, ws->pull_err.as<int32_t>(), &launches, st);
+        if (e != cudaSuccess) le = e;
+    };
+    t.shape = 32;
+    const FullTiles f = full_tiles(nt, dg.n_pieces, dg.n_active);
+    float best = tune_blocks(t.bps[32], [&] { full(f.wide > 0 ? f.per - 1 : nt); });
+    if (f.wide > 0) best = tune_blocks(t.bps[f.tile], [&] { full(nt); });
+    const PullTuning base = t;
+    PullTuning pick = t;
+    for (int32_t shape : {16, kPullPairs, kPullTma}) {
+        if (shape == kPullTma && !pull_tma_available()) continue;
+        t = base;
+        t.shape = shape;
+        t.bps[kPullTma] = 1;  // the TMA launch: one block of 192 KB shared memory per SM
+        const float ms = shape == kPullTma ? time_pull([&] { full(nt); }) : tune_blocks(t.bps[shape], [&] { full(nt); });
+        if (ms < kTunerGain * best) best = ms, pick = t;
     }
-    if (pull_tma_available()) {  // the TMA gathers (one block of 192 KB shared memory per SM)
-        PS_CUDA(ws->pull_err.ensure(sizeof(int32_t)));
-        PS_CUDA(cudaMemsetAsync(ws->pull_err.p, 0, sizeof(int32_t), st));
-        cudaError_t le = cudaSuccess;
-        const float best = time_pull([&] {
-            le = launch_pull_tma(dg, Da, P, P, 0, 1 << 30, Mb, P, 0, 1 << 30, 2, 1, nullptr, ws->pull_err.as<int32_t>(),
-                                 st);
-        });
-        PS_CUDA(le);
-        wide_bps[kPullTma] = 1;
-        int32_t herr = 0;
-        PS_CUDA(cudaMemcpyAsync(&herr, ws->pull_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        PS_CUDA(cudaStreamSynchronize(st));
-        if (herr) return fail(PROBESIM_E_TIMEOUT, "a TMA row gather of the pull did not complete in time");
-        per_col[kPullTma] = best / 3.0 / 64.0;
-    }
+    PS_CUDA(le);
     PS_CUDA(cudaGetLastError());
-    int32_t pick = 32;
-    for (int32_t T : {16, kPullPairs, kPullTma})
-        if (per_col[T] > 0 && per_col[T] < per_col[pick]) pick = T;
-    g->tune_bps[32] = wide_bps[32];
-    g->tune_bps[pick] = wide_bps[pick];
-    g->tune_wide = pick;
-    g->tuned = 1;
-    PS_CUDA(cudaGetLastError());
+    int32_t herr = 0;
+    PS_CUDA(cudaMemcpyAsync(&herr, ws->pull_err.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    PS_CUDA(cudaStreamSynchronize(st));
+    if (herr) return fail(PROBESIM_E_TIMEOUT, "a TMA row gather of the pull did not complete in time");
+    g->tune = pick;
     return PROBESIM_OK;
 }
 
@@ -1803,20 +1821,30 @@ probesim_status probesim_set_tuning(probesim_graph *g, int32_t wide_tile, const 
             if (blocks_per_sm[i] < 1 || blocks_per_sm[i] > 32)
                 return fail(PROBESIM_E_INVALID, "blocks_per_sm must lie in [1, 32]");
     std::lock_guard<std::mutex> lk(g->mu);
-    g->tune_wide = wide_tile;
+    g->tune.shape = wide_tile;
     if (blocks_per_sm) {
-        for (int i = 0; i < 6; ++i) g->tune_bps[1 << i] = blocks_per_sm[i];
-        g->tune_bps[kPullPairs] = blocks_per_sm[6];
-        g->tune_bps[kPullTma] = blocks_per_sm[7];
+        for (int i = 0; i < 6; ++i) g->tune.bps[1 << i] = blocks_per_sm[i];
+        for (int i = 0; i < 5; ++i) g->tune.narrow[1 << i] = blocks_per_sm[i];
+        g->tune.bps[kPullWide] = g->tune.bps[kPullMid] = blocks_per_sm[5];
+        g->tune.bps[kPullPairs] = blocks_per_sm[6];
+        g->tune.bps[kPullTma] = blocks_per_sm[7];
     }
     return PROBESIM_OK;
 }
 
 probesim_status probesim_get_tuning(const probesim_graph *g, int32_t *wide_tile, int32_t *blocks_per_sm) {
     if (!g) return fail(PROBESIM_E_INVALID, "graph is null");
-    if (wide_tile) *wide_tile = g->tune_wide;
-    if (blocks_per_sm)
-        for (int i = 0; i < 6; ++i) blocks_per_sm[i] = g->tune_bps[1 << i] ? g->tune_bps[1 << i] : 8;
+    const PullTuning &t = g->tune;
+    if (wide_tile) *wide_tile = t.shape;
+    if (blocks_per_sm) {  // of the kernels that pull below depth 0: the narrow tails, the wide tiles
+        const std::shared_ptr<StoreVersion> v = const_cast<probesim_graph *>(g)->current();
+        const bool narrow = narrow_tail(v->dg.n_pieces_active);
+        const int32_t wide = v->dg.n_active <= kPullWideRows ? kPullWide : kPullMid;
+        for (int i = 0; i < 6; ++i) {
+            const int32_t b = i == 5 ? t.bps[wide] : (narrow ? t.narrow[1 << i] : t.bps[1 << i]);
+            blocks_per_sm[i] = b ? b : kPullBlocks;
+        }
+    }
     return PROBESIM_OK;
 }
 

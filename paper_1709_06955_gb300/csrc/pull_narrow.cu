@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(256) k_pull_narrow(const int32_t *__restrict__
 
 void launch_pull_narrow(const DeviceGraph &g, const float *D, int32_t dpitch, float *MD, int32_t pitch, int32_t tile,
                         int32_t blocks_per_sm, const uint32_t *zmask, cudaStream_t s) {
-    const int blocks = grid_for(g.n_pieces * 8, 256, blocks_per_sm > 0 ? blocks_per_sm : 8);
+    const int blocks = grid_for(g.n_pieces * 8, 256, blocks_per_sm > 0 ? blocks_per_sm : kPullBlocks);
 #define PS_NARROW(T, U)                                                                                               \
     pdl_launch(k_pull_narrow<T, U>, dim3(blocks), dim3(256), 0, s, g.piece_v, g.piece_beg, g.piece_len, g.n_pieces,   \
                g.in_col, g.w, D, dpitch, MD, pitch, g.n, zmask)
