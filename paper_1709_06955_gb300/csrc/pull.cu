@@ -205,7 +205,7 @@ void launch_pull(const DeviceGraph &g, const float *D, int32_t dpitch, int64_t d
     const int NT = tile == kPullPairs ? 2 : 1;
     const int L = T >= 4 ? T / 4 : 1;
     const int64_t threads_needed = g.n_pieces * L;
-    const int blocks = grid_for(threads_needed, 256, blocks_per_sm > 0 ? blocks_per_sm : kPullBlocks);
+    const int blocks = grid_for(threads_needed, 256, blocks_per_sm > 0 ? blocks_per_sm : 8);
     dim3 grid(blocks, (ntiles + NT - 1) / NT);
 #define PS_PULL(T, NT)                                                                                              \
     k_pull<T, NT><<<grid, 256, 0, s>>>(g.piece_v, g.piece_beg, g.piece_len, g.n_pieces, g.in_col, g.w, D, dpitch, MD, \
