@@ -7,7 +7,6 @@
 #include <atomic>
 #include <memory>
 #include <mutex>
-#include <shared_mutex>
 #include <string>
 #include <vector>
 
@@ -42,7 +41,7 @@ struct Workspace {
     DevBuf counts, node_list, sched;  // level schedule: node counts and lists per depth, uploaded plan
     ps::LevelPlan plan;               // its host side
     DevBuf md_a, md_b, out_stage;     // the two score buffers; host-output staging
-    DevBuf r_part, r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
+    DevBuf r_ent[2], r_first[2], r_counts, r_counts2, r_ctr;
     DevBuf tk_hist, tk_state, tk_tie, tk_cid, tk_cval, tk_ids, tk_qk, tk_short;
     // frontier engine: walk-prefix slots, switched flags, probes, frontier lists, deferral stack, tasks, global tables,
     // estimates
@@ -73,7 +72,7 @@ struct Workspace {
     void release() {
         DevBuf *bufs[] = {&qbuf, &walks, &lens, &ctr, &t_key, &t_node, &t_parent, &t_depth, &t_query, &t_weight,
                           &t_height, &t_slot, &t_gamma, &t_G, &counts, &node_list,
-                          &sched, &md_a, &md_b, &out_stage, &r_part, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
+                          &sched, &md_a, &md_b, &out_stage, &r_ent[0], &r_ent[1], &r_first[0], &r_first[1],
                           &r_counts, &r_counts2, &r_ctr, &tk_hist, &tk_state, &tk_tie,
                           &tk_cid, &tk_cval, &tk_ids, &tk_qk, &tk_short, &f_wslot, &f_tsw, &f_slot, &f_misc, &f_pr32, &f_pr64, &f_acc,
                           &f_tab, &f_list[0], &f_list[1], &f_stack, &f_tasks, &f_keys, &pm_in, &pm_meets, &pull_err};

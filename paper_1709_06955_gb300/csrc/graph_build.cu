@@ -7,11 +7,11 @@
 //   2. an LSD radix sort of the keys (below)
 //   3. repeats and loops dropped: a flag per key, its prefix sums, a compaction
 //   4. the caller-id in-list offsets (run boundaries of the sorted keys) and out-degrees; the renumbering by
-//      descending out-degree, ties by caller id, as a radix sort of n keys ((m - outdeg) << bs | id), by the upper half alone: the
-//      keys start in id order and the sort is stable
+//      descending out-degree, ties by caller id, as a radix sort of n keys ((m - outdeg) << bs | id), by the upper
+//      half alone: the keys start in id order and the sort is stable
 //   5. the in-lists per internal row in the caller's source order (each row's run of sorted keys mapped through
-//      ext2int), and the out-lists from a radix sort of (source << bs | destination) in internal ids, by the source alone: the
-//      keys start in destination order
+//      ext2int), and the out-lists from a radix sort of (source << bs | destination) in internal ids, by the source
+//      alone: the keys start in destination order
 // w and the pull pieces then come from the kernels the update path uses.
 //
 // Radix sort: 8-bit digits, least significant first, tiles of 4096 keys.  Per digit pass, one kernel counts
@@ -36,7 +36,8 @@ static_assert(kRadixThreads == kRadix, "the digit scans use one thread per digit
 int64_t radix_tiles(int64_t count) { return (count + kRadixTile - 1) / kRadixTile; }
 
 // Each warp counts into its own table; its lanes that share the first lane's digit add once, which takes the load off
-// the one counter of a skewed digit.  (11 million keys: 55 to 78 us a pass with a match over the warp's 32 digits, 15 to 25 now.)
+// the one counter of a skewed digit.  (11 million keys: 55 to 78 us a pass with a match over the warp's 32 digits, 15 to
+// 25 now.)
 __global__ void __launch_bounds__(kRadixThreads) k_radix_hist(const uint64_t *__restrict__ keys, int64_t count,
                                                               int shift, long long *__restrict__ counts,
                                                               int64_t ntiles) {

@@ -1,9 +1,10 @@
 // Device-side update of the graph store: one batch of edge insertions or deletions merged into the CSR
 // arrays without rebuilding them on the host.
 //
-// The host sorts the (deduplicated, loop-free) batch twice: by (destination, source in the caller's id order)
-// for the in-lists, whose order is the caller's source-id order (walks pick the k-th entry of it), and by
-// (source, destination in internal id order) for the out-lists.  The device then
+// The batch comes deduplicated, without loops and in two orders, sorted on the device (graph_build.cu's radix sort): by
+// (destination, source in the caller's id order) for the in-lists, whose order is the caller's source-id order (walks
+// pick the k-th entry of it), and by (source, destination in internal id order) for the out-lists.  Then the kernels
+// below
 //   1. marks the batch entries that change the graph (an insert of an absent edge, a delete of a present one)
 //      by binary search in the current rows, and counts the change of every row's degree;
 //   2. forms the new offsets (prefix sums of the new degrees);

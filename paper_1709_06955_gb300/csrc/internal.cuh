@@ -400,8 +400,8 @@ void launch_inst_init(const QueryBatch &q, const DeviceGraph &g, const int32_t *
                       unsigned long long *check, const int32_t *walk_slot, const uint8_t *t_sw, cudaStream_t s);
 void launch_add_i32(int32_t *a, const int32_t *b, int64_t count, cudaStream_t s);  // a += b
 // E: about the level's work items (sizes the grid)
-void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const uint32_t *qkey, uint32_t seed, uint32_t t_keep, const RandLevel &L, int64_t E,
-                       cudaStream_t s);
+void launch_rand_level(const DeviceGraph &g, const int32_t *walks, int32_t l_max, const uint32_t *qkey, uint32_t seed,
+                       uint32_t t_keep, const RandLevel &L, int64_t E, cudaStream_t s);
 void launch_rand_finalize(int32_t n, int32_t B, const int32_t *qnode, const int32_t *counts, const float *inv_nr,
                           const int32_t *ext2int, float shift, float *out, cudaStream_t s);
 

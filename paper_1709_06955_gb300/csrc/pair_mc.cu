@@ -3,8 +3,9 @@
 // with r >= ln(1/delta) / (2 eps^2) it is within eps of s(u, v) with probability 1 - delta (Chernoff).  It serves
 // as the single-pair "expert" that gauges pooled top-k candidates on graphs too large for the Power Method.
 //
-// The two walks of a walk pair t advance in lockstep, their i-th nodes compared at every position both reach.  Walk t from u draws Philox counter (t, s, 0, 0) under key (seed, key_u) at step s -- the draws
-// of query key_u's walk t in the single-source path -- and likewise from v under (seed, key_v).
+// The two walks of a walk pair t advance in lockstep, their i-th nodes compared at every position both reach.  Walk t
+// from u draws Philox counter (t, s, 0, 0) under key (seed, key_u) at step s -- the draws of query key_u's walk t in the
+// single-source path -- and likewise from v under (seed, key_v).
 #include <algorithm>
 
 #include "internal.cuh"

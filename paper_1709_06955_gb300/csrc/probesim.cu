@@ -7,7 +7,6 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
-#include <shared_mutex>
 #include <new>
 #include <string>
 #include <vector>

@@ -63,8 +63,8 @@ struct probesim_server {
 
 // Device bytes a query takes in a batch.  The regrouped deterministic engine holds about 0.25 n_r score vectors
 // of n FP32 in three buffers at its widest depth.  The frontier and randomized engines hold an estimate row
-// (8 + 4 bytes per node) and walk rows of the query's n_r walks (8 bytes per node slot); their level tables and
-// hash sets adapt to the worker's share of the budget (passes, deferred ranges, walk ranges).
+// (8 + 4 bytes per node) and walk rows of the query's n_r walks (8 bytes per node slot); their level lists, tables and
+// tasks adapt to the worker's share of the budget (deferred probe ranges, walk ranges).
 static double query_bytes(const probesim_server *s, const probesim_query &q) {
     const double nr = (double)ps::num_walks_for(s->g, q.eps), n = (double)s->g->n;
     const probesim_config &c = s->g->cfg;
